@@ -46,9 +46,13 @@ __host__ __device__ inline uint32_t pc_ref_type(uint32_t r) { return r >> 30; }
 __host__ __device__ inline uint32_t pc_ref_local(uint32_t r) { return (r >> 28) & 3u; }
 __host__ __device__ inline uint32_t pc_ref_id(uint32_t r) { return r & 0x0FFFFFFFu; }
 
+// contribution code of a block's value list: hinge(1) | row's local vertex(2) | column's(2) | id(27)
+#define PC_CODE_HINGE 0x80000000u
+#define PC_CODE_ID 0x07FFFFFFu
+
 // per-element buffer strides (floats)
-#define PC_TRI_STRIDE 64     // 9 forces + 6 upper 3x3 Hessian blocks (54) + 1 pad
-#define PC_HINGE_STRIDE 24   // 12 forces + 12 scaled angle gradient
+#define PC_TRI_STRIDE 32     // right-hand-side shares (9) + Hessian factors (22) + 1 pad
+#define PC_HINGE_STRIDE 16   // 4 x (scaled angle gradient, right-hand-side factor)
 #define PC_CONTACT_STRIDE 20 // 12 forces + normal(3) + weights(3) + scale(1) + pad
 
 // PCG scalar block, lives in device memory
@@ -104,6 +108,9 @@ struct pc_ctx {
     int32_t *scol = nullptr;       // [snnz]
     int32_t *vinc_ptr = nullptr;   // [V+1]
     uint32_t *vinc = nullptr;      // [3T + 4H] element refs grouped by vertex
+    int32_t *val_ptr = nullptr;    // [snnz + 1] value list of each static block
+    uint32_t *val_codes = nullptr; // contribution codes (row vertex != column vertex), in incidence order
+    uint8_t *pin_adj = nullptr;    // [V] some column of the row's static pattern (not its own) is pinned
     int64_t enn = 0;
     int32_t *erp = nullptr;        // [V+1] edge one-rings (CSR)
     int32_t *ecol = nullptr;       // [enn] edge neighbours, sorted per vertex

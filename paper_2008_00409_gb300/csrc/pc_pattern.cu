@@ -268,6 +268,47 @@ __global__ void rowptr_from_keys_kernel(int V, const uint64_t *ukeys, int64_t n,
     rp[r] = (int32_t)pc_lower_bound_u64(ukeys, n, (uint64_t)r * (uint64_t)V);
 }
 
+// Value lists: for every static block (row i, column j) the elements that contribute to it
+// with i and j at different local vertices, in the row's incidence order, so that value
+// assembly sums a block without searching (48 codes of 4 bytes per row on a cloth). One
+// thread per row owns all the row's blocks: a counting pass (codes == null), a scan of the
+// counts, a filling pass (cur: each block's next free place).
+__global__ void value_lists_kernel(int V, const int32_t *__restrict__ srp, const int32_t *__restrict__ scol,
+                                   const int32_t *__restrict__ vinc_ptr, const uint32_t *__restrict__ vinc,
+                                   const int32_t *__restrict__ tri, const int32_t *__restrict__ hinge, int32_t *cur,
+                                   uint32_t *codes)
+{
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= V) return;
+    const int s0 = srp[r], s1 = srp[r + 1];
+    for (int i = vinc_ptr[r]; i < vinc_ptr[r + 1]; ++i) {
+        const uint32_t ref = vinc[i], k = pc_ref_local(ref), id = pc_ref_id(ref);
+        const bool hg = pc_ref_type(ref) == PC_REF_HINGE;
+        const int n = hg ? 4 : 3;
+        const int32_t *v = hg ? hinge + 4ll * id : tri + 3ll * id;
+        for (int l = 0; l < n; ++l) {
+            if (l == (int)k) continue;
+            int lo = s0, hi = s1;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (scol[mid] < v[l]) lo = mid + 1; else hi = mid;
+            }
+            if (codes) codes[cur[lo]] = (hg ? PC_CODE_HINGE : 0u) | (k << 29) | ((uint32_t)l << 27) | id;
+            cur[lo] += 1;
+        }
+    }
+}
+
+__global__ void pin_adj_kernel(int V, const int32_t *__restrict__ srp, const int32_t *__restrict__ scol,
+                               const uint8_t *__restrict__ pinned, uint8_t *adj)
+{
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= V) return;
+    uint8_t any = 0;
+    for (int i = srp[r]; i < srp[r + 1]; ++i) any |= scol[i] != r && pinned[scol[i]] ? 1 : 0;
+    adj[r] = any;
+}
+
 // Mean rest length of each vertex's mesh edges (0 for an isolated vertex), in FP64.
 __global__ void rest_len_kernel(int V, const int32_t *__restrict__ erp, const int32_t *__restrict__ ecol,
                                 const float *__restrict__ rest, float *out)
@@ -296,7 +337,8 @@ static void free_ctx(pc_ctx *c)
     pc_batched_free(c);
     pc_mlp_ctx_free(c);
     void *ptrs[] = {c->tri, c->rest, c->tri_dmi, c->tri_area, c->tri_rgram, c->mass, c->pinned, c->hinge, c->hcoef,
-                    c->hrest, c->srp, c->scol, c->erp, c->ecol, c->rest_len, c->vinc_ptr, c->vinc, c->dkeys, c->dnew, c->dflag, c->dscan, c->ckeys,
+                    c->hrest, c->srp, c->scol, c->erp, c->ecol, c->rest_len, c->val_ptr,
+                    c->val_codes, c->pin_adj, c->vinc_ptr, c->vinc, c->dkeys, c->dnew, c->dflag, c->dscan, c->ckeys,
                     c->cinc, c->cinc_ptr, c->tri_buf, c->hinge_buf, c->cont_buf, c->r, c->z, c->p0, c->p1, c->q,
                     c->dinv, c->dtmp, c->rhs32, c->x64, c->r64, c->partials, c->sc, c->A_rp, c->A_ci, c->A_vals, c->A_dres,
                     c->A_b, c->A_dv, c->h_state, c->h_pairs, c->h_w, c->sort.keys_alt, c->sort.vals_alt, c->sort.hist,
@@ -443,6 +485,19 @@ static pc_status create_impl(pc_ctx *c, const int32_t *tris, const float *rest, 
         c->launches++;
         rowptr_from_keys_kernel<<<pc_blocks(V + 1ll, 256), 256, 0, st>>>(V, ukeys, c->snnz, c->srp);
         c->launches++;
+        // value lists of the static blocks (at most 6 codes per triangle and 12 per hinge)
+        if ((s = dalloc(&c->val_ptr, c->snnz + 1)) != PC_OK) break;
+        if ((s = dalloc(&c->val_codes, 6ll * T + 12ll * H)) != PC_OK) break;
+        if ((s = dalloc(&c->pin_adj, V)) != PC_OK) break;
+        PC_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int32_t) * (size_t)c->snnz, st));
+        value_lists_kernel<<<pc_blocks(V, 128), 128, 0, st>>>(V, c->srp, c->scol, c->vinc_ptr, c->vinc, c->tri,
+                                                              c->hinge, flag, nullptr);
+        if ((s = pc_exclusive_scan(c, flag, c->val_ptr, c->snnz, st)) != PC_OK) break;
+        PC_CUDA_TRY(cudaMemcpyAsync(flag, c->val_ptr, sizeof(int32_t) * (size_t)c->snnz, cudaMemcpyDeviceToDevice, st));
+        value_lists_kernel<<<pc_blocks(V, 128), 128, 0, st>>>(V, c->srp, c->scol, c->vinc_ptr, c->vinc, c->tri,
+                                                              c->hinge, flag, c->val_codes);
+        pin_adj_kernel<<<pc_blocks(V, 256), 256, 0, st>>>(V, c->srp, c->scol, c->pinned, c->pin_adj);
+        c->launches += 3;
         // edge one-rings (mesh edge neighbours of each vertex, sorted): the neighbourhood
         // of the learned warm start's features
         const int64_t nek = 6ll * T;

@@ -105,130 +105,192 @@ __device__ __forceinline__ void strain_from_edges(const dfl *e1, const dfl *e2, 
     G11 = 0.5f * (d1 * m01 + d3 * m11);
 }
 
-// One thread per triangle, everything at x_t. Record: right-hand-side contributions
-// c_k = h f_k - sum_l (h^2 H_kl) v_l for k = 0, 1, 2 (the element's share of
-// b = h (f - h K v), the first-order form of h f(x_t + h v_t), Eq. 2-3), then the h^2
-// Hessian blocks (0,0) (0,1) (0,2) (1,1) (1,2) (2,2), each 3x3 row-major. Since each
-// Hessian row sums to zero, sum_l H_kl v_l is formed as sum_l H_kl (v_l - v_k).
-__global__ void __launch_bounds__(128) tri_eval_kernel(int T, const int32_t *__restrict__ tri,
+// One thread per triangle, everything at x_t. With F the deformation gradient, g_k the
+// shape gradients, Fg_k = F g_k, S+ the clamped stress and c = h^2 A0 (h (h + beta) A0 with
+// damping), the Hessian block (k, l) is
+//   c (mu Fg_l Fg_k^T + lam Fg_k Fg_l^T + mu (g_k.g_l) F F^T + (g_k.S+ g_l) I),
+// so the record holds those factors (32 floats: one 128-byte line) instead of the six
+// upper blocks (54 floats), and the rows expand the block they need (tri_block below).
+// Record, as eight float4: (c_0, c mu) (c_1, s11) (c_2, s12) (Fg_1, s22) (Fg_2, gg00)
+// (M00 M01 M02 gg01) (M11 M12 M22 gg02) (gg11 gg12 gg22 -), M = c mu F F^T, s = c g.S+ g.
+// c_k = h f_k - sum_l (h^2 H_kl) v_l is the element's share of b = h (f - h K v), the
+// first-order form of h f(x_t + h v_t) (Eq. 2-3); since each Hessian row sums to zero,
+// sum_l H_kl v_l is formed as sum_l H_kl (v_l - v_k).
+// Bound by DRAM (reads 56 B of rest data per triangle, writes 128 B): the records are
+// staged in shared memory so that every store is a full line. 1.65M triangles: 523 us with
+// 256-byte records stored a float at a time.
+#define TE_THREADS 128
+
+struct TriFactors {
+    float Fg[3][3];  // F g_k
+    float M[6];      // c mu F F^T, upper: 00 01 02 11 12 22
+    float gg[6];     // g_k . g_l, upper: 00 01 02 11 12 22
+    float s[6];      // c g_k . S+ g_l, same order
+    float cm, cl;    // c mu, c lam
+};
+
+// Entry (a, b) of the Hessian block (k, l), k <= l.
+__device__ __forceinline__ float tri_entry(const TriFactors &R, int k, int l, int a, int b)
+{
+    const int m = a == 0 || b == 0 ? a + b : a + b + 1;
+    float v = R.gg[tri_blk(k, l)] * R.M[m];
+    v = fmaf(R.cm * R.Fg[l][a], R.Fg[k][b], v);
+    v = fmaf(R.cl * R.Fg[k][a], R.Fg[l][b], v);
+    return a == b ? v + R.s[tri_blk(k, l)] : v;
+}
+
+__global__ void __launch_bounds__(TE_THREADS) tri_eval_kernel(int T, const int32_t *__restrict__ tri,
                                                        const float *__restrict__ x, const float *__restrict__ v,
                                                        const float *__restrict__ dmi_all,
                                                        const float *__restrict__ area, const float *__restrict__ rgram,
                                                        float mu, float lam, float h, float hk,
                                                        float *__restrict__ out)
 {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    int i0 = tri[3 * t], i1 = tri[3 * t + 1], i2 = tri[3 * t + 2];
-    float dmi[4] = {dmi_all[4 * t], dmi_all[4 * t + 1], dmi_all[4 * t + 2], dmi_all[4 * t + 3]};
-    float rg[6];
+    __shared__ float s_rec[TE_THREADS][PC_TRI_STRIDE + 1];
+    const int t = blockIdx.x * TE_THREADS + threadIdx.x;
+    if (t < T) {
+        int i0 = tri[3 * t], i1 = tri[3 * t + 1], i2 = tri[3 * t + 2];
+        const float4 dm = reinterpret_cast<const float4 *>(dmi_all)[t];
+        const float dmi[4] = {dm.x, dm.y, dm.z, dm.w};
+        float rg[6];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) rg[k] = rgram[6 * t + k];
-    const float A0 = area[t];
-    float x0[3], x1[3], x2[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        x0[a] = x[3 * i0 + a]; x1[a] = x[3 * i1 + a]; x2[a] = x[3 * i2 + a];
-    }
-    dfl e1[3], e2[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        e1[a] = two_sum(x1[a], -x0[a]);
-        e2[a] = two_sum(x2[a], -x0[a]);
-    }
-    // shape-function gradients: g1 = row 0 of Dm^-1, g2 = row 1, g0 = -g1 - g2
-    float g[3][2] = {{-dmi[0] - dmi[2], -dmi[1] - dmi[3]}, {dmi[0], dmi[1]}, {dmi[2], dmi[3]}};
-    float G00, G01, G11;
-    strain_from_edges(e1, e2, rg, dmi, G00, G01, G11);
-    const float tr = G00 + G11;
-    const float S00 = 2.0f * mu * G00 + lam * tr, S01 = 2.0f * mu * G01, S11 = 2.0f * mu * G11 + lam * tr;
-    float F[3][2];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        F[a][0] = e1[a].hi * dmi[0] + e2[a].hi * dmi[2];
-        F[a][1] = e1[a].hi * dmi[1] + e2[a].hi * dmi[3];
-    }
-    float f[3][3];  // forces at x_t
-    {
-        float P[3][2];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            P[a][0] = F[a][0] * S00 + F[a][1] * S01;
-            P[a][1] = F[a][0] * S01 + F[a][1] * S11;
+        for (int k = 0; k < 3; ++k) {
+            const float2 r2 = reinterpret_cast<const float2 *>(rgram)[3ll * t + k];
+            rg[2 * k] = r2.x;
+            rg[2 * k + 1] = r2.y;
         }
+        const float A0 = area[t];
+        float x0[3], x1[3], x2[3], v0[3], d1[3], d2[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            f[1][a] = -A0 * (P[a][0] * g[1][0] + P[a][1] * g[1][1]);
-            f[2][a] = -A0 * (P[a][0] * g[2][0] + P[a][1] * g[2][1]);
+            x0[a] = x[3 * i0 + a]; x1[a] = x[3 * i1 + a]; x2[a] = x[3 * i2 + a];
+            v0[a] = v[3 * i0 + a];
+            d1[a] = v[3 * i1 + a] - v0[a];
+            d2[a] = v[3 * i2 + a] - v0[a];
+        }
+        dfl e1[3], e2[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            e1[a] = two_sum(x1[a], -x0[a]);
+            e2[a] = two_sum(x2[a], -x0[a]);
+        }
+        // shape-function gradients: g1 = row 0 of Dm^-1, g2 = row 1, g0 = -g1 - g2
+        float g[3][2] = {{-dmi[0] - dmi[2], -dmi[1] - dmi[3]}, {dmi[0], dmi[1]}, {dmi[2], dmi[3]}};
+        float G00, G01, G11;
+        strain_from_edges(e1, e2, rg, dmi, G00, G01, G11);
+        const float tr = G00 + G11;
+        const float S00 = 2.0f * mu * G00 + lam * tr, S01 = 2.0f * mu * G01, S11 = 2.0f * mu * G11 + lam * tr;
+        float F[3][2];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            F[a][0] = e1[a].hi * dmi[0] + e2[a].hi * dmi[2];
+            F[a][1] = e1[a].hi * dmi[1] + e2[a].hi * dmi[3];
+        }
+        float f[3][3];  // forces at x_t
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float P0 = F[a][0] * S00 + F[a][1] * S01, P1 = F[a][0] * S01 + F[a][1] * S11;
+            f[1][a] = -A0 * (P0 * g[1][0] + P1 * g[1][1]);
+            f[2][a] = -A0 * (P0 * g[2][0] + P1 * g[2][1]);
             f[0][a] = -(f[1][a] + f[2][a]);
         }
-    }
-    // ---- Hessian at x_t (stress clamped to its positive part in the geometric term)
-    {
+        // Hessian factors at x_t (stress clamped to its positive part in the geometric term)
         float Sp00, Sp01, Sp11;
         sym2_positive(S00, S01, S11, Sp00, Sp01, Sp11);
-        float Fg[3][3], FFt[3][3];
+        TriFactors R;
+        const float c = hk * A0;
+        R.cm = c * mu;
+        R.cl = c * lam;
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) Fg[k][a] = F[a][0] * g[k][0] + F[a][1] * g[k][1];
+            for (int a = 0; a < 3; ++a) R.Fg[k][a] = F[a][0] * g[k][0] + F[a][1] * g[k][1];
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int b = a; b < 3; ++b) FFt[a][b] = F[a][0] * F[b][0] + F[a][1] * F[b][1];
-        const float c = hk * A0;
-        float *o = out + (int64_t)PC_TRI_STRIDE * t + 9;
+            for (int b = a; b < 3; ++b)
+                R.M[a == 0 ? b : a + b + 1] = R.cm * (F[a][0] * F[b][0] + F[a][1] * F[b][1]);
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
             for (int l = k; l < 3; ++l) {
-                float gg = g[k][0] * g[l][0] + g[k][1] * g[l][1];
-                float gSg = g[k][0] * (Sp00 * g[l][0] + Sp01 * g[l][1]) + g[k][1] * (Sp01 * g[l][0] + Sp11 * g[l][1]);
-                float *B = o + 9 * tri_blk(k, l);
+                R.gg[tri_blk(k, l)] = g[k][0] * g[l][0] + g[k][1] * g[l][1];
+                R.s[tri_blk(k, l)] = c * (g[k][0] * (Sp00 * g[l][0] + Sp01 * g[l][1]) +
+                                          g[k][1] * (Sp01 * g[l][0] + Sp11 * g[l][1]));
+            }
+        // right-hand-side shares c_k = h f_k - sum_{l != k} Hs_kl (v_l - v_k)
+        float ck[3][3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) ck[k][a] = h * f[k][a];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int l = k + 1; l < 3; ++l) {
+                float d[3];  // v_l - v_k
+#pragma unroll
+                for (int a = 0; a < 3; ++a) d[a] = (l == 1 ? d1[a] : d2[a]) - (k == 1 ? d1[a] : 0.f);
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
 #pragma unroll
                     for (int b = 0; b < 3; ++b) {
-                        if (k == l && b < a) continue;
-                        float ffab = a <= b ? FFt[a][b] : FFt[b][a];
-                        float val = mu * Fg[l][a] * Fg[k][b] + mu * gg * ffab + lam * Fg[k][a] * Fg[l][b];
-                        if (a == b) val += gSg;
-                        B[3 * a + b] = c * val;
-                        if (k == l && a != b) B[3 * b + a] = c * val;
+                        const float e = tri_entry(R, k, l, a, b);
+                        ck[k][a] = fmaf(-e, d[b], ck[k][a]);
+                        ck[l][b] = fmaf(e, d[a], ck[l][b]);
                     }
             }
-    }
-    // ---- right-hand-side contributions c_k = h f_k - sum_{l != k} Hs_kl (v_l - v_k)
-    {
-        const float *Bs = out + (int64_t)PC_TRI_STRIDE * t + 9;
-        const int vid[3] = {i0, i1, i2};
-        float vv[3][3];
+        float *o = s_rec[threadIdx.x];
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) vv[k][a] = v[3 * vid[k] + a];
-        float *o = out + (int64_t)PC_TRI_STRIDE * t;
+            for (int a = 0; a < 3; ++a) o[4 * k + a] = ck[k][a];
+        o[3] = R.cm;
+        o[7] = R.s[3];
+        o[11] = R.s[4];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            float ck[3] = {h * f[k][0], h * f[k][1], h * f[k][2]};
-#pragma unroll
-            for (int l = 0; l < 3; ++l) {
-                if (l == k) continue;
-                float dv0 = vv[l][0] - vv[k][0], dv1 = vv[l][1] - vv[k][1], dv2 = vv[l][2] - vv[k][2];
-                const float *B = Bs + 9 * tri_blk(k < l ? k : l, k < l ? l : k);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    // row a of block (k, l): B[a][*] if k < l, else column a of block (l, k)
-                    float b0 = k < l ? B[3 * a] : B[a], b1 = k < l ? B[3 * a + 1] : B[3 + a],
-                          b2 = k < l ? B[3 * a + 2] : B[6 + a];
-                    ck[a] -= b0 * dv0 + b1 * dv1 + b2 * dv2;
-                }
-            }
-#pragma unroll
-            for (int a = 0; a < 3; ++a) o[3 * k + a] = ck[a];
+        for (int a = 0; a < 3; ++a) {
+            o[12 + a] = R.Fg[1][a];
+            o[16 + a] = R.Fg[2][a];
+            o[20 + a] = R.M[a];
+            o[24 + a] = R.M[3 + a];
+            o[28 + a] = R.gg[3 + a];
         }
-        o[63] = 0.0f;
+        o[15] = R.s[5];
+        o[19] = R.gg[0];
+        o[23] = R.gg[1];
+        o[27] = R.gg[2];
+        o[31] = 0.f;
     }
+    __syncthreads();
+    const int n = min(TE_THREADS, T - (int)blockIdx.x * TE_THREADS) * PC_TRI_STRIDE;
+    float *o = out + (int64_t)blockIdx.x * TE_THREADS * PC_TRI_STRIDE;
+    for (int i = threadIdx.x; i < n; i += TE_THREADS) o[i] = s_rec[i / PC_TRI_STRIDE][i % PC_TRI_STRIDE];
+}
+
+// The factors of triangle record `id` (cl_cm = lam / mu).
+__device__ __forceinline__ TriFactors tri_load(const float *__restrict__ buf, uint32_t id, float cl_cm)
+{
+    const float4 *r = reinterpret_cast<const float4 *>(buf) + (int64_t)(PC_TRI_STRIDE / 4) * id;
+    const float cm = reinterpret_cast<const float *>(r)[3], s11 = reinterpret_cast<const float *>(r)[7],
+                s12 = reinterpret_cast<const float *>(r)[11];
+    const float4 f1 = r[3], f2 = r[4], m0 = r[5], m1 = r[6], q = r[7];
+    TriFactors R;
+    R.cm = cm;
+    R.cl = cl_cm * cm;
+    R.Fg[1][0] = f1.x; R.Fg[1][1] = f1.y; R.Fg[1][2] = f1.z;
+    R.Fg[2][0] = f2.x; R.Fg[2][1] = f2.y; R.Fg[2][2] = f2.z;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) R.Fg[0][a] = -(R.Fg[1][a] + R.Fg[2][a]);
+    R.M[0] = m0.x; R.M[1] = m0.y; R.M[2] = m0.z;
+    R.M[3] = m1.x; R.M[4] = m1.y; R.M[5] = m1.z;
+    R.gg[0] = f2.w; R.gg[1] = m0.w; R.gg[2] = m1.w;
+    R.gg[3] = q.x; R.gg[4] = q.y; R.gg[5] = q.z;
+    R.s[3] = s11; R.s[4] = s12; R.s[5] = f1.w;
+    R.s[1] = -(s11 + s12);
+    R.s[2] = -(s12 + f1.w);
+    R.s[0] = -(R.s[1] + R.s[2]);
+    return R;
 }
 
 // ------------------------------------------------------------------------- bending hinges
@@ -260,11 +322,13 @@ __device__ __forceinline__ float hinge_angle_grad(float3 a1, float3 a2, float3 a
     return theta;
 }
 
-// One thread per hinge, at x_t. Record: right-hand-side contributions on (wing0, wing1,
-// edge0, edge1), c_k = h f_k - q_k (q . v), then the scaled angle gradient
-// q = h sqrt(2 kb c_h) grad(theta), so the Gauss-Newton Hessian block (k, l) is q_k q_l^T.
-// The gradient sums to zero over the four vertices, so q . v uses velocities relative
-// to edge0.
+// One thread per hinge, at x_t. With q_k = h sqrt(2 kb c_h) grad_k(theta) (h^2 -> h (h + beta)
+// with damping) the Gauss-Newton Hessian block (k, l) is q_k q_l^T, and the right-hand-side
+// contribution h f_k - q_k (q . v) is q_k times one scalar w, because f_k is parallel to
+// grad_k too: h f_k = -h (2 kb c_h) (theta - theta_rest) grad_k. Record: four float4 (q_k, w),
+// 64 bytes, instead of 12 contributions and 12 gradients. The gradient sums to zero over
+// the four vertices, so q . v uses velocities relative to edge0. Bound by DRAM (reads 24 B
+// of rest data and writes 64 B per hinge); 2.48M hinges: 247 us with 96-byte records.
 __global__ void __launch_bounds__(128) hinge_eval_kernel(int H, const int32_t *__restrict__ hinge,
                                                          const float *__restrict__ x, const float *__restrict__ v,
                                                          const float *__restrict__ hcoef,
@@ -273,31 +337,26 @@ __global__ void __launch_bounds__(128) hinge_eval_kernel(int H, const int32_t *_
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= H) return;
-    int vid[4] = {hinge[4 * i], hinge[4 * i + 1], hinge[4 * i + 2], hinge[4 * i + 3]};
+    const int4 hv = reinterpret_cast<const int4 *>(hinge)[i];
+    const int vid[4] = {hv.x, hv.y, hv.z, hv.w};
     float3 X[4], W[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) { X[k] = ld3(x, vid[k]); W[k] = ld3(v, vid[k]); }
     const float kc = hcoef[i];
-    float *o = out + (int64_t)PC_HINGE_STRIDE * i;
     float3 grad[4];
     // positions relative to edge0
     float3 a1 = sub(X[0], X[2]), a2 = sub(X[1], X[2]), a4 = sub(X[3], X[2]);
     float th = hinge_angle_grad(a1, a2, a4, grad);
-    float s = -kc * (th - hrest[i]);  // f_k = s grad_k
     float sc = sqrtf(hk * kc);
     float3 q[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) q[k] = mul(sc, grad[k]);
     float qv = dot(q[0], sub(W[0], W[2])) + dot(q[1], sub(W[1], W[2])) + dot(q[3], sub(W[3], W[2]));
+    // h f_k = -h kc (theta - rest) grad_k = -(h / hk) sc (theta - rest) q_k
+    const float w = -(h / hk) * sc * (th - hrest[i]) - qv;
+    float4 *o = reinterpret_cast<float4 *>(out) + (int64_t)(PC_HINGE_STRIDE / 4) * i;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        o[3 * k] = h * s * grad[k].x - q[k].x * qv;
-        o[3 * k + 1] = h * s * grad[k].y - q[k].y * qv;
-        o[3 * k + 2] = h * s * grad[k].z - q[k].z * qv;
-        o[12 + 3 * k] = q[k].x;
-        o[12 + 3 * k + 1] = q[k].y;
-        o[12 + 3 * k + 2] = q[k].z;
-    }
+    for (int k = 0; k < 4; ++k) o[k] = make_float4(q[k].x, q[k].y, q[k].z, w);
 }
 
 // ------------------------------------------------------------------------- contacts
@@ -355,186 +414,301 @@ __global__ void contact_eval_kernel(int P, const int32_t *__restrict__ pairs, co
 
 // ------------------------------------------------------------------------- row reduction
 
-#define RR_WARPS 4
-#define RR_ENTRIES 128  // 32 references x up to 4 blocks
+#define RR_ROWS 32                     // rows per CTA
+#define RR_THREADS 128
+#define RR_CAP (RR_ROWS * 18)          // blocks of a tile staged in shared memory
 
-// Fetch element reference `ref`'s contribution to its local vertex's row: the
-// right-hand-side share (3 floats) and one block per element vertex (3 or 4), with the
-// column of each.
-__device__ __forceinline__ int fetch_contribution(uint32_t ref, const int32_t *__restrict__ tri,
-                                                  const int32_t *__restrict__ hinge,
-                                                  const int32_t *__restrict__ pairs,
-                                                  const float *__restrict__ tri_buf,
-                                                  const float *__restrict__ hinge_buf,
-                                                  const float *__restrict__ cont_buf, float *blk /*[4][9]*/,
-                                                  int *cols /*[4]*/, float *f /*[3]*/)
+// Contributions to one block (row, col), col != row, from the mesh's elements, in incidence
+// order: the static list of (type, k, l, id) codes that pc_create made for the block
+// (value_lists_kernel in pc_pattern.cu). Every product is rounded before it is added; block
+// (col, row) has the same elements in the same order and the products commute, so A is
+// bitwise symmetric.
+__device__ __forceinline__ void add_static(const uint32_t *__restrict__ codes, int c0, int c1,
+                                           const float *__restrict__ tri_buf, const float4 *__restrict__ hinge_buf,
+                                           float cl_cm, float acc[9])
 {
-    uint32_t type = pc_ref_type(ref), k = pc_ref_local(ref), id = pc_ref_id(ref);
-    if (type == PC_REF_TRI) {
-        const float *o = tri_buf + (int64_t)PC_TRI_STRIDE * id;
-        f[0] = o[3 * k]; f[1] = o[3 * k + 1]; f[2] = o[3 * k + 2];
-        for (int l = 0; l < 3; ++l) {
-            cols[l] = tri[3 * id + l];
-            const float *B = o + 9 + 9 * tri_blk(k < l ? k : l, k < l ? l : k);
-            if (k <= (uint32_t)l) {
-                for (int e = 0; e < 9; ++e) blk[9 * l + e] = B[e];
-            } else {
-                for (int a = 0; a < 3; ++a)
-                    for (int b = 0; b < 3; ++b) blk[9 * l + 3 * a + b] = B[3 * b + a];
+    for (int c = c0; c < c1; ++c) {
+        const uint32_t code = codes[c];
+        const int k = (int)((code >> 29) & 3u), l = (int)((code >> 27) & 3u);
+        const uint32_t id = code & PC_CODE_ID;
+        if (code & PC_CODE_HINGE) {
+            const float4 qk = hinge_buf[4ll * id + k], ql = hinge_buf[4ll * id + l];
+            const float a[3] = {qk.x, qk.y, qk.z}, b[3] = {ql.x, ql.y, ql.z};
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) acc[3 * i + j] = __fadd_rn(acc[3 * i + j], __fmul_rn(a[i], b[j]));
+        } else {
+            const TriFactors R = tri_load(tri_buf, id, cl_cm);
+            // the block of the vertex pair in its canonical order (lower local index first),
+            // transposed for the other row
+            const int lo = min(k, l), hi = max(k, l);
+            float F0[3], F1[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                F0[a] = lo == 0 ? R.Fg[0][a] : R.Fg[1][a];
+                F1[a] = hi == 1 ? R.Fg[1][a] : R.Fg[2][a];
             }
-        }
-        return 3;
-    }
-    if (type == PC_REF_HINGE) {
-        const float *o = hinge_buf + (int64_t)PC_HINGE_STRIDE * id;
-        f[0] = o[3 * k]; f[1] = o[3 * k + 1]; f[2] = o[3 * k + 2];
-        float qk[3] = {o[12 + 3 * k], o[12 + 3 * k + 1], o[12 + 3 * k + 2]};
-        for (int l = 0; l < 4; ++l) {
-            cols[l] = hinge[4 * id + l];
-            const float *ql = o + 12 + 3 * l;
+            const float gg = lo == 1 ? R.gg[4] : (hi == 1 ? R.gg[1] : R.gg[2]);
+            const float s = lo == 1 ? R.s[4] : (hi == 1 ? R.s[1] : R.s[2]);
+            float B[9];
+            const float m[9] = {R.M[0], R.M[1], R.M[2], R.M[1], R.M[3], R.M[4], R.M[2], R.M[4], R.M[5]};
+#pragma unroll
             for (int a = 0; a < 3; ++a)
-                for (int b = 0; b < 3; ++b) blk[9 * l + 3 * a + b] = qk[a] * ql[b];
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    float v = __fmul_rn(gg, m[3 * a + b]);
+                    v = fmaf(__fmul_rn(R.cm, F1[a]), F0[b], v);
+                    v = fmaf(__fmul_rn(R.cl, F0[a]), F1[b], v);
+                    B[3 * a + b] = a == b ? __fadd_rn(v, s) : v;
+                }
+            const bool tr = k > l;
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) acc[3 * a + b] = __fadd_rn(acc[3 * a + b], tr ? B[3 * b + a] : B[3 * a + b]);
         }
-        return 4;
     }
-    const float *o = cont_buf + (int64_t)PC_CONTACT_STRIDE * id;
-    f[0] = o[3 * k]; f[1] = o[3 * k + 1]; f[2] = o[3 * k + 2];
-    float n[3] = {o[12], o[13], o[14]};
-    float s[4] = {1.0f, -o[15], -o[16], -o[17]};
-    float c = o[18];
-    for (int l = 0; l < 4; ++l) {
-        cols[l] = pairs[4 * id + l];
-        float cs = c * (s[k] * s[l]);
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) blk[9 * l + 3 * a + b] = cs * (n[a] * n[b]);
-    }
-    return 4;
 }
 
-// One warp per row. Lane s owns slot s of the row (in chunks of 32 slots); lanes stage
-// the contributions of up to 32 incident elements at a time in shared memory, and each
-// slot owner adds the staged blocks whose column matches its own, in staging order
-// (static incidence order, then contact order). Then mass, pins and the right-hand side.
-__global__ void __launch_bounds__(32 * RR_WARPS) row_reduce_kernel(
-    int V, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const int32_t *__restrict__ vinc_ptr,
-    const uint32_t *__restrict__ vinc, const int32_t *__restrict__ cinc_ptr, const uint32_t *__restrict__ cinc,
-    const int32_t *__restrict__ tri, const int32_t *__restrict__ hinge, const int32_t *__restrict__ pairs,
-    const float *__restrict__ tri_buf, const float *__restrict__ hinge_buf, const float *__restrict__ cont_buf,
-    const float *__restrict__ mass, const uint8_t *__restrict__ pinned, float gx, float gy, float gz, float h,
-    float md, float ha, const float *__restrict__ v, float *__restrict__ vals, float *__restrict__ b,
-    float *__restrict__ dres)
+// Contributions of the row's contacts to block (row, col), in contact order.
+__device__ __forceinline__ void add_contacts(const uint32_t *__restrict__ cinc, int c0, int c1,
+                                             const int32_t *__restrict__ pairs, const float *__restrict__ cont_buf,
+                                             int col, float acc[9])
 {
-    __shared__ float s_blk[RR_WARPS][RR_ENTRIES][9];
-    __shared__ int s_col[RR_WARPS][RR_ENTRIES];
-    __shared__ float s_f[RR_WARPS][32][3];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = blockIdx.x * RR_WARPS + warp;
-    if (row >= V) return;
-    const int s0 = rp[row], nslots = rp[row + 1] - s0;
-    const int i0 = vinc_ptr[row], ni = vinc_ptr[row + 1] - i0;
-    const int c0 = cinc_ptr[row], nc = cinc_ptr[row + 1] - c0;
-    const int nref = ni + nc;
-    const float m = mass[row];
-    const float mA = md * m;  // diagonal mass term (1 + h alpha) m of an unpinned row
-    const bool prow = pinned[row] != 0;
-    float fsum[3] = {0.f, 0.f, 0.f};
-    float dsum[9];
+    for (int i = c0; i < c1; ++i) {
+        const uint32_t ref = cinc[i], k = pc_ref_local(ref), id = pc_ref_id(ref);
+        const int32_t *pv = pairs + 4ll * id;
+        const int l = pv[0] == col ? 0 : pv[1] == col ? 1 : pv[2] == col ? 2 : pv[3] == col ? 3 : -1;
+        if (l < 0) continue;
+        const float *o = cont_buf + (int64_t)PC_CONTACT_STRIDE * id;
+        const float sk = k == 0 ? 1.0f : -o[14 + k], sl = l == 0 ? 1.0f : -o[14 + l];
+        const float cs = o[18] * (sk * sl);
+        const float n[3] = {o[12], o[13], o[14]};
 #pragma unroll
-    for (int e = 0; e < 9; ++e) dsum[e] = 0.f;
-
-    for (int sc = 0; sc < nslots; sc += 32) {
-        const bool has = sc + lane < nslots;
-        const int slot = s0 + sc + lane;
-        const int col = has ? ci[slot] : -1;
-        float acc[9];
+        for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int e = 0; e < 9; ++e) acc[e] = 0.f;
-        for (int rc = 0; rc < nref; rc += 32) {
-            const int k = rc + lane;
-            float blk[36];
-            int cols[4] = {-1, -1, -1, -1};
-            float f[3] = {0.f, 0.f, 0.f};
-            if (k < nref) {
-                uint32_t ref = k < ni ? vinc[i0 + k] : cinc[c0 + (k - ni)];
-                fetch_contribution(ref, tri, hinge, pairs, tri_buf, hinge_buf, cont_buf, blk, cols, f);
-            }
-#pragma unroll
-            for (int l = 0; l < 4; ++l) {
-                s_col[warp][4 * lane + l] = cols[l];
-                if (cols[l] >= 0)
-#pragma unroll
-                    for (int e = 0; e < 9; ++e) s_blk[warp][4 * lane + l][e] = blk[9 * l + e];
-            }
-            s_f[warp][lane][0] = f[0];
-            s_f[warp][lane][1] = f[1];
-            s_f[warp][lane][2] = f[2];
-            __syncwarp();
-            const int cnt = min(32, nref - rc);
-            for (int e = 0; e < 4 * cnt; ++e) {
-                if (s_col[warp][e] == col) {
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) acc[q] += s_blk[warp][e][q];
-                }
-            }
-            if (sc == 0 && lane == 0) {
-                for (int e = 0; e < cnt; ++e) {
-                    fsum[0] += s_f[warp][e][0];
-                    fsum[1] += s_f[warp][e][1];
-                    fsum[2] += s_f[warp][e][2];
-                }
-            }
-            __syncwarp();
-        }
-        if (has) {
-            const bool pcol = pinned[col] != 0;
-            float outv[9];
-            if (prow || pcol) {
-#pragma unroll
-                for (int q = 0; q < 9; ++q) outv[q] = 0.f;
-                if (col == row) outv[0] = outv[4] = outv[8] = m;
-                if (pcol && !prow && col != row) {
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) dsum[q] += acc[q];
-                }
-            } else {
-#pragma unroll
-                for (int q = 0; q < 9; ++q) outv[q] = acc[q];
-                if (col == row) {
-                    outv[0] += mA;
-                    outv[4] += mA;
-                    outv[8] += mA;
-                }
-            }
-            float *dst = vals + 9ll * slot;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) dst[q] = outv[q];
-        }
+            for (int b = 0; b < 3; ++b) acc[3 * a + b] = __fadd_rn(acc[3 * a + b], __fmul_rn(cs, __fmul_rn(n[a], n[b])));
     }
-    // difference-form diagonal: m I minus the unzeroed blocks toward pinned neighbours
+}
+
+struct RowArgs {
+    int V;
+    const int32_t *rp, *ci;            // this step's pattern
+    const int32_t *srp, *scol;         // static pattern
+    const int32_t *lptr;               // [static blocks + 1] contributions of each static block
+    const uint32_t *codes;
+    const int32_t *vinc_ptr;
+    const uint32_t *vinc;
+    const int32_t *cinc_ptr;
+    const uint32_t *cinc;
+    const int32_t *pairs;
+    const float *tri_buf;
+    const float4 *hinge_buf;
+    const float *cont_buf;
+    const float *mass;
+    const uint8_t *pinned, *pin_adj;   // pinned vertex; some static neighbour is pinned
+    float gx, gy, gz, h, md, ha, cl_cm;
+    const float *v;
+    float *vals, *b, *dres;
+};
+
+// The unzeroed block at dynamic slot `slot` of `row` (column `col` != row).
+__device__ __forceinline__ void row_block(const RowArgs &a, int row, int slot, int col, int s0, int s1, int t0, int t1,
+                                          int n0, int n1, float acc[9])
+{
 #pragma unroll
-    for (int q = 0; q < 9; ++q)
-        for (int o = 16; o > 0; o >>= 1) dsum[q] += __shfl_xor_sync(0xffffffffu, dsum[q], o);
-    if (lane == 0) {
-        if (dres) {
-            float *d = dres + 9ll * row;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) d[q] = prow ? 0.f : -dsum[q];
-            const float md_row = prow ? m : mA;
-            d[0] += md_row;
-            d[4] += md_row;
-            d[8] += md_row;
+    for (int q = 0; q < 9; ++q) acc[q] = 0.f;
+    int ss = t0 + (slot - s0);  // static slot: the same place unless contacts added columns to the row
+    if (s1 - s0 != t1 - t0) {
+        int lo = t0, hi = t1;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (a.scol[mid] < col) lo = mid + 1; else hi = mid;
         }
-        float *bb = b + 3ll * row;
+        ss = lo < t1 && a.scol[lo] == col ? lo : -1;
+    }
+    if (ss >= 0) add_static(a.codes, a.lptr[ss], a.lptr[ss + 1], a.tri_buf, a.hinge_buf, a.cl_cm, acc);
+    if (n1 > n0) add_contacts(a.cinc, n0, n1, a.pairs, a.cont_buf, col, acc);
+}
+
+// One CTA per 32 rows. Warp 0 first forms the rows' diagonal blocks, right-hand sides and
+// difference-form diagonals, one thread per row over the row's incident elements; the
+// other blocks go one per thread, over the block's own contribution list, in chunks of 32
+// handed out by a shared counter (warp 0 joins when its rows are done; which warp takes a
+// chunk does not change any sum). Blocks are staged in shared memory and leave as whole
+// lines; a tile with more than RR_CAP blocks writes them directly.
+// Bound by DRAM and L2: 44 B per block written (vals and its column read), about 5
+// contributions of 64..128 B per block read through L1. At 830k rows / 10.9M blocks: before,
+// a warp per row staged every expanded block and each lane compared all of them with
+// its column, 2,825 us.
+__global__ void __launch_bounds__(RR_THREADS) row_reduce_kernel(RowArgs a)
+{
+    __shared__ float s_blk[RR_CAP * 9];
+    __shared__ int s_rp[RR_ROWS + 1], s_sp[RR_ROWS + 1], s_cp[RR_ROWS + 1];
+    __shared__ int s_next;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r0 = blockIdx.x * RR_ROWS, nr = min(RR_ROWS, a.V - r0);
+    for (int i = threadIdx.x; i <= nr; i += RR_THREADS) {
+        s_rp[i] = a.rp[r0 + i];
+        s_sp[i] = a.srp[r0 + i];
+        s_cp[i] = a.cinc_ptr[r0 + i];
+    }
+    if (threadIdx.x == 0) s_next = 0;
+    __syncthreads();
+    const int b0 = s_rp[0], nblk = s_rp[nr] - b0;
+    const bool staged = nblk <= RR_CAP;
+
+    if (warp == 0 && lane < nr) {
+        const int row = r0 + lane;
+        const int s0 = s_rp[lane], s1 = s_rp[lane + 1], t0 = s_sp[lane], t1 = s_sp[lane + 1];
+        const int n0 = s_cp[lane], n1 = s_cp[lane + 1];
+        const float m = a.mass[row];
+        const float mA = a.md * m;  // diagonal mass term (1 + h alpha) m of an unpinned row
+        const bool prow = a.pinned[row] != 0;
+        float f[3] = {0.f, 0.f, 0.f};
+        float u[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // upper triangle 00 01 02 11 12 22
+        const int i1 = a.vinc_ptr[row + 1];
+        for (int i = a.vinc_ptr[row]; i < i1; ++i) {
+            const uint32_t ref = a.vinc[i], k = pc_ref_local(ref), id = pc_ref_id(ref);
+            if (pc_ref_type(ref) == PC_REF_HINGE) {
+                const float4 q = a.hinge_buf[4ll * id + k];
+                f[0] = fmaf(q.x, q.w, f[0]);
+                f[1] = fmaf(q.y, q.w, f[1]);
+                f[2] = fmaf(q.z, q.w, f[2]);
+                u[0] = __fadd_rn(u[0], __fmul_rn(q.x, q.x));
+                u[1] = __fadd_rn(u[1], __fmul_rn(q.x, q.y));
+                u[2] = __fadd_rn(u[2], __fmul_rn(q.x, q.z));
+                u[3] = __fadd_rn(u[3], __fmul_rn(q.y, q.y));
+                u[4] = __fadd_rn(u[4], __fmul_rn(q.y, q.z));
+                u[5] = __fadd_rn(u[5], __fmul_rn(q.z, q.z));
+            } else {
+                const float4 c = reinterpret_cast<const float4 *>(a.tri_buf)[8ll * id + k];
+                f[0] += c.x;
+                f[1] += c.y;
+                f[2] += c.z;
+                const TriFactors R = tri_load(a.tri_buf, id, a.cl_cm);
+                float F[3];
+#pragma unroll
+                for (int e = 0; e < 3; ++e) F[e] = k == 0 ? R.Fg[0][e] : k == 1 ? R.Fg[1][e] : R.Fg[2][e];
+                const float gg = k == 0 ? R.gg[0] : k == 1 ? R.gg[3] : R.gg[5];
+                const float s = k == 0 ? R.s[0] : k == 1 ? R.s[3] : R.s[5];
+                const float cf = R.cm + R.cl;
+                u[0] += fmaf(cf * F[0], F[0], fmaf(gg, R.M[0], s));
+                u[1] += fmaf(cf * F[0], F[1], gg * R.M[1]);
+                u[2] += fmaf(cf * F[0], F[2], gg * R.M[2]);
+                u[3] += fmaf(cf * F[1], F[1], fmaf(gg, R.M[3], s));
+                u[4] += fmaf(cf * F[1], F[2], gg * R.M[4]);
+                u[5] += fmaf(cf * F[2], F[2], fmaf(gg, R.M[5], s));
+            }
+        }
+        bool adj = a.pin_adj[row] != 0;
+        for (int i = n0; i < n1; ++i) {
+            const uint32_t ref = a.cinc[i], k = pc_ref_local(ref), id = pc_ref_id(ref);
+            const float *o = a.cont_buf + (int64_t)PC_CONTACT_STRIDE * id;
+            f[0] += o[3 * k];
+            f[1] += o[3 * k + 1];
+            f[2] += o[3 * k + 2];
+            const float sk = k == 0 ? 1.0f : -o[14 + k], cs = o[18] * (sk * sk);
+            const float n[3] = {o[12], o[13], o[14]};
+            u[0] = __fadd_rn(u[0], __fmul_rn(cs, __fmul_rn(n[0], n[0])));
+            u[1] = __fadd_rn(u[1], __fmul_rn(cs, __fmul_rn(n[0], n[1])));
+            u[2] = __fadd_rn(u[2], __fmul_rn(cs, __fmul_rn(n[0], n[2])));
+            u[3] = __fadd_rn(u[3], __fmul_rn(cs, __fmul_rn(n[1], n[1])));
+            u[4] = __fadd_rn(u[4], __fmul_rn(cs, __fmul_rn(n[1], n[2])));
+            u[5] = __fadd_rn(u[5], __fmul_rn(cs, __fmul_rn(n[2], n[2])));
+            const int32_t *pv = a.pairs + 4ll * id;
+            adj |= a.pinned[pv[0]] || a.pinned[pv[1]] || a.pinned[pv[2]] || a.pinned[pv[3]];
+        }
+        float B[9] = {u[0], u[1], u[2], u[1], u[3], u[4], u[2], u[4], u[5]};
+        // the diagonal's slot; its list holds elements that meet the vertex twice (two
+        // triangles on the same three vertices): none on an ordinary mesh
+        int lo = s0, hi = s1;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (a.ci[mid] < row) lo = mid + 1; else hi = mid;
+        }
+        const int ds = lo;
+        int sl = t0, sh = t1;
+        if (s1 - s0 == t1 - t0) {
+            sl = t0 + (ds - s0);
+        } else {
+            while (sl < sh) {
+                const int mid = (sl + sh) >> 1;
+                if (a.scol[mid] < row) sl = mid + 1; else sh = mid;
+            }
+        }
+        if (a.lptr[sl + 1] > a.lptr[sl])
+            add_static(a.codes, a.lptr[sl], a.lptr[sl + 1], a.tri_buf, a.hinge_buf, a.cl_cm, B);
+        // difference-form diagonal: m I minus the unzeroed blocks toward pinned neighbours
+        if (a.dres) {
+            float D[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            if (adj && !prow)
+                for (int slot = s0; slot < s1; ++slot) {
+                    const int col = a.ci[slot];
+                    if (col == row || !a.pinned[col]) continue;
+                    float acc[9];
+                    row_block(a, row, slot, col, s0, s1, t0, t1, n0, n1, acc);
+#pragma unroll
+                    for (int q = 0; q < 9; ++q) D[q] -= acc[q];
+                }
+            D[0] += prow ? m : mA;
+            D[4] += prow ? m : mA;
+            D[8] += prow ? m : mA;
+#pragma unroll
+            for (int q = 0; q < 9; ++q) a.dres[9ll * row + q] = D[q];
+        }
+        float *bb = a.b + 3ll * row;
         if (prow) {
             bb[0] = bb[1] = bb[2] = 0.f;
+#pragma unroll
+            for (int q = 0; q < 9; ++q) B[q] = 0.f;
+            B[0] = B[4] = B[8] = m;
         } else {
             // gravity and the mass-damping force at v_t, both times h
-            const float hm = h * m, ham = ha * m;
-            bb[0] = fsum[0] + hm * gx - ham * v[3ll * row];
-            bb[1] = fsum[1] + hm * gy - ham * v[3ll * row + 1];
-            bb[2] = fsum[2] + hm * gz - ham * v[3ll * row + 2];
+            const float hm = a.h * m, ham = a.ha * m;
+            bb[0] = f[0] + hm * a.gx - ham * a.v[3ll * row];
+            bb[1] = f[1] + hm * a.gy - ham * a.v[3ll * row + 1];
+            bb[2] = f[2] + hm * a.gz - ham * a.v[3ll * row + 2];
+            B[0] += mA;
+            B[4] += mA;
+            B[8] += mA;
         }
+        float *dst = staged ? s_blk + 9 * (ds - b0) : a.vals + 9ll * ds;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) dst[q] = B[q];
     }
+    __syncwarp();
+
+    for (;;) {
+        int c = 0;
+        if (lane == 0) c = atomicAdd(&s_next, 32);
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if (c >= nblk) break;
+        const int i = c + lane;
+        if (i >= nblk) continue;
+        const int slot = b0 + i;
+        int r = 0;  // the row: last r with s_rp[r] <= slot
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1)
+            if (r + step < nr && s_rp[r + step] <= slot) r += step;
+        const int row = r0 + r, col = a.ci[slot];
+        if (col == row) continue;
+        float acc[9];
+        if (a.pinned[row] || a.pinned[col]) {
+#pragma unroll
+            for (int q = 0; q < 9; ++q) acc[q] = 0.f;
+        } else {
+            row_block(a, row, slot, col, s_rp[r], s_rp[r + 1], s_sp[r], s_sp[r + 1], s_cp[r], s_cp[r + 1], acc);
+        }
+        float *dst = staged ? s_blk + 9 * i : a.vals + 9ll * slot;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) dst[q] = acc[q];
+    }
+    if (!staged) return;
+    __syncthreads();
+    float *o = a.vals + 9ll * b0;
+    for (int i = threadIdx.x; i < 9 * nblk; i += RR_THREADS) o[i] = s_blk[i];
 }
 
 extern "C" pc_status pc_assemble_values(pc_ctx *ctx, const pc_bsr *A, const float *x, const float *v,
@@ -553,7 +727,7 @@ extern "C" pc_status pc_assemble_values(pc_ctx *ctx, const pc_bsr *A, const floa
     const float hk = h * (h + ctx->mat.damp_stiff);
     const float md = 1.0f + h * ctx->mat.damp_mass, ha = h * ctx->mat.damp_mass;
     if (T > 0)
-        PC_LAUNCH(ctx, tri_eval_kernel, pc_blocks(T, 128), 128, 0, st, T, ctx->tri, x, v, ctx->tri_dmi, ctx->tri_area,
+        PC_LAUNCH(ctx, tri_eval_kernel, pc_blocks(T, TE_THREADS), TE_THREADS, 0, st, T, ctx->tri, x, v, ctx->tri_dmi, ctx->tri_area,
                   ctx->tri_rgram, ctx->mu, ctx->lam, h, hk, ctx->tri_buf);
     if (H > 0)
         PC_LAUNCH(ctx, hinge_eval_kernel, pc_blocks(H, 128), 128, 0, st, H, ctx->hinge, x, v, ctx->hcoef, ctx->hrest, h,
@@ -561,9 +735,36 @@ extern "C" pc_status pc_assemble_values(pc_ctx *ctx, const pc_bsr *A, const floa
     if (P > 0)
         PC_LAUNCH(ctx, contact_eval_kernel, pc_blocks(P, 128), 128, 0, st, P, contacts->pairs, contacts->w, x, v,
                   ctx->mat.k_contact, h, hk, ctx->mat.contact_thickness, ctx->cont_buf);
-    PC_LAUNCH(ctx, row_reduce_kernel, pc_blocks(V, RR_WARPS), 32 * RR_WARPS, 0, st, V, A->row_ptr, A->col_idx,
-              ctx->vinc_ptr, ctx->vinc, ctx->cinc_ptr, ctx->cinc, ctx->tri, ctx->hinge,
-              P > 0 ? contacts->pairs : nullptr, ctx->tri_buf, ctx->hinge_buf, ctx->cont_buf, ctx->mass, ctx->pinned,
-              ctx->mat.gravity[0], ctx->mat.gravity[1], ctx->mat.gravity[2], h, md, ha, v, vals, b, dres);
+    RowArgs r{};
+    r.V = V;
+    r.rp = A->row_ptr;
+    r.ci = A->col_idx;
+    r.srp = ctx->srp;
+    r.scol = ctx->scol;
+    r.lptr = ctx->val_ptr;
+    r.codes = ctx->val_codes;
+    r.vinc_ptr = ctx->vinc_ptr;
+    r.vinc = ctx->vinc;
+    r.cinc_ptr = ctx->cinc_ptr;
+    r.cinc = ctx->cinc;
+    r.pairs = P > 0 ? contacts->pairs : nullptr;
+    r.tri_buf = ctx->tri_buf;
+    r.hinge_buf = reinterpret_cast<const float4 *>(ctx->hinge_buf);
+    r.cont_buf = ctx->cont_buf;
+    r.mass = ctx->mass;
+    r.pinned = ctx->pinned;
+    r.pin_adj = ctx->pin_adj;
+    r.gx = ctx->mat.gravity[0];
+    r.gy = ctx->mat.gravity[1];
+    r.gz = ctx->mat.gravity[2];
+    r.h = h;
+    r.md = md;
+    r.ha = ha;
+    r.cl_cm = ctx->lam / ctx->mu;
+    r.v = v;
+    r.vals = vals;
+    r.b = b;
+    r.dres = dres;
+    PC_LAUNCH(ctx, row_reduce_kernel, pc_blocks(V, RR_ROWS), RR_THREADS, 0, st, r);
     return PC_OK;
 }
