@@ -118,12 +118,13 @@ struct pc_ctx {
 
     // per-step contact data
     uint64_t *dkeys = nullptr;     // [6 * maxP] dynamic pattern keys (sorted)
-    uint64_t *dnew = nullptr;      // [6 * maxP] keys not in the static pattern
-    int32_t *dflag = nullptr;      // [6 * maxP + 1]
+    uint64_t *dnew = nullptr;      // [6 * maxP] new columns by row (int32), or keys not in the static pattern
+    int32_t *dflag = nullptr;      // [6 * maxP + 1] entries' arrival numbers, or flags
     int32_t *dscan = nullptr;      // [6 * maxP + 1]
     uint64_t *ckeys = nullptr;     // [4 * maxP] incidence keys (vertex)
     uint32_t *cinc = nullptr;      // [4 * maxP] contact refs grouped by vertex
     int32_t *cinc_ptr = nullptr;   // [V+1]
+    int32_t *row_cnt = nullptr;    // [2V + 2] per-row counts, heavy-row flag, offsets of the new columns
     int32_t n_new = 0;
     int32_t n_contacts = 0;        // contacts of the last pattern call
     const int32_t *last_pairs = nullptr;

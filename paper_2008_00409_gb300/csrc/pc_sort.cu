@@ -159,11 +159,56 @@ __global__ void scan_add_kernel(int32_t *out, int64_t n, const int32_t *tile_sum
     }
 }
 
+// Up to SCAN_SMALL values in one CTA: one launch instead of three (each about 3 us, which
+// is what a small system's scans cost).
+#define SCAN_SMALL 16384
+#define SCAN_SMALL_THREADS 1024
+__global__ void __launch_bounds__(SCAN_SMALL_THREADS) scan_small_kernel(const int32_t *in, int32_t *out, int n)
+{
+    __shared__ int32_t s_warp[SCAN_SMALL_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = (n + SCAN_SMALL_THREADS - 1) / SCAN_SMALL_THREADS;  // <= 16
+    const int b = threadIdx.x * per;
+    int32_t v[SCAN_SMALL / SCAN_SMALL_THREADS], s = 0;
+#pragma unroll
+    for (int k = 0; k < SCAN_SMALL / SCAN_SMALL_THREADS; ++k) {
+        v[k] = k < per && b + k < n ? in[b + k] : 0;
+        s += v[k];
+    }
+    int32_t x = s;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();  // every input has been read: `in` and `out` may alias
+    if (warp == 0) {
+        int32_t w = s_warp[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        s_warp[lane] = w;
+    }
+    __syncthreads();
+    int32_t ex = (warp > 0 ? s_warp[warp - 1] : 0) + x - s;
+#pragma unroll
+    for (int k = 0; k < SCAN_SMALL / SCAN_SMALL_THREADS; ++k) {
+        if (k < per && b + k < n) out[b + k] = ex;
+        ex += v[k];
+    }
+    if (threadIdx.x == 0) out[n] = s_warp[SCAN_SMALL_THREADS / 32 - 1];
+}
+
 // out[0..n-1] = exclusive scan of in, out[n] = total. `in` and `out` may alias.
 pc_status pc_exclusive_scan(pc_ctx *ctx, const int32_t *in, int32_t *out, int64_t n, cudaStream_t st)
 {
     if (n <= 0) {
         PC_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(int32_t), st));
+        return PC_OK;
+    }
+    if (n <= SCAN_SMALL) {
+        PC_LAUNCH(ctx, scan_small_kernel, 1, SCAN_SMALL_THREADS, 0, st, in, out, (int)n);
         return PC_OK;
     }
     int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
