@@ -168,6 +168,15 @@ struct pc_ctx {
     int64_t od_nnzb = 0;                             // blocks of the last copy
     float *dsc = nullptr;                            // [V] scalar difference diagonal or -1
     struct pc_fuse_bar *fbar = nullptr;              // grid barrier of the fused PCG update
+    // patch storage (pc_patch.cuh): row order (once per context) and the records of the last solve
+    int pt_rows = 0, pt_n = 0;                       // rows per patch, patches
+    int64_t pt_cap = 0;                              // bytes of the store
+    int32_t *pt_old = nullptr, *pt_new = nullptr;    // [V] original number of a new one, and back
+    void *pt_desc = nullptr;                         // [pt_n] PatchDesc
+    uint8_t *pt_cnt = nullptr;                       // [pt_n pt_rows] kept blocks per row
+    int32_t *pt_size = nullptr;                      // [2][pt_n + 1] record sizes, offsets
+    int32_t *pt_info = nullptr;                      // [8]
+    unsigned char *pt_store = nullptr;
     // proximity query: cell list (8 entries per triangle) and counts
     int64_t px_cap = 0;
     uint64_t *px_keys = nullptr;
@@ -295,6 +304,14 @@ pc_status pc_warm_guess(pc_ctx *c, const pc_bsr *A, const float *v, float h, int
                         int32_t *guess, double *guess_res, double *guess_energy, double *guess_coef,
                         double *combo_energy, cudaStream_t st);
 void pc_mlp_ctx_free(pc_ctx *c);
+// Patch storage of the system being solved (pc_patch.cu): allocation and row order, and the
+// records of one matrix (ok = false: the matrix does not suit it and nothing is usable).
+struct PatchInfo {
+    bool ok;
+    int32_t max_bytes, max_halo, max_own;  // largest record, largest halo, most kept blocks
+};
+pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st);
+pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, PatchInfo *out, cudaStream_t st);
 // The whole solve in one thread-block cluster (pc_cluster.cu). Runs when the system fits
 // the cluster's shared memory (*ran = true, returns the solve's status); otherwise
 // returns PC_OK with *ran = false, or PC_ERR_CAPACITY when `required`. Needs c->dinv

@@ -120,6 +120,8 @@ static __device__ bool last_block_reduce_df(float *hi, float *lo, int n, double 
 #include "pc_spmv.cuh"
 #include "pc_spmv_sym.cuh"
 #include "pc_spmv_sell.cuh"
+#include "pc_patch.cuh"
+static_assert(PT_RED_SLOTS == RED_SLOTS, "the partials array is shared");
 
 // ------------------------------------------------------------------------- preconditioner
 
@@ -161,10 +163,12 @@ __device__ __forceinline__ void st3(float *__restrict__ a, int row, float4 v)
 // to PC_ERR_ARG; a bad row's entries are not read).
 template <bool BLOCK>
 __global__ void dinv_kernel(int V, int64_t nnzb, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                            const float *__restrict__ vals, float *__restrict__ dinv, uint32_t *err)
+                            const float *__restrict__ vals, float *__restrict__ dinv, uint32_t *err,
+                            const int32_t *__restrict__ new_of)
 {
     int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= V) return;
+    const int w = new_of ? new_of[r] : r;  // the row's place among the solve's vectors
     const int k0 = rp[r], k1 = rp[r + 1];
     int s = -1;
     if (k0 < 0 || k1 < k0 || (int64_t)k1 > nnzb) {
@@ -180,7 +184,7 @@ __global__ void dinv_kernel(int V, int64_t nnzb, const int32_t *__restrict__ rp,
     for (int e = 0; e < 9; ++e) B[e] = s >= 0 ? (double)vals[9ll * s + e] : 0.0;
     bool ok = s >= 0 && B[0] > 0.0 && B[4] > 0.0 && B[8] > 0.0 && isfinite(B[0] + B[4] + B[8]);
     if (!BLOCK) {
-        float *d = dinv + 3ll * r;  // packed: three floats per row
+        float *d = dinv + 3ll * w;  // packed: three floats per row
         d[0] = ok ? (float)(1.0 / B[0]) : 1.f;
         d[1] = ok ? (float)(1.0 / B[4]) : 1.f;
         d[2] = ok ? (float)(1.0 / B[8]) : 1.f;
@@ -192,13 +196,13 @@ __global__ void dinv_kernel(int V, int64_t nnzb, const int32_t *__restrict__ rp,
         double det = B[0] * c00 + B[1] * c10 + B[2] * c20;
         ok = ok && det > 0.0 && isfinite(det);
         if (ok) {
-            dinv4[3ll * r] = make_float4((float)(c00 / det), (float)(c01 / det), (float)(c02 / det), 0.f);
-            dinv4[3ll * r + 1] = make_float4((float)(c10 / det), (float)(c11 / det), (float)(c12 / det), 0.f);
-            dinv4[3ll * r + 2] = make_float4((float)(c20 / det), (float)(c21 / det), (float)(c22 / det), 0.f);
+            dinv4[3ll * w] = make_float4((float)(c00 / det), (float)(c01 / det), (float)(c02 / det), 0.f);
+            dinv4[3ll * w + 1] = make_float4((float)(c10 / det), (float)(c11 / det), (float)(c12 / det), 0.f);
+            dinv4[3ll * w + 2] = make_float4((float)(c20 / det), (float)(c21 / det), (float)(c22 / det), 0.f);
         } else {
-            dinv4[3ll * r] = make_float4(1.f, 0.f, 0.f, 0.f);
-            dinv4[3ll * r + 1] = make_float4(0.f, 1.f, 0.f, 0.f);
-            dinv4[3ll * r + 2] = make_float4(0.f, 0.f, 1.f, 0.f);
+            dinv4[3ll * w] = make_float4(1.f, 0.f, 0.f, 0.f);
+            dinv4[3ll * w + 1] = make_float4(0.f, 1.f, 0.f, 0.f);
+            dinv4[3ll * w + 2] = make_float4(0.f, 0.f, 1.f, 0.f);
         }
     }
     if (!ok) pc_set_err(err, PC_DERR_NONFINITE);
@@ -345,18 +349,20 @@ __global__ void __launch_bounds__(EW_THREADS) pcg_init_kernel(int V, const float
                                                                const float *__restrict__ dinv4,
                                                                float4 *__restrict__ z4, float4 *__restrict__ p4,
                                                                float *__restrict__ x4, double tol, int max_iter,
-                                                               double *partials, pc_scalars *sc, int fused)
+                                                               double *partials, pc_scalars *sc, int fused,
+                                                               const int32_t *__restrict__ new_of)
 {
     double rz = 0.0, rr = 0.0, bb = 0.0;
     for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < V; row += gridDim.x * blockDim.x) {
         const float b0 = b[3ll * row], b1 = b[3ll * row + 1], b2 = b[3ll * row + 2];
         const float4 r = make_float4(b0 - q[3ll * row], b1 - q[3ll * row + 1], b2 - q[3ll * row + 2], 0.f);
-        const float4 z = apply_precond<BLOCK>(dinv4, row, r);
-        st3(r4, row, r);
-        z4[row] = z;
+        const int w = new_of ? new_of[row] : row;
+        const float4 z = apply_precond<BLOCK>(dinv4, w, r);
+        st3(r4, w, r);
+        z4[w] = z;
         // the fused update leaves p ready for the next product: start from p = z
-        p4[row] = fused ? z : make_float4(0.f, 0.f, 0.f, 0.f);
-        st3(x4, row, make_float4(0.f, 0.f, 0.f, 0.f));
+        p4[w] = fused ? z : make_float4(0.f, 0.f, 0.f, 0.f);
+        st3(x4, w, make_float4(0.f, 0.f, 0.f, 0.f));
         rz += (double)dot3(r, z);
         rr += (double)dot3(r, r);
         bb += (double)b0 * b0 + (double)b1 * b1 + (double)b2 * b2;
@@ -591,7 +597,8 @@ __global__ void __launch_bounds__(EW_THREADS) residual_replace_kernel(
     int V, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const float *__restrict__ vals,
     const float *__restrict__ dres, const float *__restrict__ b, const double *__restrict__ x64,
     const float *__restrict__ dinv4, float *__restrict__ r4, float4 *__restrict__ z4, float4 *__restrict__ p4,
-    int first, double tol, int max_iter, double *partials, pc_scalars *sc, int fused)
+    int first, double tol, int max_iter, double *partials, pc_scalars *sc, int fused,
+    const int32_t *__restrict__ new_of)
 {
     double rz = 0.0, rr = 0.0, bb = 0.0;
     for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < V; row += gridDim.x * blockDim.x) {
@@ -606,25 +613,26 @@ __global__ void __launch_bounds__(EW_THREADS) residual_replace_kernel(
             rf[a2] = (float)rv;
         }
         const float4 r = make_float4(rf[0], rf[1], rf[2], 0.f);
-        const float4 z = apply_precond<BLOCK>(dinv4, row, r);
+        const int w = new_of ? new_of[row] : row;  // the vectors may be in the patches' row order
+        const float4 z = apply_precond<BLOCK>(dinv4, w, r);
         if (fused) {
             // p already holds z_old + beta p_prev (the fused update applied the direction
             // step): swap z_old for the replaced z, p = z + beta p_prev as without fusion
             if (first) {
-                p4[row] = z;
+                p4[w] = z;
             } else {
-                const float4 zo = apply_precond<BLOCK>(dinv4, row, ld3(r4, row));
-                float4 pv = p4[row];
+                const float4 zo = apply_precond<BLOCK>(dinv4, w, ld3(r4, w));
+                float4 pv = p4[w];
                 pv.x += z.x - zo.x;
                 pv.y += z.y - zo.y;
                 pv.z += z.z - zo.z;
-                p4[row] = pv;
+                p4[w] = pv;
             }
         } else if (first) {
-            p4[row] = make_float4(0.f, 0.f, 0.f, 0.f);
+            p4[w] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        st3(r4, row, r);
-        z4[row] = z;
+        st3(r4, w, r);
+        z4[w] = z;
         rz += (double)dot3(r, z);
     }
     double v[3] = {rz, rr, bb};
@@ -655,21 +663,22 @@ __global__ void __launch_bounds__(EW_THREADS) residual_replace_kernel(
 }
 
 // x64 += increment; increment = 0 (per row, float4 increment)
-__global__ void fold_kernel(int V, float *x4, double *x64)
+__global__ void fold_kernel(int V, float *x4, double *x64, const int32_t *__restrict__ new_of)
 {
     for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < V; row += gridDim.x * blockDim.x) {
-        const float4 d = ld3(x4, row);
+        const int w = new_of ? new_of[row] : row;
+        const float4 d = ld3(x4, w);
         x64[3ll * row] += (double)d.x;
         x64[3ll * row + 1] += (double)d.y;
         x64[3ll * row + 2] += (double)d.z;
-        st3(x4, row, make_float4(0.f, 0.f, 0.f, 0.f));
+        st3(x4, w, make_float4(0.f, 0.f, 0.f, 0.f));
     }
 }
 // dv += increment (FP32 solve)
-__global__ void add_increment_kernel(int V, const float *x4, float *dv)
+__global__ void add_increment_kernel(int V, const float *x4, float *dv, const int32_t *__restrict__ new_of)
 {
     for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < V; row += gridDim.x * blockDim.x) {
-        const float4 d = ld3(x4, row);
+        const float4 d = ld3(x4, new_of ? new_of[row] : row);
         dv[3ll * row] += d.x;
         dv[3ll * row + 1] += d.y;
         dv[3ll * row + 2] += d.z;
@@ -892,6 +901,9 @@ struct SolveCtx {
     bool fuse;     // update and direction in one kernel (pcg_update_dir_kernel)
     int fu_grid, fu_rows;
     int capr = SP_CAPR_WIDE;  // the product's stage width (blocks per row)
+    bool patch = false;       // the products read the patch storage, the vectors are in its row order
+    int pt_grid = 0, pt_smem = 0, pt_rec = 0, pt_halo = 0;
+    const int32_t *new_of = nullptr;  // the vectors' place of an original row (null: the same)
 };
 
 // ------------------------------------------------------------------------- symmetric storage
@@ -1029,14 +1041,15 @@ static pc_status build_sell(pc_ctx *c, const pc_bsr *A, const float *vals, bool 
 // dsc[i] = s when the difference-form diagonal of row i is exactly s I with s > 0 (every
 // row away from pins: its lumped mass term), else -1 (the product then reads all nine
 // entries). The product is bitwise the same either way.
-__global__ void dsc_kernel(int V, const float *__restrict__ dres, float *__restrict__ dsc)
+__global__ void dsc_kernel(int V, const float *__restrict__ dres, float *__restrict__ dsc,
+                           const int32_t *__restrict__ new_of)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= V) return;
     const float *D = dres + 9ll * i;
     const bool scalar = D[1] == 0.f && D[2] == 0.f && D[3] == 0.f && D[5] == 0.f && D[6] == 0.f && D[7] == 0.f &&
                         D[0] == D[4] && D[4] == D[8] && D[0] > 0.f;
-    dsc[i] = scalar ? D[0] : -1.f;
+    dsc[new_of ? new_of[i] : i] = scalar ? D[0] : -1.f;
 }
 
 // ------------------------------------------------------------------------- off-diagonal BSR
@@ -1140,7 +1153,8 @@ pc_status pc_build_offdiag_async(pc_ctx *c, const pc_bsr *A, const float *vals, 
     PC_TRY(pc_exclusive_scan(c, c->od_cnt, c->od_rp, V, st));
     PC_LAUNCH(c, od_fill_kernel, pc_blocks(32ll * V, 256), 256, 0, st, V, A->row_ptr, A->col_idx, vals, c->od_dpos,
               c->od_rp, c->od_cap, c->od_ci, c->od_vals, c->d_err);
-    if (dres && c->dsc) PC_LAUNCH(c, dsc_kernel, pc_blocks(V, 256), 256, 0, st, V, dres, c->dsc);
+    if (dres && c->dsc) PC_LAUNCH(c, dsc_kernel, pc_blocks(V, 256), 256, 0, st, V, dres, c->dsc,
+                                    static_cast<const int32_t *>(nullptr));
     return PC_OK;
 }
 
@@ -1169,10 +1183,10 @@ static pc_status read_scalars(pc_ctx *c, cudaStream_t st)
 static pc_status replace_residual(const SolveCtx &s, float *x32, int first, double tol, int max_iter)
 {
     pc_ctx *c = s.c;
-    if (!first) PC_LAUNCH(c, fold_kernel, ew_grid(c, c->V), EW_THREADS, 0, s.st, c->V, x32, c->x64);
+    if (!first) PC_LAUNCH(c, fold_kernel, ew_grid(c, c->V), EW_THREADS, 0, s.st, c->V, x32, c->x64, s.new_of);
     DISPATCH2(c, residual_replace_kernel, s.diff, s.block, ew_grid(c, c->V), EW_THREADS, s.st, c->V, s.A->row_ptr,
               s.A->col_idx, s.vals, s.dres, s.b, c->x64, c->dinv, c->r, (float4 *)c->z,
-              (float4 *)c->p0, first, tol, max_iter, c->partials, c->sc, (int)s.fuse);
+              (float4 *)c->p0, first, tol, max_iter, c->partials, c->sc, (int)s.fuse, s.new_of);
     return PC_OK;
 }
 
@@ -1222,7 +1236,7 @@ static pc_status launch_iterations(const SolveCtx &s, float *x, int count)
     a.partials = c->partials;
     a.sc = c->sc;
     a.err = c->d_err;
-    const int n_pq = s.sell ? sell_grid(c) : s.sym ? sym_grid(c) : spmv_grid(c, s.capr);
+    const int n_pq = s.patch ? s.pt_grid : s.sell ? sell_grid(c) : s.sym ? sym_grid(c) : spmv_grid(c, s.capr);
     c->ev_iter0 = c->sc_host->iter;  // the scalars were read before this chunk
     for (int k = 0; k < count; ++k) {
         // two sampled products per chunk: the first (after the host's check and the fold of
@@ -1234,7 +1248,25 @@ static pc_status launch_iterations(const SolveCtx &s, float *x, int count)
             PC_LAUNCH_PDL(c, pcg_direction_kernel, dir_grid(c, c->V), EW_THREADS, 0, s.st, c->V,
                           (const float4 *)c->z, (float4 *)c->p0, (const pc_scalars *)c->sc);
         if (timed) PC_CUDA_TRY(cudaEventRecord(c->ev[slot ? 6 : 0], s.st));
-        if (s.sym) {
+        if (s.patch) {
+            PatchArgs y{};
+            y.V = c->V;
+            y.R = c->pt_rows;
+            y.n = c->pt_n;
+            y.desc = static_cast<const PatchDesc *>(c->pt_desc);
+            y.store = c->pt_store;
+            y.rec_cap = s.pt_rec;
+            y.halo_cap = s.pt_halo;
+            y.dsc = c->dsc;
+            y.dres = s.dres;
+            y.old_of = c->pt_old;
+            y.x4 = (const float4 *)c->p0;
+            y.y4 = (float4 *)c->q;
+            y.partials = c->partials;
+            y.sc = c->sc;
+            y.err = c->d_err;
+            PC_LAUNCH_PDL(c, patch_spmv_kernel, s.pt_grid, PT_ROWS, s.pt_smem, s.st, y);
+        } else if (s.sym) {
             SymArgs y{};
             y.V = c->V;
             y.urp = c->sym_urp;
@@ -1290,7 +1322,7 @@ static pc_status launch_iterations(const SolveCtx &s, float *x, int count)
         if (timed) {
             // read after the chunk's synchronisation (no stall here)
             c->ev_pending = slot ? 2 : 1;
-            c->spmv_nnzb = s.offdiag ? c->od_nnzb : s.A->nnzb;
+            c->spmv_nnzb = s.patch ? s.A->nnzb - c->V : s.offdiag ? c->od_nnzb : s.A->nnzb;
         }
     }
     return PC_OK;
@@ -1331,6 +1363,43 @@ extern "C" pc_status pc_pcg_solve(pc_ctx *ctx, const pc_bsr *A, const float *val
     return pcg_solve_impl(ctx, A, vals, dres, b, dv, opts, info, stream);
 }
 
+static pc_status launch_dinv(const SolveCtx &s)
+{
+    pc_ctx *c = s.c;
+    if (s.block)
+        PC_LAUNCH(c, dinv_kernel<true>, pc_blocks(c->V, 256), 256, 0, s.st, c->V, s.A->nnzb, s.A->row_ptr,
+                  s.A->col_idx, s.vals, c->dinv, c->d_err, s.new_of);
+    else
+        PC_LAUNCH(c, dinv_kernel<false>, pc_blocks(c->V, 256), 256, 0, s.st, c->V, s.A->nnzb, s.A->row_ptr,
+                  s.A->col_idx, s.vals, c->dinv, c->d_err, s.new_of);
+    return PC_OK;
+}
+
+// Patch storage for the difference-form products where the matrix suits it and at least
+// three CTAs of the product fit an SM beside each other (with fewer, the copies of one no
+// longer hide behind the others): the vectors then take the patches' row order.
+static pc_status try_patch(SolveCtx &s)
+{
+    pc_ctx *c = s.c;
+    PatchInfo pi{};
+    PC_TRY(pc_patch_build(c, s.A, s.vals, &pi, s.st));
+    if (!pi.ok) return PC_OK;
+    int limit = 0;
+    PC_CUDA_TRY(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device));
+    s.pt_halo = pi.max_halo;
+    s.pt_rec = (pi.max_bytes + 127) / 128 * 128;
+    s.pt_smem = s.pt_rec + 12 * (c->pt_rows + pi.max_halo);
+    if (s.pt_smem > limit / 3) return PC_OK;
+    PC_CUDA_TRY(cudaFuncSetAttribute(patch_spmv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, s.pt_smem));
+    int occ = 0;
+    PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, patch_spmv_kernel, PT_ROWS, s.pt_smem));
+    if (occ < 3) return PC_OK;
+    s.pt_grid = std::min(std::min(c->pt_n, c->num_sms * occ), c->max_red_blocks);
+    s.patch = true;
+    s.new_of = c->pt_new;
+    return launch_dinv(s);
+}
+
 static pc_status pcg_solve_impl(pc_ctx *ctx, const pc_bsr *A, const float *vals, const float *dres,
                                 const float *b, float *dv, const pc_solve_opts *opts, pc_solve_info *info,
                                 void *stream)
@@ -1355,12 +1424,7 @@ static pc_status pcg_solve_impl(pc_ctx *ctx, const pc_bsr *A, const float *vals,
     if (s.fuse) PC_CUDA_TRY(cudaMemsetAsync(ctx->fbar, 0, sizeof(pc_fuse_bar), st));
     PC_CUDA_TRY(cudaMemsetAsync(ctx->d_err, 0, sizeof(uint32_t), st));
     // the preconditioner's pass also validates the pattern; nothing else reads it before
-    if (s.block)
-        PC_LAUNCH(ctx, dinv_kernel<true>, pc_blocks(V, 256), 256, 0, st, V, A->nnzb, A->row_ptr, A->col_idx, vals,
-                  ctx->dinv, ctx->d_err);
-    else
-        PC_LAUNCH(ctx, dinv_kernel<false>, pc_blocks(V, 256), 256, 0, st, V, A->nnzb, A->row_ptr, A->col_idx, vals,
-                  ctx->dinv, ctx->d_err);
+    PC_TRY(launch_dinv(s));
     uint32_t bits = 0;
     PC_TRY(pc_read_errors(ctx, st, &bits));  // synchronises the stream
     if (bits & PC_DERR_INDEX) return PC_ERR_ARG;
@@ -1374,10 +1438,14 @@ static pc_status pcg_solve_impl(pc_ctx *ctx, const pc_bsr *A, const float *vals,
     if (o.storage == PC_STORAGE_SYM) PC_TRY(build_sym(ctx, A, vals, &s.sym, st));
     if (o.storage == PC_STORAGE_SELL) PC_TRY(build_sell(ctx, A, vals, &s.sell, st));
     // the diagonal blocks multiply p_i - p_i = 0 in the difference form only
-    if (o.storage == PC_STORAGE_OFFDIAG && s.diff) PC_TRY(build_offdiag(ctx, A, vals, &s.offdiag, st));
-    if (s.diff && ctx->dsc) PC_LAUNCH(ctx, dsc_kernel, pc_blocks(V, 256), 256, 0, st, V, dres, ctx->dsc);
+    if (o.storage == PC_STORAGE_OFFDIAG && s.diff) {
+        if (ctx->dsc && ctx->pt_store) PC_TRY(try_patch(s));
+        if (!s.patch) PC_TRY(build_offdiag(ctx, A, vals, &s.offdiag, st));
+    }
+    if (s.diff && ctx->dsc) PC_LAUNCH(ctx, dsc_kernel, pc_blocks(V, 256), 256, 0, st, V, dres, ctx->dsc,
+                                          s.new_of);
     // the narrower stages (more CTAs per SM) when every tile of the streamed matrix fits
-    const bool tmax = !s.sym && !s.sell && ctx->d_count && ctx->h_count;
+    const bool tmax = !s.sym && !s.sell && !s.patch && ctx->d_count && ctx->h_count;
     if (tmax) {
         PC_CUDA_TRY(cudaMemsetAsync(ctx->d_count + 3, 0, sizeof(int64_t), st));
         PC_LAUNCH(ctx, tile_max_kernel, pc_blocks((V + SP_ROWS - 1) / SP_ROWS, 256), 256, 0, st, V,
@@ -1411,11 +1479,11 @@ static pc_status pcg_solve_impl(pc_ctx *ctx, const pc_bsr *A, const float *vals,
         if (s.block)
             PC_LAUNCH(ctx, pcg_init_kernel<true>, ew_grid(ctx, V), EW_THREADS, 0, st, V, b, ctx->rhs32,
                       ctx->r, ctx->dinv, (float4 *)ctx->z, (float4 *)ctx->p0, x,
-                      o.tol, o.max_iter, ctx->partials, ctx->sc, (int)s.fuse);
+                      o.tol, o.max_iter, ctx->partials, ctx->sc, (int)s.fuse, s.new_of);
         else
             PC_LAUNCH(ctx, pcg_init_kernel<false>, ew_grid(ctx, V), EW_THREADS, 0, st, V, b, ctx->rhs32,
                       ctx->r, ctx->dinv, (float4 *)ctx->z, (float4 *)ctx->p0, x,
-                      o.tol, o.max_iter, ctx->partials, ctx->sc, (int)s.fuse);
+                      o.tol, o.max_iter, ctx->partials, ctx->sc, (int)s.fuse, s.new_of);
     }
     PC_TRY(read_scalars(ctx, st));
     double rr_last = ctx->sc_host->rr;
@@ -1452,7 +1520,7 @@ static pc_status pcg_solve_impl(pc_ctx *ctx, const pc_bsr *A, const float *vals,
         // noise that the stiff matrix amplifies) then stays far below what a residual
         // replacement measures, and replacements do not undo the iterations' progress.
         if (mixed && launched > 0)
-            PC_LAUNCH(ctx, fold_kernel, ew_grid(ctx, V), EW_THREADS, 0, st, V, x, ctx->x64);
+            PC_LAUNCH(ctx, fold_kernel, ew_grid(ctx, V), EW_THREADS, 0, st, V, x, ctx->x64, s.new_of);
         PC_TRY(launch_iterations(s, x, chunk));
         launched += chunk;
         PC_TRY(read_scalars(ctx, st));
@@ -1467,7 +1535,7 @@ static pc_status pcg_solve_impl(pc_ctx *ctx, const pc_bsr *A, const float *vals,
     double rr = fin.rr, bb = fin.bb;
     if (mixed) {
         if (fin.iter > iter_last) {  // stopped early (limit / breakdown): fold what there is
-            PC_LAUNCH(ctx, fold_kernel, ew_grid(ctx, V), EW_THREADS, 0, st, V, x, ctx->x64);
+            PC_LAUNCH(ctx, fold_kernel, ew_grid(ctx, V), EW_THREADS, 0, st, V, x, ctx->x64, s.new_of);
         }
         PC_LAUNCH(ctx, f64_to_f32_kernel, ew_grid(ctx, n), EW_THREADS, 0, st, n, ctx->x64, dv);
         if (fin.iter > iter_last) {
@@ -1480,7 +1548,7 @@ static pc_status pcg_solve_impl(pc_ctx *ctx, const pc_bsr *A, const float *vals,
             bb = ctx->sc_host->bb;
         }
     } else {
-        PC_LAUNCH(ctx, add_increment_kernel, ew_grid(ctx, V), EW_THREADS, 0, st, V, x, dv);
+        PC_LAUNCH(ctx, add_increment_kernel, ew_grid(ctx, V), EW_THREADS, 0, st, V, x, dv, s.new_of);
         if (s.diff) PC_LAUNCH(ctx, residual_check_kernel<true>, ew_grid(ctx, V), EW_THREADS, 0, st, V, A->row_ptr,
                               A->col_idx, vals, dres, b, dv, ctx->partials, ctx->sc);
         else PC_LAUNCH(ctx, residual_check_kernel<false>, ew_grid(ctx, V), EW_THREADS, 0, st, V, A->row_ptr,
