@@ -174,8 +174,12 @@ struct pc_ctx {
     int32_t *pt_old = nullptr, *pt_new = nullptr;    // [V] original number of a new one, and back
     void *pt_desc = nullptr;                         // [pt_n] PatchDesc
     uint8_t *pt_cnt = nullptr;                       // [pt_n pt_rows] kept blocks per row
+    uint8_t *pt_named = nullptr;                     // [V] rows in some patch's halo
     int32_t *pt_size = nullptr;                      // [2][pt_n + 1] record sizes, offsets
     int32_t *pt_info = nullptr;                      // [8]
+    unsigned long long *pt_slots = nullptr;          // the resident schedule's published sums, then its abort flag
+    unsigned long long *pt_z = nullptr;              // [V][4] its exchanged z rows
+    uint32_t pt_epoch = 0;                           // its next epoch (0: slots and pt_z must be cleared)
     unsigned char *pt_store = nullptr;
     // proximity query: cell list (8 entries per triangle) and counts
     int64_t px_cap = 0;

@@ -111,7 +111,10 @@ __global__ void order_kernel(int V, const uint32_t *__restrict__ vals, int32_t *
 pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
 {
     const int V = c->V;
-    c->pt_rows = PT_ROWS;
+    // one patch per SM where that many rows' records can stay in shared memory (the resident
+    // schedule), else the streamed product's patches
+    const int per_sm = ((V + c->num_sms - 1) / c->num_sms + 31) / 32 * 32;
+    c->pt_rows = per_sm <= PT_RESIDENT_ROWS ? per_sm : PT_ROWS;
     c->pt_n = (V + c->pt_rows - 1) / c->pt_rows;
     // kept blocks at most all of them; entries 4 bytes each, twice that with the slices' padding
     c->pt_cap = 48 * c->A_cap + (int64_t)c->pt_n * 1024;
@@ -120,9 +123,14 @@ pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
     PC_CUDA_TRY(cudaMalloc(&c->pt_new, sizeof(int32_t) * (size_t)V));
     PC_CUDA_TRY(cudaMalloc(&c->pt_desc, sizeof(PatchDesc) * (size_t)c->pt_n));
     PC_CUDA_TRY(cudaMalloc(&c->pt_cnt, (size_t)c->pt_n * c->pt_rows));
+    PC_CUDA_TRY(cudaMalloc(&c->pt_named, (size_t)V));
     PC_CUDA_TRY(cudaMalloc(&c->pt_size, sizeof(int32_t) * 2 * (c->pt_n + 1ll)));
     PC_CUDA_TRY(cudaMalloc(&c->pt_info, sizeof(int32_t) * 8));
     PC_CUDA_TRY(cudaMalloc(&c->pt_store, (size_t)c->pt_cap));
+    if (c->pt_n <= c->num_sms) {
+        PC_CUDA_TRY(cudaMalloc(&c->pt_slots, sizeof(uint64_t) * (12 * (size_t)c->pt_n * c->pt_n + 1)));
+        PC_CUDA_TRY(cudaMalloc(&c->pt_z, 4 * sizeof(uint64_t) * (size_t)V));
+    }
     uint64_t *keys = nullptr;
     uint32_t *vals = nullptr;
     float *box = nullptr;
@@ -166,7 +174,7 @@ struct BuildArgs {
     const float *vals;
     const int32_t *new_of, *old_of;
     PatchDesc *desc;
-    uint8_t *cnt;           // kept blocks of each row
+    uint8_t *cnt, *named;   // kept blocks of each row; rows in some patch's halo
     int32_t *size, *at;     // record sizes and offsets, in 16-byte units
     int32_t *info;          // [0] no record (count), [1] largest record, [2] largest halo, [3] failure (fill), [4] most kept blocks
     int64_t cap;            // bytes of the store
@@ -298,6 +306,7 @@ __global__ void patch_count_kernel(BuildArgs a)
     }
     __syncthreads();
     const int nh = halo_sort(s_list, s_n);
+    for (int i = threadIdx.x; i < nh; i += blockDim.x) a.named[s_list[i]] = 1;
     if (threadIdx.x == 0) {
         PatchDesc d{};
         d.n_own = s_own;
@@ -467,6 +476,7 @@ pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, PatchInf
     a.old_of = c->pt_old;
     a.desc = static_cast<PatchDesc *>(c->pt_desc);
     a.cnt = c->pt_cnt;
+    a.named = c->pt_named;
     a.size = c->pt_size;
     a.at = c->pt_size + c->pt_n + 1;
     a.info = c->pt_info;
@@ -474,6 +484,7 @@ pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, PatchInf
     a.store = c->pt_store;
     const int threads = a.R < 128 ? 128 : a.R > 512 ? 512 : a.R;
     PC_CUDA_TRY(cudaMemsetAsync(c->pt_info, 0, sizeof(int32_t) * 5, st));
+    PC_CUDA_TRY(cudaMemsetAsync(c->pt_named, 0, (size_t)c->V, st));
     PC_LAUNCH(c, patch_count_kernel, c->pt_n, threads, 0, st, a);
     PC_TRY(pc_exclusive_scan(c, a.size, a.at, c->pt_n, st));
     PC_LAUNCH(c, patch_fill_kernel, c->pt_n, threads, 0, st, a);

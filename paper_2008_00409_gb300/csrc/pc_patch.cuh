@@ -32,6 +32,7 @@
 #include "pc_tma.cuh"
 
 #define PT_ROWS 128                       // rows per patch of the streamed product
+#define PT_RESIDENT_ROWS 480              // largest patch whose records and vectors can fit one SM's shared memory
 #define PT_MAX_ROWS 1024                  // largest patch the records can describe
 #define PT_SLICES (PT_MAX_ROWS / 32)
 #define PT_MAX_OWN 64                     // most kept blocks of one row

@@ -121,6 +121,7 @@ static __device__ bool last_block_reduce_df(float *hi, float *lo, int n, double 
 #include "pc_spmv_sym.cuh"
 #include "pc_spmv_sell.cuh"
 #include "pc_patch.cuh"
+#include "pc_resident.cuh"
 static_assert(PT_RED_SLOTS == RED_SLOTS, "the partials array is shared");
 
 // ------------------------------------------------------------------------- preconditioner
@@ -903,6 +904,8 @@ struct SolveCtx {
     int capr = SP_CAPR_WIDE;  // the product's stage width (blocks per row)
     bool patch = false;       // the products read the patch storage, the vectors are in its row order
     int pt_grid = 0, pt_smem = 0, pt_rec = 0, pt_halo = 0;
+    bool resident = false;    // the iterations run in pcg_resident_kernel
+    int pt_share = 0, pt_split = 0;
     const int32_t *new_of = nullptr;  // the vectors' place of an original row (null: the same)
 };
 
@@ -1375,6 +1378,66 @@ static pc_status launch_dinv(const SolveCtx &s)
     return PC_OK;
 }
 
+static const void *resident_kernel(const SolveCtx &s)
+{
+    if (s.pt_split == 4)
+        return s.block ? (const void *)pcg_resident_kernel<4, true> : (const void *)pcg_resident_kernel<4, false>;
+    return s.block ? (const void *)pcg_resident_kernel<2, true> : (const void *)pcg_resident_kernel<2, false>;
+}
+
+// Iterations until the solve stops or needs a residual replacement.
+static pc_status launch_resident(const SolveCtx &s, float *x, const pc_solve_opts &o, double rr_last, int iter_last)
+{
+    pc_ctx *c = s.c;
+    const bool mixed = o.precision == PC_PREC_MIXED;
+    ResArgs a{};
+    a.V = c->V;
+    a.R = c->pt_rows;
+    a.n = c->pt_n;
+    a.desc = static_cast<const PatchDesc *>(c->pt_desc);
+    a.store = c->pt_store;
+    a.rec_cap = s.pt_rec;
+    a.share_cap = s.pt_share;
+    a.halo_cap = s.pt_halo;
+    a.dsc = c->dsc;
+    a.dres = s.dres;
+    a.old_of = c->pt_old;
+    a.named = c->pt_named;
+    a.dinv = c->dinv;
+    a.x = x;
+    a.r = c->r;
+    a.p = (float4 *)c->p0;
+    a.z = c->pt_z;
+    a.x64 = mixed ? c->x64 : nullptr;
+    a.rr_last = rr_last;
+    a.refresh2 = o.refresh * o.refresh;
+    a.iter_last = iter_last;
+    a.refresh_every = o.refresh_every;
+    a.check_every = o.check_every;
+    a.slots = c->pt_slots;
+    a.abort_flag = reinterpret_cast<unsigned *>(c->pt_slots + RES_WORDS(c->pt_n));
+    // two epochs per iteration; never one that is still written anywhere
+    const int64_t span = 2ll * (o.max_iter - c->sc_host->iter) + 4;
+    if (c->pt_epoch == 0 || (int64_t)c->pt_epoch + span > 0xffffffffll) {
+        PC_CUDA_TRY(cudaMemsetAsync(c->pt_slots, 0, sizeof(uint64_t) * (RES_WORDS(c->pt_n) + 1), s.st));
+        PC_CUDA_TRY(cudaMemsetAsync(c->pt_z, 0, 4 * sizeof(uint64_t) * (size_t)c->V, s.st));
+        c->pt_epoch = 1;
+    }
+    a.epoch0 = c->pt_epoch;
+    c->pt_epoch = 0;  // known again once the launch has been waited for
+    a.sc = c->sc;
+    a.err = c->d_err;
+    a.budget = c->bar_wait_cycles > 0 ? (long long)c->bar_wait_cycles : PT_WAIT_BUDGET;
+    void *args[] = {&a};
+    PC_CUDA_TRY(cudaLaunchCooperativeKernel(resident_kernel(s), dim3(c->pt_n), dim3(s.pt_split * c->pt_rows), args,
+                                            (size_t)s.pt_smem, s.st));
+    c->launches++;
+    const int iter0 = c->sc_host->iter;
+    PC_TRY(read_scalars(c, s.st));
+    if (c->sc_host->status != PC_ERR_TIMEOUT) c->pt_epoch = a.epoch0 + 2u * (unsigned)(c->sc_host->iter - iter0) + 1u;
+    return PC_OK;
+}
+
 // Patch storage for the difference-form products where the matrix suits it and at least
 // three CTAs of the product fit an SM beside each other (with fewer, the copies of one no
 // longer hide behind the others): the vectors then take the patches' row order.
@@ -1388,13 +1451,33 @@ static pc_status try_patch(SolveCtx &s)
     PC_CUDA_TRY(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device));
     s.pt_halo = pi.max_halo;
     s.pt_rec = (pi.max_bytes + 127) / 128 * 128;
-    s.pt_smem = s.pt_rec + 12 * (c->pt_rows + pi.max_halo);
-    if (s.pt_smem > limit / 3) return PC_OK;
-    PC_CUDA_TRY(cudaFuncSetAttribute(patch_spmv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, s.pt_smem));
-    int occ = 0;
-    PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, patch_spmv_kernel, PT_ROWS, s.pt_smem));
-    if (occ < 3) return PC_OK;
-    s.pt_grid = std::min(std::min(c->pt_n, c->num_sms * occ), c->max_red_blocks);
+    if (c->pt_slots) {
+        // one CTA per patch for the whole solve, if everything fits (the fused update's stop
+        // tests and direction step; fuse = 0 keeps the separate kernels)
+        if (!s.fuse || c->pt_n > c->num_sms) return PC_OK;
+        int coop = 0, most = 0, occ = 0;
+        PC_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
+        PC_CUDA_TRY(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+        s.pt_split = c->pt_rows <= 256 ? 4 : 2;
+        s.pt_share = pi.max_own + 1;
+        s.pt_smem = s.pt_rec + 16 * s.pt_share + 12 * (c->pt_rows + pi.max_halo) + 12 * (s.pt_split - 1) * c->pt_rows;
+        const void *k = resident_kernel(s);
+        cudaFuncAttributes fa;
+        PC_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
+        if (!coop || s.pt_smem + (int)fa.sharedSizeBytes > most) return PC_OK;
+        PC_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, s.pt_smem));
+        PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, s.pt_split * c->pt_rows, s.pt_smem));
+        if (occ < 1) return PC_OK;
+        s.resident = true;
+    } else {
+        s.pt_smem = s.pt_rec + 12 * (c->pt_rows + pi.max_halo);
+        if (s.pt_smem > limit / 3) return PC_OK;
+        PC_CUDA_TRY(cudaFuncSetAttribute(patch_spmv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, s.pt_smem));
+        int occ = 0;
+        PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, patch_spmv_kernel, PT_ROWS, s.pt_smem));
+        if (occ < 3) return PC_OK;
+        s.pt_grid = std::min(std::min(c->pt_n, c->num_sms * occ), c->max_red_blocks);
+    }
     s.patch = true;
     s.new_of = c->pt_new;
     return launch_dinv(s);
@@ -1511,6 +1594,12 @@ static pc_status pcg_solve_impl(pc_ctx *ctx, const pc_bsr *A, const float *vals,
             PC_TRY(read_scalars(ctx, st));
             rr_last = ctx->sc_host->rr;
             iter_last = ctx->sc_host->iter;
+            continue;
+        }
+        if (s.resident) {
+            PC_TRY(launch_resident(s, x, o, rr_last, iter_last));  // and the scalars are read
+            if (ctx->sc_host->iter == h.iter && !ctx->sc_host->done) return PC_ERR_TIMEOUT;  // no progress: cannot be
+            launched = ctx->sc_host->iter;
             continue;
         }
         int chunk = o.check_every;
