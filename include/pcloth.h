@@ -29,10 +29,10 @@
  *  - A context (pc_ctx) holds one mesh's rest state and all scratch memory of the
  *    assembly and solve calls, allocated once by pc_create. The calls that allocate
  *    device memory are: pc_create; pc_mlp_create (training state); pc_set_warm_mlp
- *    (the context's feature and guess buffers, on the first attach); pc_mlp_infer (a
- *    4-byte timeout flag, on its first call in each host thread on each device, kept
- *    until the process exits); pc_step_batched (the CUDA graph it instantiates on its
- *    first call for a system shape). pc_pcg_solve_static allocates nothing at all.
+ *    (the context's feature and guess buffers, on the first attach); pc_step_batched
+ *    (the CUDA graph it instantiates on its first call for a system shape). pc_mlp_infer
+ *    keeps one pinned host word per host thread. pc_pcg_solve_static allocates nothing
+ *    at all.
  */
 #ifndef PCLOTH_H
 #define PCLOTH_H

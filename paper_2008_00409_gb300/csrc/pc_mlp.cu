@@ -48,22 +48,27 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 
 // ------------------------------------------------------------------------- inference (tcgen05)
 
-// One CTA of four warps per 128-row tile (persistent over tiles): the three layers are
+// One CTA of eight warps per 128-row tile (persistent over tiles): the three layers are
 // tcgen05 MMAs (M = 128, K = 16 per instruction, BF16 operands from shared memory, FP32
 // accumulators in tensor memory), issued by one thread and committed to an mbarrier;
-// warp w reads tensor-memory lanes 32w.. (its 32 rows), adds the bias, applies the ReLU
-// and writes the BF16 activations back to shared memory as the next layer's A operand.
+// warp w reads tensor-memory lanes 32 (w % 4).. (its 32 rows) and half the columns, adds the
+// bias, applies the ReLU and writes the BF16 activations back to shared memory as the next
+// layer's A operand. Bound by the latency of the dependent steps of a tile (input, three
+// products, three epilogues), so what counts is tiles in flight: four CTAs per SM (their
+// 4 x 128 columns are all of the SM's 512), two threads per row, and the next tile's inputs
+// fetched during the products. 501,264 rows: 75 us with two CTAs of four warps per SM.
 #define TC_ROWS 128
-#define TC_THREADS 128
+#define TC_THREADS 256
 #define TC_TMEM_COLS 128  // D1 at column 0, D2 at 64, D3 at 0 again
 #define TC_OFF_W1 0       // 64 x 16 BF16 (2 KB)
 #define TC_OFF_W2 2048    // 64 x 64 (8 KB)
 #define TC_OFF_W3 10240   // 16 x 64, outputs 3..15 zero (2 KB)
 #define TC_OFF_X 12288    // 128 x 16 (4 KB)
 #define TC_OFF_H 16384    // 128 x 64 (16 KB)
-// padded so that at most two CTAs share an SM: their 2 x 128 tensor-memory columns
+// padded so that at most four CTAs share an SM: their 4 x 128 tensor-memory columns
 // always fit in the SM's 512, so an allocation never waits
-#define TC_SMEM_BYTES (100 * 1024)
+#define TC_SMEM_BYTES (50 * 1024)
+#define TC_CTAS_PER_SM 4
 #define TC_WAIT_BUDGET (1ll << 31)  // cycles (about a second) before an MMA wait gives up
 
 // byte offset of element (row, k) of a K-major operand with K columns (no swizzle)
@@ -77,12 +82,12 @@ __device__ __forceinline__ void tc_put(unsigned char *base, int row, int k, int 
     *reinterpret_cast<__nv_bfloat16 *>(base + tc_off(row, k, K)) = __float2bfloat16_rn(v);
 }
 
-// Bias + ReLU of 64 accumulator columns (tensor memory, this thread's row) into the BF16
-// A operand (row t, K = 64).
-__device__ __forceinline__ void tc_hidden(uint32_t taddr, const float *bias, unsigned char *H, int t)
+// Bias + ReLU of accumulator columns c0 .. c0 + 31 (tensor memory, this thread's row) into the
+// BF16 A operand (row t, K = 64).
+__device__ __forceinline__ void tc_hidden(uint32_t taddr, const float *bias, unsigned char *H, int t, int c0)
 {
 #pragma unroll
-    for (int c = 0; c < 64; c += 16) {
+    for (int c = c0; c < c0 + 32; c += 16) {
         float v[16];
         tc_ld16(taddr + c, v);
         uint32_t q[8];
@@ -95,7 +100,31 @@ __device__ __forceinline__ void tc_hidden(uint32_t taddr, const float *bias, uns
 }
 
 // dv0 = dv_prev + sd_y * net(standardised feat) + mu_y; rows with fixed[r] != 0 get 0.
-__global__ void __launch_bounds__(TC_THREADS) mlp_infer_kernel(int64_t n, const float *params, const float *stats,
+struct TcInput {
+    float x[MLP_IN];
+};
+
+// The row's features: three 16-byte loads where the array allows them.
+__device__ __forceinline__ void tc_input(const float *feat, bool wide, int64_t r, int64_t n, TcInput &in)
+{
+    if (r >= n) return;
+    const float *x = feat + MLP_IN * r;
+    if (wide) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float4 v = reinterpret_cast<const float4 *>(x)[k];
+            in.x[4 * k] = v.x;
+            in.x[4 * k + 1] = v.y;
+            in.x[4 * k + 2] = v.z;
+            in.x[4 * k + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < MLP_IN; ++k) in.x[k] = x[k];
+    }
+}
+
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_PER_SM) mlp_infer_kernel(int64_t n, const float *params, const float *stats,
                                                                const float *feat, const float *dv_prev,
                                                                const uint8_t *fixed, float *dv0, uint32_t *err)
 {
@@ -105,6 +134,11 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_infer_kernel(int64_t n, const 
     __shared__ int s_fail;
     __shared__ float b1[MLP_HID], b2[MLP_HID], b3[4], mx[MLP_IN], sx[MLP_IN], my[4], sy[4];
     const int t = threadIdx.x, warp = t >> 5;
+    const int tr = t & (TC_ROWS - 1), half = t / TC_ROWS;  // row of the tile, half of the columns
+    const bool wide = (reinterpret_cast<uintptr_t>(feat) & 15u) == 0;
+    const int64_t ntiles = (n + TC_ROWS - 1) / TC_ROWS;
+    TcInput in;
+    if (half == 0) tc_input(feat, wide, (int64_t)blockIdx.x * TC_ROWS + tr, n, in);
     // weights as BF16 operands (B = W, N x K, K-major)
     for (int i = t; i < MLP_HID * 16; i += TC_THREADS) {
         const int r = i >> 4, k = i & 15;
@@ -142,28 +176,34 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_infer_kernel(int64_t n, const 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
-    const uint32_t lanes = (uint32_t)(32 * warp) << 16;
+    const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
     const uint32_t idesc64 = tc_idesc_bf16(TC_ROWS, 64), idesc16 = tc_idesc_bf16(TC_ROWS, 16);
     unsigned char *X = tsm + TC_OFF_X, *H = tsm + TC_OFF_H;
     uint32_t phase = 0;
-    const int64_t ntiles = (n + TC_ROWS - 1) / TC_ROWS;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t r = tile * TC_ROWS + t;
-        // ---- standardised inputs of row t as the BF16 A operand (K = 16, inputs 12..15 zero)
-        {
+        const int64_t r = tile * TC_ROWS + tr;
+        // ---- standardised inputs of the row as the BF16 A operand (K = 16, inputs 12..15 zero)
+        float prev[MLP_OUT] = {0.f, 0.f, 0.f};
+        bool fx = false;
+        if (half == 0) {
             float v[16];
 #pragma unroll
             for (int k = 0; k < 16; ++k) v[k] = 0.f;
             if (r < n) {
-                const float *x = feat + MLP_IN * r;
 #pragma unroll
-                for (int k = 0; k < MLP_IN; ++k) v[k] = (x[k] - mx[k]) / sx[k];
+                for (int k = 0; k < MLP_IN; ++k) v[k] = (in.x[k] - mx[k]) / sx[k];
             }
             uint32_t q[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) q[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-            *reinterpret_cast<uint4 *>(X + tc_off(t, 0, 16)) = make_uint4(q[0], q[1], q[2], q[3]);
-            *reinterpret_cast<uint4 *>(X + tc_off(t, 8, 16)) = make_uint4(q[4], q[5], q[6], q[7]);
+            *reinterpret_cast<uint4 *>(X + tc_off(tr, 0, 16)) = make_uint4(q[0], q[1], q[2], q[3]);
+            *reinterpret_cast<uint4 *>(X + tc_off(tr, 8, 16)) = make_uint4(q[4], q[5], q[6], q[7]);
+            if (r < n) {
+                fx = fixed && fixed[r];
+#pragma unroll
+                for (int o = 0; o < MLP_OUT; ++o) prev[o] = dv_prev ? dv_prev[3 * r + o] : 0.f;
+            }
+            tc_input(feat, wide, r + (int64_t)gridDim.x * TC_ROWS, n, in);
         }
         // three layers: MMA(s) by thread 0, wait on the commit, epilogue by every thread
         for (int layer = 0; layer < 3; ++layer) {
@@ -192,19 +232,16 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_infer_kernel(int64_t n, const 
             tc_fence_after();
             if (s_fail) break;
             if (layer == 0) {
-                tc_hidden(tmem + lanes, b1, H, t);
+                tc_hidden(tmem + lanes, b1, H, tr, 32 * half);
             } else if (layer == 1) {
-                tc_hidden(tmem + lanes + 64, b2, H, t);
-            } else {
+                tc_hidden(tmem + lanes + 64, b2, H, tr, 32 * half);
+            } else if (half == 0) {
                 float y[16];
                 tc_ld16(tmem + lanes, y);
                 if (r < n) {
-                    const bool fx = fixed && fixed[r];
 #pragma unroll
-                    for (int o = 0; o < MLP_OUT; ++o) {
-                        const float d = dv_prev ? dv_prev[3 * r + o] : 0.f;
-                        dv0[3 * r + o] = fx ? 0.f : fmaf(y[o] + b3[o], sy[o], my[o]) + d;
-                    }
+                    for (int o = 0; o < MLP_OUT; ++o)
+                        dv0[3 * r + o] = fx ? 0.f : fmaf(y[o] + b3[o], sy[o], my[o]) + prev[o];
                 }
             }
         }
@@ -213,16 +250,24 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_infer_kernel(int64_t n, const 
     // every tensor-memory read of this CTA is complete before the columns are released
     tc_fence_before();
     __syncthreads();
-    if (s_fail && t == 0) pc_set_err(err, PC_DERR_TIMEOUT);
+    if (s_fail && t == 0) {
+        *(volatile uint32_t *)err = PC_DERR_TIMEOUT;
+        __threadfence_system();
+    }
     if (warp == 0) tc_dealloc(tmem, TC_TMEM_COLS);
 }
 
 // ------------------------------------------------------------------------- training (tcgen05)
 //
-// One CTA of four warps per SM (persistent over 128-row tiles; its shared memory keeps a
+// One CTA of sixteen warps per SM (persistent over 128-row tiles; its shared memory keeps a
 // second CTA off the SM, so the CTA owns all 512 tensor-memory columns). Per tile, one
-// thread issues the tensor-core products and every thread handles its own row in the
-// epilogues (warp w reads tensor-memory lanes 32w.., the tile's rows 32w..):
+// thread issues the tensor-core products and every thread handles 16 columns of one row in
+// the epilogues (warp w reads tensor-memory lanes 32 (w % 4).., the tile's rows, and columns
+// 16 (w / 4)..). A tile is a chain of seven dependent products and their epilogues, one tile
+// at a time per SM, so it is bound by the epilogues' latency: with four warps (a thread per
+// row, all 64 columns) a step of 65,536 rows took 82 us in this kernel. The bias gradients'
+// column sums over a warp's rows (tt_column_sums) take 16 shuffles per 16 columns instead
+// of 80:
 //   forward   D1 = X W1^T, D2 = H1 W2^T, D3 = H2 W3^T                  (M = 128 rows)
 //   backward  dH2 = dY W3, dH1 = dZ2 W2                                (M = 128 rows)
 //   gradients [dZ2^T ; dZ1^T] [H1^T ; X^T]^T   (M = 128: dW2 and dW1 are its diagonal
@@ -236,7 +281,7 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_infer_kernel(int64_t n, const 
 // the loss are summed on the CUDA cores from the unrounded FP32 signals, per warp in a
 // fixed order, so training stays bit-reproducible.
 #define TT_ROWS 128
-#define TT_THREADS 128
+#define TT_THREADS 512
 #define TT_TMEM_COLS 512  // D1 / dH2 at 0, D2 / dH1 at 64, D3 at 128, gradients at 256 and 352
 #define TT_GW12 256       // 80 columns: [dW2 | dW1] blocks
 #define TT_GW3 352        // 16 columns: dW3^T
@@ -256,11 +301,42 @@ __global__ void __launch_bounds__(TC_THREADS) mlp_infer_kernel(int64_t n, const 
 #define TT_TDY 149504     // 16 x 128: dY^T (rows 3..15 zero)
 #define TT_SMEM 153600    // 150 KB: one CTA per SM
 
-// Sum over the warp's 32 rows (lane 0 holds the total).
+// Sum over the warp's 32 rows (every lane holds the total).
 __device__ __forceinline__ float tt_warp_sum(float v)
 {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+
+// Sums over the warp's 32 rows of 16 columns at once: each step adds the partner lane's
+// values as the butterfly above does, and keeps the half of the columns that the lane's bit
+// selects. Lanes 2 c and 2 c + 1, read with c's four bits from the highest lane bit down,
+// end with column c: the same sums, bit for bit, as 16 butterflies.
+__device__ __forceinline__ float tt_column_sums(const float (&v)[16], int lane, int &col)
+{
+    float a[8], b[4], c[2], d;
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4, h2 = lane & 2;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float give = h16 ? v[i] : v[8 + i], keep = h16 ? v[8 + i] : v[i];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float give = h8 ? a[i] : a[4 + i], keep = h8 ? a[4 + i] : a[i];
+        b[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float give = h4 ? b[i] : b[2 + i], keep = h4 ? b[2 + i] : b[i];
+        c[i] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+    }
+    {
+        const float give = h2 ? c[0] : c[1], keep = h2 ? c[1] : c[0];
+        d = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+    }
+    col = (h16 ? 8 : 0) + (h8 ? 4 : 0) + (h4 ? 2 : 0) + (h2 ? 1 : 0);
+    return d + __shfl_xor_sync(0xffffffffu, d, 1);
 }
 
 // Thread 0 issues `nk` K-steps of an M = 128 product into tensor memory and commits; every
@@ -303,6 +379,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1) mlp_train_kernel(int64_t n, con
     __shared__ float sdb[4][2 * MLP_HID + 4];  // per-warp bias-gradient sums: db1, db2, db3
     __shared__ double sloss[4];
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int tr = t & (TT_ROWS - 1), rw = warp & 3, cb = 16 * (t / TT_ROWS);  // row, row warp, first column
     // weights in the four layouts the products read; every other buffer starts at zero
     // (the padding columns of X, dY, their transposes and of W3 are never written again)
     for (int i = t; i < (TT_SMEM - TT_X) / 16; i += TT_THREADS)
@@ -345,7 +422,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1) mlp_train_kernel(int64_t n, con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_slot, lanes = (uint32_t)(32 * warp) << 16;
+    const uint32_t tmem = tmem_slot, lanes = (uint32_t)(32 * rw) << 16;
     const uint32_t id64 = tc_idesc_bf16(TT_ROWS, 64), id16 = tc_idesc_bf16(TT_ROWS, 16);
     const uint32_t id80 = tc_idesc_bf16(TT_ROWS, 80);
     unsigned char *X = tsm + TT_X, *H1 = tsm + TT_H1, *H2 = tsm + TT_H2, *DY = tsm + TT_DY, *DZ2 = tsm + TT_DZ2;
@@ -356,122 +433,124 @@ __global__ void __launch_bounds__(TT_THREADS, 1) mlp_train_kernel(int64_t n, con
     bool first = true;
     const int64_t ntiles = (n + TT_ROWS - 1) / TT_ROWS;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t r = tile * TT_ROWS + t;
+        const int64_t r = tile * TT_ROWS + tr;
         const int64_t R = r < n ? (rows ? (int64_t)rows[r] : r) : 0;
-        // ---- standardised inputs: row t of X and column t of X^T (rows past n are zero)
-        {
+        float tn[MLP_OUT] = {0.f, 0.f, 0.f};  // standardised targets (column block 0)
+        // ---- standardised inputs: the row of X and the column of X^T (rows past n are zero)
+        if (cb == 0) {
             float v[16];
 #pragma unroll
             for (int k = 0; k < 16; ++k) v[k] = 0.f;
             if (r < n) {
                 const float *x = feat + (int64_t)MLP_IN * R;
+                float xv[MLP_IN];
 #pragma unroll
-                for (int k = 0; k < MLP_IN; ++k) v[k] = (x[k] - mx[k]) / sx[k];
+                for (int k = 0; k < MLP_IN; ++k) xv[k] = x[k];
+#pragma unroll
+                for (int o = 0; o < MLP_OUT; ++o) tn[o] = ((target[3 * R + o] - xv[3 + o]) - my[o]) / sy[o];  // dv - dv_prev
+#pragma unroll
+                for (int k = 0; k < MLP_IN; ++k) v[k] = (xv[k] - mx[k]) / sx[k];
             }
             uint32_t q[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) q[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-            *reinterpret_cast<uint4 *>(X + tc_off(t, 0, 16)) = make_uint4(q[0], q[1], q[2], q[3]);
-            *reinterpret_cast<uint4 *>(X + tc_off(t, 8, 16)) = make_uint4(q[4], q[5], q[6], q[7]);
+            *reinterpret_cast<uint4 *>(X + tc_off(tr, 0, 16)) = make_uint4(q[0], q[1], q[2], q[3]);
+            *reinterpret_cast<uint4 *>(X + tc_off(tr, 8, 16)) = make_uint4(q[4], q[5], q[6], q[7]);
 #pragma unroll
-            for (int k = 0; k < MLP_IN; ++k) tc_put(TB, 64 + k, t, 128, v[k]);
+            for (int k = 0; k < MLP_IN; ++k) tc_put(TB, 64 + k, tr, 128, v[k]);
         }
         // ---- forward: layer 1 (K = 16), bias + ReLU into H1 and H1^T
-        uint64_t m1 = 0, m2 = 0;
+        uint32_t m1 = 0, m2 = 0;  // this thread's 16 columns: pre-activation > 0
         if (!tt_mma(tmem, X, 16, tsm + TT_W1, 16, 1, id64, false, &bar, phase, &s_fail)) break;
-#pragma unroll
-        for (int c = 0; c < 64; c += 16) {
+        {
             float v[16];
-            tc_ld16(tmem + lanes + c, v);
-            uint32_t q[8];
+            tc_ld16(tmem + lanes + cb, v);
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                const float z = v[i] + b1[c + i];
-                m1 |= (uint64_t)(z > 0.f) << (c + i);
+                const float z = v[i] + b1[cb + i];
+                m1 |= (uint32_t)(z > 0.f) << i;
                 v[i] = fmaxf(z, 0.f);
-                tc_put(TB, c + i, t, 128, v[i]);
+                tc_put(TB, cb + i, tr, 128, v[i]);
             }
+            uint32_t q[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) q[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-            *reinterpret_cast<uint4 *>(H1 + tc_off(t, c, 64)) = make_uint4(q[0], q[1], q[2], q[3]);
-            *reinterpret_cast<uint4 *>(H1 + tc_off(t, c + 8, 64)) = make_uint4(q[4], q[5], q[6], q[7]);
+            *reinterpret_cast<uint4 *>(H1 + tc_off(tr, cb, 64)) = make_uint4(q[0], q[1], q[2], q[3]);
+            *reinterpret_cast<uint4 *>(H1 + tc_off(tr, cb + 8, 64)) = make_uint4(q[4], q[5], q[6], q[7]);
         }
         // ---- layer 2 (K = 64): H2 and H2^T
         if (!tt_mma(tmem + 64, H1, 64, tsm + TT_W2, 64, 4, id64, false, &bar, phase, &s_fail)) break;
-#pragma unroll
-        for (int c = 0; c < 64; c += 16) {
+        {
             float v[16];
-            tc_ld16(tmem + lanes + 64 + c, v);
-            uint32_t q[8];
+            tc_ld16(tmem + lanes + 64 + cb, v);
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                const float z = v[i] + b2[c + i];
-                m2 |= (uint64_t)(z > 0.f) << (c + i);
+                const float z = v[i] + b2[cb + i];
+                m2 |= (uint32_t)(z > 0.f) << i;
                 v[i] = fmaxf(z, 0.f);
-                tc_put(TH2, c + i, t, 128, v[i]);
+                tc_put(TH2, cb + i, tr, 128, v[i]);
             }
+            uint32_t q[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) q[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-            *reinterpret_cast<uint4 *>(H2 + tc_off(t, c, 64)) = make_uint4(q[0], q[1], q[2], q[3]);
-            *reinterpret_cast<uint4 *>(H2 + tc_off(t, c + 8, 64)) = make_uint4(q[4], q[5], q[6], q[7]);
+            *reinterpret_cast<uint4 *>(H2 + tc_off(tr, cb, 64)) = make_uint4(q[0], q[1], q[2], q[3]);
+            *reinterpret_cast<uint4 *>(H2 + tc_off(tr, cb + 8, 64)) = make_uint4(q[4], q[5], q[6], q[7]);
         }
         // ---- layer 3 (K = 64, N = 16): output error dY = (y - t) / n into dY and dY^T
         if (!tt_mma(tmem + 128, H2, 64, tsm + TT_W3, 64, 4, id16, false, &bar, phase, &s_fail)) break;
-        {
+        if (cb == 0) {
             float v[16];
             tc_ld16(tmem + lanes + 128, v);
             float dy[MLP_OUT] = {0.f, 0.f, 0.f};
             if (r < n) {
 #pragma unroll
                 for (int o = 0; o < MLP_OUT; ++o) {
-                    const float raw = target[3 * R + o] - feat[(int64_t)MLP_IN * R + 3 + o];  // dv - dv_prev
-                    const float tn = (raw - my[o]) / sy[o];
-                    const float e = (v[o] + b3[o]) - tn;
+                    const float e = (v[o] + b3[o]) - tn[o];
                     loss += (double)e * (double)e;
                     dy[o] = e * inv_n;
                 }
             }
-            *reinterpret_cast<uint4 *>(DY + tc_off(t, 0, 16)) =
+            *reinterpret_cast<uint4 *>(DY + tc_off(tr, 0, 16)) =
                 make_uint4(pack_bf16(dy[0], dy[1]), pack_bf16(dy[2], 0.f), 0u, 0u);
 #pragma unroll
             for (int o = 0; o < MLP_OUT; ++o) {
-                tc_put(TDY, o, t, 128, dy[o]);
+                tc_put(TDY, o, tr, 128, dy[o]);
                 const float s_ = tt_warp_sum(dy[o]);
-                if (lane == 0) sdb[warp][2 * MLP_HID + o] += s_;
+                if (lane == 0) sdb[rw][2 * MLP_HID + o] += s_;
             }
         }
         // ---- dH2 = dY W3 (K = 16): dZ2 = dH2 [Z2 > 0] into dZ2 and dZ2^T (TZ rows 0..63)
         if (!tt_mma(tmem, DY, 16, tsm + TT_W3T, 16, 1, id64, false, &bar, phase, &s_fail)) break;
-#pragma unroll
-        for (int c = 0; c < 64; c += 16) {
+        {
             float v[16];
-            tc_ld16(tmem + lanes + c, v);
-            uint32_t q[8];
+            tc_ld16(tmem + lanes + cb, v);
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                v[i] = ((m2 >> (c + i)) & 1u) ? v[i] : 0.f;
-                tc_put(TZ, c + i, t, 128, v[i]);
-                const float s_ = tt_warp_sum(v[i]);
-                if (lane == 0) sdb[warp][MLP_HID + c + i] += s_;
+                v[i] = ((m2 >> i) & 1u) ? v[i] : 0.f;
+                tc_put(TZ, cb + i, tr, 128, v[i]);
             }
+            uint32_t q[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) q[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-            *reinterpret_cast<uint4 *>(DZ2 + tc_off(t, c, 64)) = make_uint4(q[0], q[1], q[2], q[3]);
-            *reinterpret_cast<uint4 *>(DZ2 + tc_off(t, c + 8, 64)) = make_uint4(q[4], q[5], q[6], q[7]);
+            *reinterpret_cast<uint4 *>(DZ2 + tc_off(tr, cb, 64)) = make_uint4(q[0], q[1], q[2], q[3]);
+            *reinterpret_cast<uint4 *>(DZ2 + tc_off(tr, cb + 8, 64)) = make_uint4(q[4], q[5], q[6], q[7]);
+            int col;
+            const float s_ = tt_column_sums(v, lane, col);
+            if ((lane & 1) == 0) sdb[rw][MLP_HID + cb + col] += s_;
         }
         // ---- dH1 = dZ2 W2 (K = 64): dZ1 = dH1 [Z1 > 0] into dZ1^T (TZ rows 64..127)
         if (!tt_mma(tmem + 64, DZ2, 64, tsm + TT_W2T, 64, 4, id64, false, &bar, phase, &s_fail)) break;
-#pragma unroll
-        for (int c = 0; c < 64; c += 16) {
+        {
             float v[16];
-            tc_ld16(tmem + lanes + 64 + c, v);
+            tc_ld16(tmem + lanes + 64 + cb, v);
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                v[i] = ((m1 >> (c + i)) & 1u) ? v[i] : 0.f;
-                tc_put(TZ, 64 + c + i, t, 128, v[i]);
-                const float s_ = tt_warp_sum(v[i]);
-                if (lane == 0) sdb[warp][c + i] += s_;
+                v[i] = ((m1 >> i) & 1u) ? v[i] : 0.f;
+                tc_put(TZ, 64 + cb + i, tr, 128, v[i]);
             }
+            int col;
+            const float s_ = tt_column_sums(v, lane, col);
+            if ((lane & 1) == 0) sdb[rw][cb + col] += s_;
         }
         // ---- weight gradients over the tile's rows (K = 128), accumulated in tensor memory
         if (!tt_mma(tmem + TT_GW12, TZ, 128, TB, 128, 8, id80, !first, &bar, phase, &s_fail)) break;
@@ -481,7 +560,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1) mlp_train_kernel(int64_t n, con
     // ---- this CTA's partials: dW2 (rows 0..63, columns 0..63 of the first gradient),
     // dW1 (rows 64..127, columns 64..75), dW3^T (rows 0..63 of the second)
     float *out = part + (int64_t)blockIdx.x * PC_MLP_NPARAMS;
-    if (!s_fail) {
+    if (!s_fail && warp < 4) {
         if (warp < 2) {
             const int i = 32 * warp + lane;  // dW2 row (output unit) / dW3^T row (hidden unit)
 #pragma unroll
@@ -504,7 +583,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1) mlp_train_kernel(int64_t n, con
         }
     }
     for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-    if (lane == 0) sloss[warp] = loss;
+    if (lane == 0 && warp < 4) sloss[warp] = loss;
     // every tensor-memory read of this CTA is complete before the columns are released
     tc_fence_before();
     __syncthreads();
@@ -521,16 +600,31 @@ __global__ void __launch_bounds__(TT_THREADS, 1) mlp_train_kernel(int64_t n, con
     if (warp == 0) tc_dealloc(tmem, TT_TMEM_COLS);
 }
 
-// grad = sum of the CTA partials in CTA order (FP64 accumulation); with adam != 0 also the
-// Adam update of the FP32 master weights: m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
-// p -= lr (m / bc1) / (sqrt(v / bc2) + eps) with bc = 1 - beta^t.
-__global__ void mlp_reduce_adam_kernel(int nparts, const float *part, float *grad, int adam, float *params, float *m,
-                                       float *v, float lr, float beta1, float beta2, float eps, float bc1, float bc2)
+// grad = sum of the CTA partials (FP64 accumulation: RA_GROUPS runs of CTAs in order, then the
+// runs in order); with adam != 0 also the Adam update of the FP32 master weights:
+// m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2, p -= lr (m / bc1) / (sqrt(v / bc2) + eps) with
+// bc = 1 - beta^t. One thread per parameter summed 152 partials in one chain of loads and
+// FP64 additions, 28 us; the runs take warps of their own (each still reads 32 neighbouring
+// parameters).
+#define RA_GROUPS 16
+__global__ void __launch_bounds__(32 * RA_GROUPS) mlp_reduce_adam_kernel(int nparts, const float *part, float *grad,
+                                                                         int adam, float *params, float *m, float *v,
+                                                                         float lr, float beta1, float beta2, float eps,
+                                                                         float bc1, float bc2)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= PC_MLP_NPARAMS) return;
+    __shared__ double s_acc[RA_GROUPS][32];
+    const int lane = threadIdx.x & 31, group = threadIdx.x >> 5;
+    const int p = blockIdx.x * 32 + lane;
+    const int per = (nparts + RA_GROUPS - 1) / RA_GROUPS, c0 = min(group * per, nparts), c1 = min(c0 + per, nparts);
     double acc = 0.0;
-    for (int c = 0; c < nparts; ++c) acc += (double)part[(int64_t)c * PC_MLP_NPARAMS + p];
+    if (p < PC_MLP_NPARAMS) {
+#pragma unroll 10
+        for (int c = c0; c < c1; ++c) acc += (double)part[(int64_t)c * PC_MLP_NPARAMS + p];
+    }
+    s_acc[group][lane] = acc;
+    __syncthreads();
+    if (group != 0 || p >= PC_MLP_NPARAMS) return;
+    for (int g = 1; g < RA_GROUPS; ++g) acc += s_acc[g][lane];
     const float gr = (float)acc;
     if (grad) grad[p] = gr;
     if (adam) {
@@ -747,21 +841,26 @@ extern "C" pc_status pc_mlp_infer(int64_t n, const float *params, const float *s
     PC_CUDA_TRY(cudaGetDevice(&dev));
     PC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     PC_CUDA_TRY(cudaFuncSetAttribute(mlp_infer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES));
-    static thread_local uint32_t *d_err = nullptr;  // timeout flag of this host thread's launches
+    // this host thread's timeout flag: a word of host memory that only a kernel whose wait gave
+    // up writes, so a call needs no clearing and no copy, only the wait for its own launch
+    static thread_local uint32_t *h_err = nullptr, *d_err = nullptr;
     static thread_local int err_dev = -1;
-    if (!d_err || err_dev != dev) {
-        PC_CUDA_TRY(cudaMalloc(&d_err, sizeof(uint32_t)));
+    if (!h_err) {
+        PC_CUDA_TRY(cudaHostAlloc(&h_err, sizeof(uint32_t), cudaHostAllocMapped | cudaHostAllocPortable));
+        *h_err = 0;
+    }
+    if (err_dev != dev) {
+        PC_CUDA_TRY(cudaHostGetDevicePointer(&d_err, h_err, 0));
         err_dev = dev;
     }
-    PC_CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(uint32_t), st));
     const int64_t tiles = (n + TC_ROWS - 1) / TC_ROWS;
-    const int grid = (int)std::min<int64_t>(tiles, 2ll * sms);
+    const int grid = (int)std::min<int64_t>(tiles, (int64_t)TC_CTAS_PER_SM * sms);
     MLP_LAUNCH(mlp_infer_kernel, grid, TC_THREADS, TC_SMEM_BYTES, st, n, params, stats, feat, dv_prev, fixed, dv0,
                d_err);
-    uint32_t h_err = 0;
-    PC_CUDA_TRY(cudaMemcpyAsync(&h_err, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     PC_CUDA_TRY(cudaStreamSynchronize(st));
-    return h_err ? PC_ERR_TIMEOUT : PC_OK;
+    if (*(volatile uint32_t *)h_err == 0) return PC_OK;
+    *h_err = 0;
+    return PC_ERR_TIMEOUT;
 }
 
 static pc_status mlp_grad_impl(pc_mlp *M, int64_t n, const int32_t *rows, const float *params, const float *stats,
@@ -784,7 +883,7 @@ static pc_status mlp_grad_impl(pc_mlp *M, int64_t n, const int32_t *rows, const 
         bc1 = (float)(1.0 - pow((double)b1, (double)M->t));
         bc2 = (float)(1.0 - pow((double)b2, (double)M->t));
     }
-    MLP_LAUNCH(mlp_reduce_adam_kernel, (PC_MLP_NPARAMS + 255) / 256, 256, 0, st, grid, M->part, grad, adam ? 1 : 0,
+    MLP_LAUNCH(mlp_reduce_adam_kernel, (PC_MLP_NPARAMS + 31) / 32, 32 * RA_GROUPS, 0, st, grid, M->part, grad, adam ? 1 : 0,
                (float *)params, M->m, M->v, lr, b1, b2, eps, bc1, bc2);
     if (loss) {
         MLP_LAUNCH(mlp_loss_sum_kernel, 1, 32, 0, st, grid, M->loss_part, M->loss);
@@ -827,7 +926,7 @@ extern "C" pc_status pc_mlp_adam_apply(pc_mlp *M, float *params, const float *gr
     M->t += 1;
     const float bc1 = (float)(1.0 - pow((double)o->beta1, (double)M->t));
     const float bc2 = (float)(1.0 - pow((double)o->beta2, (double)M->t));
-    MLP_LAUNCH(mlp_reduce_adam_kernel, (PC_MLP_NPARAMS + 255) / 256, 256, 0, st, 1, M->part, (float *)nullptr, 1,
+    MLP_LAUNCH(mlp_reduce_adam_kernel, (PC_MLP_NPARAMS + 31) / 32, 32 * RA_GROUPS, 0, st, 1, M->part, (float *)nullptr, 1,
                params, M->m, M->v, o->lr, o->beta1, o->beta2, o->eps, bc1, bc2);
     return PC_OK;
 }
