@@ -187,7 +187,11 @@ struct pc_ctx {
     uint32_t *px_vals = nullptr;
     int32_t *px_cnt = nullptr, *px_off = nullptr;    // [T+1]
     int32_t *px_vcnt = nullptr, *px_voff = nullptr;  // [V+1]
-    uint32_t *px_max = nullptr;
+    uint32_t *px_max = nullptr;                      // [7] extent of the boxes
+    float4 *px_box = nullptr;                        // [T][2] grown boxes
+    uint32_t *px_hits = nullptr;                     // [PX_HITS][V]
+    int64_t px_first_cap = 0;                        // cells the table holds
+    int32_t *px_first = nullptr;                     // [px_first_cap + 1]
 
     // context-owned step system
     int32_t *A_rp = nullptr, *A_ci = nullptr;

@@ -7,12 +7,19 @@
 //
 // Uniform grid, rebuilt per call: the cell size is the largest triangle bounding box
 // grown by delta (so every grown box covers at most 2 x 2 x 2 cells); each triangle is
-// listed under every cell its grown box overlaps (key = packed cell coordinates), the
-// list is put in key order by the stable radix sort (triangles of a cell stay in index
-// order), and each vertex tests the triangles listed under its own cell: a vertex within
-// delta of a triangle lies in that triangle's grown box, hence in one of its cells. Two
-// passes over the vertices (count, scan, write) give the pairs ordered by vertex, then
-// by triangle, without atomics.
+// listed under every cell its grown box overlaps, the list is put in cell order by the
+// stable radix sort (triangles of a cell stay in index order), and each vertex tests the
+// triangles listed under its own cell: a vertex within delta of a triangle lies in that
+// triangle's grown box, hence in one of its cells. A pass over the vertices counts each
+// one's pairs and remembers the first PX_HITS of them, a scan gives their places, and a
+// second pass writes them: ordered by vertex, then by triangle, without atomics.
+//
+// Cells are numbered inside the boxes' own extent, so that the sort needs the bits of that
+// many cells (17 for three 301 x 301 sheets: 3 passes) and not of 3 packed 21-bit
+// coordinates (8 passes, 400 of the query's 1,130 us), and a vertex finds its cell's list
+// in a table instead of by binary search. A vertex meets about 55 triangles in its cell;
+// the grown box of each (32 bytes, kept per triangle) rejects most before the ring and the
+// distance are looked at, and only the first pass looks (both did: 320 us each).
 //
 // The region of the closest point (Voronoi classification of a point against a
 // triangle, Ericson 2005, Sec. 5.1.5) and the test d^2 < delta^2 are decided in FP32
@@ -24,6 +31,13 @@
 
 #define PX_CELLS_PER_TRI 8
 #define PX_COORD_BIAS (1 << 20)  // cell coordinates must lie in [-2^20, 2^20)
+#define PX_HITS 16               // pairs of a vertex remembered from the counting pass
+
+// The numbered cells: first coordinates, extents (nx, ny), and how many there are.
+struct PxGrid {
+    int x0, y0, z0;
+    int64_t nx, ny, n;
+};
 
 __device__ __forceinline__ float3 px_ld(const float *x, int i)
 {
@@ -91,28 +105,63 @@ __device__ __forceinline__ bool px_cell(float v, float inv, int &i)
     i = (int)f;
     return true;
 }
-__device__ __forceinline__ uint64_t px_key(int ix, int iy, int iz)
+// Number of the cell at (ix, iy, iz), at least 0; -1 outside the numbered extent.
+__device__ __forceinline__ int64_t px_number(const PxGrid &g, int ix, int iy, int iz)
 {
-    return ((uint64_t)(ix + PX_COORD_BIAS) << 42) | ((uint64_t)(iy + PX_COORD_BIAS) << 21) |
-           (uint64_t)(iz + PX_COORD_BIAS);
+    const int64_t x = (int64_t)ix - g.x0, y = (int64_t)iy - g.y0, z = (int64_t)iz - g.z0;
+    if (x < 0 || y < 0 || z < 0 || x >= g.nx || y >= g.ny) return -1;
+    const int64_t c = (z * g.ny + y) * g.nx + x;
+    return c < g.n ? c : -1;
 }
 
-// Largest edge of the grown boxes (non-negative floats order like their bit patterns).
-__global__ void px_extent_kernel(int T, const float *x, const int32_t *tri, float pad, uint32_t *max_bits)
+// A float as an unsigned integer of the same order, and back (host side).
+__device__ __forceinline__ uint32_t px_ordered(float f)
 {
-    float m = 0.f;
+    const uint32_t u = __float_as_uint(f);
+    return (u & 0x80000000u) ? ~u : u | 0x80000000u;
+}
+static float px_from_ordered(uint32_t u)
+{
+    u = (u & 0x80000000u) ? u & 0x7fffffffu : ~u;
+    float f;
+    memcpy(&f, &u, sizeof(f));
+    return f;
+}
+
+// Extent of the grown boxes: ext[0] the largest edge, ext[1..3] the complement of the lowest
+// corner, ext[4..6] the highest corner (ordered integers; all maxima, from zero).
+__global__ void __launch_bounds__(256) px_extent_kernel(int T, const float *x, const int32_t *tri, float pad, uint32_t *ext)
+{
+    __shared__ uint32_t s_m[7][8];
+    uint32_t m[7] = {0u, 0u, 0u, 0u, 0u, 0u, 0u};
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x) {
         float3 lo, hi;
         px_box(x, tri, t, pad, lo, hi);
-        m = fmaxf(m, fmaxf(fmaxf(hi.x - lo.x, hi.y - lo.y), hi.z - lo.z));
+        const float e = fmaxf(fmaxf(hi.x - lo.x, hi.y - lo.y), hi.z - lo.z);
+        if (e > 0.f) m[0] = max(m[0], __float_as_uint(e));
+        m[1] = max(m[1], ~px_ordered(lo.x));
+        m[2] = max(m[2], ~px_ordered(lo.y));
+        m[3] = max(m[3], ~px_ordered(lo.z));
+        m[4] = max(m[4], px_ordered(hi.x));
+        m[5] = max(m[5], px_ordered(hi.y));
+        m[6] = max(m[6], px_ordered(hi.z));
     }
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(max_bits, __float_as_uint(m));
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+        m[k] = __reduce_max_sync(0xffffffffu, m[k]);
+        if ((threadIdx.x & 31) == 0) s_m[k][threadIdx.x >> 5] = m[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 7) {
+        uint32_t v = 0u;
+        for (int w = 0; w < 8; ++w) v = max(v, s_m[threadIdx.x][w]);
+        atomicMax(ext + threadIdx.x, v);
+    }
 }
 
 // Cells per triangle (0 and an error bit when a box leaves the grid).
 __global__ void px_count_cells_kernel(int T, const float *x, const int32_t *tri, float pad, float inv,
-                                      int32_t *cnt, uint32_t *err)
+                                      int32_t *cnt, float4 *box, uint32_t *err)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t > T) return;
@@ -122,6 +171,8 @@ __global__ void px_count_cells_kernel(int T, const float *x, const int32_t *tri,
     }
     float3 lo, hi;
     px_box(x, tri, t, pad, lo, hi);
+    box[2ll * t] = make_float4(lo.x, lo.y, lo.z, hi.x);
+    box[2ll * t + 1] = make_float4(hi.y, hi.z, 0.f, 0.f);
     int i0, i1, j0, j1, k0, k1;
     if (!(px_cell(lo.x, inv, i0) && px_cell(hi.x, inv, i1) && px_cell(lo.y, inv, j0) && px_cell(hi.y, inv, j1) &&
           px_cell(lo.z, inv, k0) && px_cell(hi.z, inv, k1))) {
@@ -132,27 +183,35 @@ __global__ void px_count_cells_kernel(int T, const float *x, const int32_t *tri,
     cnt[t] = (i1 - i0 + 1) * (j1 - j0 + 1) * (k1 - k0 + 1);
 }
 
-__global__ void px_emit_cells_kernel(int T, const float *x, const int32_t *tri, float pad, float inv,
-                                     const int32_t *off, int64_t cap, uint64_t *keys, uint32_t *vals)
+__global__ void px_emit_cells_kernel(int T, const float4 *__restrict__ box, float inv, PxGrid g, const int32_t *off,
+                                     int64_t cap, uint64_t *keys, uint32_t *vals)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
-    float3 lo, hi;
-    px_box(x, tri, t, pad, lo, hi);
+    const float4 p = box[2ll * t], q = box[2ll * t + 1];
     int i0, i1, j0, j1, k0, k1;
-    if (!(px_cell(lo.x, inv, i0) && px_cell(hi.x, inv, i1) && px_cell(lo.y, inv, j0) && px_cell(hi.y, inv, j1) &&
-          px_cell(lo.z, inv, k0) && px_cell(hi.z, inv, k1)))
+    if (!(px_cell(p.x, inv, i0) && px_cell(p.w, inv, i1) && px_cell(p.y, inv, j0) && px_cell(q.x, inv, j1) &&
+          px_cell(p.z, inv, k0) && px_cell(q.y, inv, k1)))
         return;
     int64_t o = off[t];
     for (int k = k0; k <= k1; ++k)
         for (int j = j0; j <= j1; ++j)
             for (int i = i0; i <= i1; ++i) {
                 if (o < cap) {
-                    keys[o] = px_key(i, j, k);
+                    keys[o] = (uint64_t)px_number(g, i, j, k);
                     vals[o] = (uint32_t)t;
                 }
                 ++o;
             }
+}
+
+// first[c]: where cell c's list begins (c = 0 .. n), from the sorted keys.
+__global__ void px_first_kernel(int64_t K, const uint64_t *__restrict__ keys, int64_t n, int32_t *first)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i > K) return;
+    const int64_t b = i == 0 ? 0 : (int64_t)keys[i - 1] + 1, e = i == K ? n : (int64_t)keys[i];
+    for (int64_t c = b; c <= e; ++c) first[c] = (int32_t)i;
 }
 
 // true when v is among ecol[lo .. hi) (sorted)
@@ -167,58 +226,127 @@ __device__ __forceinline__ bool px_ring_has(const int32_t *ecol, int lo, int hi,
     return lo < end && ecol[lo] == v;
 }
 
-// One thread per vertex: the triangles listed under its cell. COUNT: cnt[p] = pairs of p;
-// WRITE: the pairs at off[p] ...
+struct PxArgs {
+    int V;
+    const float *x;
+    const int32_t *tri;
+    const float4 *box;
+    const uint64_t *keys;
+    const uint32_t *vals;
+    int64_t K;
+    const int32_t *first;  // null: more cells than the table holds
+    PxGrid g;
+    float inv, delta;
+    const int32_t *erp, *ecol;
+    int32_t *cnt;          // [V + 1] pairs of each vertex
+    uint32_t *hits;        // [PX_HITS][V] their first triangles
+    const int32_t *off;
+    int32_t *pairs;
+    float *w;
+    uint32_t *err;
+};
+
+// Where the list of cell `c` begins (and, with the table, ends).
+__device__ __forceinline__ void px_list(const PxArgs &a, int64_t c, int64_t &lo, int64_t &hi)
+{
+    lo = 0;
+    hi = 0;
+    if (c < 0) return;
+    if (a.first) {
+        lo = a.first[c];
+        hi = a.first[c + 1];
+        return;
+    }
+    int64_t h = a.K;
+    while (lo < h) {
+        const int64_t mid = (lo + h) >> 1;
+        if (a.keys[mid] < (uint64_t)c) lo = mid + 1;
+        else h = mid;
+    }
+    for (hi = lo; hi < a.K && a.keys[hi] == (uint64_t)c;) ++hi;
+}
+
+// Whether (p, t) is a pair, with the closest point's weights.
+__device__ __forceinline__ bool px_pair(const PxArgs &a, int p, float3 xp, int t, int r0, int r1, float d2max, int &ia,
+                                        int &ib, int &ic, float &wa, float &wb, float &wc)
+{
+    ia = a.tri[3ll * t];
+    ib = a.tri[3ll * t + 1];
+    ic = a.tri[3ll * t + 2];
+    if (ia == p || ib == p || ic == p) return false;
+    if (px_ring_has(a.ecol, r0, r1, ia) || px_ring_has(a.ecol, r0, r1, ib) || px_ring_has(a.ecol, r0, r1, ic))
+        return false;
+    return px_closest(xp, px_ld(a.x, ia), px_ld(a.x, ib), px_ld(a.x, ic), wa, wb, wc) < d2max;
+}
+
+// One thread per vertex: the triangles listed under its cell whose grown box holds it. COUNT:
+// cnt[p] = pairs of p, the first PX_HITS in hits; WRITE: the pairs at off[p] ..., from hits
+// unless there are more.
 template <bool WRITE>
-__global__ void px_pairs_kernel(int V, const float *x, const int32_t *tri, const uint64_t *keys, const uint32_t *vals,
-                                int64_t K, float inv, float delta, const int32_t *erp, const int32_t *ecol,
-                                int32_t *cnt, const int32_t *off, int32_t *pairs, float *w, uint32_t *err)
+__global__ void __launch_bounds__(128) px_pairs_kernel(PxArgs a)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > V) return;
-    if (p == V) {
-        if (!WRITE) cnt[V] = 0;
+    if (p > a.V) return;
+    if (p == a.V) {
+        if (!WRITE) a.cnt[a.V] = 0;
         return;
     }
-    const float3 xp = px_ld(x, p);
-    int ix, iy, iz;
-    if (!(px_cell(xp.x, inv, ix) && px_cell(xp.y, inv, iy) && px_cell(xp.z, inv, iz))) {
-        if (!WRITE) cnt[p] = 0;
-        pc_set_err(err, PC_DERR_INDEX);
-        return;
-    }
-    const uint64_t key = px_key(ix, iy, iz);
-    int64_t lo = 0, hi = K;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (keys[mid] < key) lo = mid + 1;
-        else hi = mid;
-    }
-    const float d2max = __fmul_rn(delta, delta);
-    const int r0 = erp[p], r1 = erp[p + 1];
+    const int have = WRITE ? a.cnt[p] : 0;
+    if (WRITE && have == 0) return;
+    const float3 xp = px_ld(a.x, p);
+    const float d2max = __fmul_rn(a.delta, a.delta);
+    const int r0 = a.erp[p], r1 = a.erp[p + 1];
+    int ia, ib, ic;
+    float wa, wb, wc;
     int n = 0;
-    const int64_t o0 = WRITE ? off[p] : 0;
-    for (int64_t i = lo; i < K && keys[i] == key; ++i) {
-        const int t = (int)vals[i];
-        const int a = tri[3ll * t], b = tri[3ll * t + 1], c = tri[3ll * t + 2];
-        if (a == p || b == p || c == p) continue;
-        if (px_ring_has(ecol, r0, r1, a) || px_ring_has(ecol, r0, r1, b) || px_ring_has(ecol, r0, r1, c)) continue;
-        float wa, wb, wc;
-        const float d2 = px_closest(xp, px_ld(x, a), px_ld(x, b), px_ld(x, c), wa, wb, wc);
-        if (!(d2 < d2max)) continue;
-        if (WRITE) {
-            const int64_t o = o0 + n;
-            pairs[4 * o] = p;
-            pairs[4 * o + 1] = a;
-            pairs[4 * o + 2] = b;
-            pairs[4 * o + 3] = c;
-            w[3 * o] = wa;
-            w[3 * o + 1] = wb;
-            w[3 * o + 2] = wc;
+    auto put = [&](int64_t o) {
+        a.pairs[4 * o] = p;
+        a.pairs[4 * o + 1] = ia;
+        a.pairs[4 * o + 2] = ib;
+        a.pairs[4 * o + 3] = ic;
+        a.w[3 * o] = wa;
+        a.w[3 * o + 1] = wb;
+        a.w[3 * o + 2] = wc;
+    };
+    if (WRITE && have <= PX_HITS) {
+        for (; n < have; ++n) {
+            px_pair(a, p, xp, (int)a.hits[(int64_t)n * a.V + p], r0, r1, d2max, ia, ib, ic, wa, wb, wc);
+            put((int64_t)a.off[p] + n);
         }
+        return;
+    }
+    int ix, iy, iz;
+    if (!(px_cell(xp.x, a.inv, ix) && px_cell(xp.y, a.inv, iy) && px_cell(xp.z, a.inv, iz))) {
+        if (!WRITE) a.cnt[p] = 0;
+        pc_set_err(a.err, PC_DERR_INDEX);
+        return;
+    }
+    // the box already exceeds delta by a hundredth; this far outside it, no rounding of the
+    // coordinates (16 units in their last place) can bring the computed distance below delta
+    const float slack = 0.05f * a.delta + 1e-6f * (fabsf(xp.x) + fabsf(xp.y) + fabsf(xp.z));
+    int64_t lo, hi;
+    px_list(a, px_number(a.g, ix, iy, iz), lo, hi);
+    for (int64_t i = lo; i < hi; ++i) {
+        const int t = (int)a.vals[i];
+        const float4 b0 = a.box[2ll * t], b1 = a.box[2ll * t + 1];
+        if (xp.x < b0.x - slack || xp.y < b0.y - slack || xp.z < b0.z - slack || xp.x > b0.w + slack ||
+            xp.y > b1.x + slack || xp.z > b1.y + slack)
+            continue;
+        if (!px_pair(a, p, xp, t, r0, r1, d2max, ia, ib, ic, wa, wb, wc)) continue;
+        if (WRITE) put((int64_t)a.off[p] + n);
+        else if (n < PX_HITS) a.hits[(int64_t)n * a.V + p] = (uint32_t)t;
         ++n;
     }
-    if (!WRITE) cnt[p] = n;
+    if (!WRITE) a.cnt[p] = n;
+}
+
+// The coordinate of the cell that holds v, as the kernels compute it (host side).
+static bool px_host_cell(float v, float inv, int *i)
+{
+    const float f = floorf(v * inv);
+    if (!(f >= -(float)PX_COORD_BIAS && f < (float)PX_COORD_BIAS)) return false;
+    *i = (int)f;
+    return true;
 }
 
 extern "C" pc_status pc_proximity_query(pc_ctx *ctx, const float *x, float delta, int32_t cap, int32_t *pairs,
@@ -233,23 +361,31 @@ extern "C" pc_status pc_proximity_query(pc_ctx *ctx, const float *x, float delta
     if (!ctx->px_keys) return PC_ERR_ARG;
     const float pad = delta * 1.01f;
     // cell size: the largest grown box (at least delta)
-    PC_CUDA_TRY(cudaMemsetAsync(ctx->px_max, 0, sizeof(uint32_t), st));
+    PC_CUDA_TRY(cudaMemsetAsync(ctx->px_max, 0, 7 * sizeof(uint32_t), st));
     const unsigned ext_grid = pc_blocks(T, 256) < (unsigned)(ctx->num_sms * 8) ? pc_blocks(T, 256) : ctx->num_sms * 8;
     PC_LAUNCH(ctx, px_extent_kernel, ext_grid, 256, 0, st, T, x, ctx->tri, pad, ctx->px_max);
-    PC_CUDA_TRY(cudaMemcpyAsync(ctx->h_count, ctx->px_max, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+    PC_CUDA_TRY(cudaMemcpyAsync(ctx->h_count, ctx->px_max, 7 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     PC_CUDA_TRY(cudaStreamSynchronize(st));
-    uint32_t bits_ext = *reinterpret_cast<uint32_t *>(ctx->h_count);
+    uint32_t ext[7];
+    memcpy(ext, ctx->h_count, sizeof(ext));
+    const uint32_t bits_ext = ext[0];
+    float corner[6];
+    for (int k = 0; k < 3; ++k) {
+        corner[k] = px_from_ordered(~ext[1 + k]);
+        corner[3 + k] = px_from_ordered(ext[4 + k]);
+    }
     float cs;
     memcpy(&cs, &bits_ext, sizeof(float));
     if (!(cs < 1e30f)) return PC_ERR_NONFINITE;
     cs = fmaxf(cs, delta) * 1.001f;
     const int64_t cap_k = ctx->px_cap;
     int64_t K = 0;
+    PxGrid g{};
     for (int attempt = 0;; ++attempt) {
         const float inv = 1.0f / cs;
         PC_CUDA_TRY(cudaMemsetAsync(ctx->d_err, 0, sizeof(uint32_t), st));
         PC_LAUNCH(ctx, px_count_cells_kernel, pc_blocks(T + 1ll, 256), 256, 0, st, T, x, ctx->tri, pad, inv,
-                  ctx->px_cnt, ctx->d_err);
+                  ctx->px_cnt, ctx->px_box, ctx->d_err);
         PC_TRY(pc_exclusive_scan(ctx, ctx->px_cnt, ctx->px_off, T, st));
         PC_CUDA_TRY(cudaMemcpyAsync(ctx->h_count, ctx->px_off + T, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         uint32_t bits = 0;
@@ -257,17 +393,48 @@ extern "C" pc_status pc_proximity_query(pc_ctx *ctx, const float *x, float delta
         if (bits) return PC_ERR_ARG;  // positions too far out for the cell grid
         K = *reinterpret_cast<int32_t *>(ctx->h_count);
         if (K <= cap_k) {
-            PC_LAUNCH(ctx, px_emit_cells_kernel, pc_blocks(T, 256), 256, 0, st, T, x, ctx->tri, pad, inv,
-                      ctx->px_off, cap_k, ctx->px_keys, ctx->px_vals);
-            PC_TRY(pc_radix_sort(ctx, ctx->px_keys, ctx->px_vals, K, 63, st));
+            int c[6];
+            for (int k = 0; k < 6; ++k)
+                if (!px_host_cell(corner[k], inv, c + k)) return PC_ERR_ARG;
+            g.x0 = c[0];
+            g.y0 = c[1];
+            g.z0 = c[2];
+            g.nx = (int64_t)c[3] - c[0] + 1;  // each extent at most 2^21: 63 bits for their product
+            g.ny = (int64_t)c[4] - c[1] + 1;
+            g.n = g.nx * g.ny * ((int64_t)c[5] - c[2] + 1);
+            PC_LAUNCH(ctx, px_emit_cells_kernel, pc_blocks(T, 256), 256, 0, st, T, ctx->px_box, inv, g, ctx->px_off,
+                      cap_k, ctx->px_keys, ctx->px_vals);
+            PC_TRY(pc_radix_sort(ctx, ctx->px_keys, ctx->px_vals, K, pc_bits_for(g.n), st));
             break;
         }
         if (attempt >= 4) return PC_ERR_CAPACITY;
         cs *= 2.0f;  // rounding put some boxes across three cells: coarser grid
     }
-    const float inv = 1.0f / cs;
-    PC_LAUNCH(ctx, px_pairs_kernel<false>, pc_blocks(V + 1ll, 128), 128, 0, st, V, x, ctx->tri, ctx->px_keys,
-              ctx->px_vals, K, inv, delta, ctx->erp, ctx->ecol, ctx->px_vcnt, nullptr, nullptr, nullptr, ctx->d_err);
+    PxArgs a{};
+    a.V = V;
+    a.x = x;
+    a.tri = ctx->tri;
+    a.box = ctx->px_box;
+    a.keys = ctx->px_keys;
+    a.vals = ctx->px_vals;
+    a.K = K;
+    // a list of its own for every cell where the table has room (sheets do: a few triangles
+    // per cell), else binary searches in the sorted keys
+    a.first = g.n <= ctx->px_first_cap ? ctx->px_first : nullptr;
+    a.g = g;
+    a.inv = 1.0f / cs;
+    a.delta = delta;
+    a.erp = ctx->erp;
+    a.ecol = ctx->ecol;
+    a.cnt = ctx->px_vcnt;
+    a.hits = ctx->px_hits;
+    a.off = ctx->px_voff;
+    a.pairs = pairs;
+    a.w = w;
+    a.err = ctx->d_err;
+    if (a.first)
+        PC_LAUNCH(ctx, px_first_kernel, pc_blocks(K + 1, 256), 256, 0, st, K, ctx->px_keys, g.n, ctx->px_first);
+    PC_LAUNCH(ctx, px_pairs_kernel<false>, pc_blocks(V + 1ll, 128), 128, 0, st, a);
     PC_TRY(pc_exclusive_scan(ctx, ctx->px_vcnt, ctx->px_voff, V, st));
     PC_CUDA_TRY(cudaMemcpyAsync(ctx->h_count, ctx->px_voff + V, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     uint32_t bits = 0;
@@ -277,14 +444,13 @@ extern "C" pc_status pc_proximity_query(pc_ctx *ctx, const float *x, float delta
     *n_out = P;
     if (P > cap) return PC_ERR_CAPACITY;
     if (P > 0)
-        PC_LAUNCH(ctx, px_pairs_kernel<true>, pc_blocks(V + 1ll, 128), 128, 0, st, V, x, ctx->tri, ctx->px_keys,
-                  ctx->px_vals, K, inv, delta, ctx->erp, ctx->ecol, nullptr, ctx->px_voff, pairs, w, ctx->d_err);
+        PC_LAUNCH(ctx, px_pairs_kernel<true>, pc_blocks(V + 1ll, 128), 128, 0, st, a);
     PC_CUDA_TRY(cudaStreamSynchronize(st));
     return PC_OK;
 }
 
-// Query buffers (called at context creation): 8 cell entries per triangle, per-triangle
-// and per-vertex counts and offsets.
+// Query buffers (called at context creation): 8 cell entries and a box per triangle, a table
+// of two cells per triangle, per-triangle and per-vertex counts and offsets, remembered pairs.
 pc_status pc_proximity_alloc(pc_ctx *c)
 {
     c->px_cap = (int64_t)PX_CELLS_PER_TRI * c->T + 1;
@@ -294,6 +460,10 @@ pc_status pc_proximity_alloc(pc_ctx *c)
     PC_CUDA_TRY(cudaMalloc(&c->px_off, sizeof(int32_t) * (c->T + 1ll)));
     PC_CUDA_TRY(cudaMalloc(&c->px_vcnt, sizeof(int32_t) * (c->V + 1ll)));
     PC_CUDA_TRY(cudaMalloc(&c->px_voff, sizeof(int32_t) * (c->V + 1ll)));
-    PC_CUDA_TRY(cudaMalloc(&c->px_max, sizeof(uint32_t)));
+    PC_CUDA_TRY(cudaMalloc(&c->px_max, 7 * sizeof(uint32_t)));
+    PC_CUDA_TRY(cudaMalloc(&c->px_box, sizeof(float4) * 2 * (size_t)(c->T > 0 ? c->T : 1)));
+    PC_CUDA_TRY(cudaMalloc(&c->px_hits, sizeof(uint32_t) * PX_HITS * (size_t)c->V));
+    c->px_first_cap = 2ll * c->T + 4096;
+    PC_CUDA_TRY(cudaMalloc(&c->px_first, sizeof(int32_t) * (size_t)(c->px_first_cap + 1)));
     return PC_OK;
 }
