@@ -111,8 +111,10 @@ __device__ __forceinline__ void strain_from_edges(const dfl *e1, const dfl *e2, 
 //   c (mu Fg_l Fg_k^T + lam Fg_k Fg_l^T + mu (g_k.g_l) F F^T + (g_k.S+ g_l) I),
 // so the record holds those factors (32 floats: one 128-byte line) instead of the six
 // upper blocks (54 floats), and the rows expand the block they need (tri_block below).
-// Record, as eight float4: (c_0, c mu) (c_1, s11) (c_2, s12) (Fg_1, s22) (Fg_2, gg00)
-// (M00 M01 M02 gg01) (M11 M12 M22 gg02) (gg11 gg12 gg22 -), M = c mu F F^T, s = c g.S+ g.
+// Record, as eight float4: (c_0, c mu) (c_1, saa) (c_2, sab) (Fg_a, sbb) (Fg_b, gg00)
+// (M00 M01 M02 gg01) (M11 M12 M22 gg02) (gg11 gg12 gg22 m), M = c mu F F^T, s = c g.S+ g.
+// m is the vertex with the longest gradient and a < b are the other two: the gradients sum to
+// zero, and the longest follows from the others without cancellation.
 // c_k = h f_k - sum_l (h^2 H_kl) v_l is the element's share of b = h (f - h K v), the
 // first-order form of h f(x_t + h v_t) (Eq. 2-3); since each Hessian row sums to zero,
 // sum_l H_kl v_l is formed as sum_l H_kl (v_l - v_k).
@@ -241,26 +243,27 @@ __global__ void __launch_bounds__(TE_THREADS) tri_eval_kernel(int T, const int32
                     }
             }
         float *o = s_rec[threadIdx.x];
+        const int m = R.gg[0] >= R.gg[3] && R.gg[0] >= R.gg[5] ? 0 : R.gg[3] >= R.gg[5] ? 1 : 2;
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
             for (int a = 0; a < 3; ++a) o[4 * k + a] = ck[k][a];
         o[3] = R.cm;
-        o[7] = R.s[3];
-        o[11] = R.s[4];
+        o[7] = m == 0 ? R.s[3] : R.s[0];
+        o[11] = m == 0 ? R.s[4] : m == 1 ? R.s[2] : R.s[1];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            o[12 + a] = R.Fg[1][a];
-            o[16 + a] = R.Fg[2][a];
+            o[12 + a] = m == 0 ? R.Fg[1][a] : R.Fg[0][a];
+            o[16 + a] = m == 2 ? R.Fg[1][a] : R.Fg[2][a];
             o[20 + a] = R.M[a];
             o[24 + a] = R.M[3 + a];
             o[28 + a] = R.gg[3 + a];
         }
-        o[15] = R.s[5];
+        o[15] = m == 2 ? R.s[3] : R.s[5];
         o[19] = R.gg[0];
         o[23] = R.gg[1];
         o[27] = R.gg[2];
-        o[31] = 0.f;
+        o[31] = __int_as_float(m);
     }
     __syncthreads();
     const int n = min(TE_THREADS, T - (int)blockIdx.x * TE_THREADS) * PC_TRI_STRIDE;
@@ -272,24 +275,32 @@ __global__ void __launch_bounds__(TE_THREADS) tri_eval_kernel(int T, const int32
 __device__ __forceinline__ TriFactors tri_load(const float *__restrict__ buf, uint32_t id, float cl_cm)
 {
     const float4 *r = reinterpret_cast<const float4 *>(buf) + (int64_t)(PC_TRI_STRIDE / 4) * id;
-    const float cm = reinterpret_cast<const float *>(r)[3], s11 = reinterpret_cast<const float *>(r)[7],
-                s12 = reinterpret_cast<const float *>(r)[11];
-    const float4 f1 = r[3], f2 = r[4], m0 = r[5], m1 = r[6], q = r[7];
+    const float cm = reinterpret_cast<const float *>(r)[3], saa = reinterpret_cast<const float *>(r)[7],
+                sab = reinterpret_cast<const float *>(r)[11];
+    const float4 fa = r[3], fb = r[4], m0 = r[5], m1 = r[6], q = r[7];
+    const int m = __float_as_int(q.w);
+    const float Fa[3] = {fa.x, fa.y, fa.z}, Fb[3] = {fb.x, fb.y, fb.z}, sbb = fa.w;
     TriFactors R;
     R.cm = cm;
     R.cl = cl_cm * cm;
-    R.Fg[1][0] = f1.x; R.Fg[1][1] = f1.y; R.Fg[1][2] = f1.z;
-    R.Fg[2][0] = f2.x; R.Fg[2][1] = f2.y; R.Fg[2][2] = f2.z;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) R.Fg[0][a] = -(R.Fg[1][a] + R.Fg[2][a]);
+    for (int e = 0; e < 3; ++e) {
+        const float Fm = -(Fa[e] + Fb[e]);
+        R.Fg[0][e] = m == 0 ? Fm : Fa[e];
+        R.Fg[1][e] = m == 0 ? Fa[e] : m == 1 ? Fm : Fb[e];
+        R.Fg[2][e] = m == 2 ? Fm : Fb[e];
+    }
     R.M[0] = m0.x; R.M[1] = m0.y; R.M[2] = m0.z;
     R.M[3] = m1.x; R.M[4] = m1.y; R.M[5] = m1.z;
-    R.gg[0] = f2.w; R.gg[1] = m0.w; R.gg[2] = m1.w;
+    R.gg[0] = fb.w; R.gg[1] = m0.w; R.gg[2] = m1.w;
     R.gg[3] = q.x; R.gg[4] = q.y; R.gg[5] = q.z;
-    R.s[3] = s11; R.s[4] = s12; R.s[5] = f1.w;
-    R.s[1] = -(s11 + s12);
-    R.s[2] = -(s12 + f1.w);
-    R.s[0] = -(R.s[1] + R.s[2]);
+    const float sam = -(saa + sab), sbm = -(sab + sbb), smm = -(sam + sbm);
+    R.s[0] = m == 0 ? smm : saa;
+    R.s[1] = m == 2 ? sab : sam;                       // (0, 1): m, a | a, m | a, b
+    R.s[2] = m == 1 ? sab : m == 0 ? sbm : sam;        // (0, 2): m, b | a, b | a, m
+    R.s[3] = m == 0 ? saa : m == 1 ? smm : sbb;
+    R.s[4] = m == 0 ? sab : sbm;                       // (1, 2): a, b | m, b | b, m
+    R.s[5] = m == 2 ? smm : sbb;
     return R;
 }
 
