@@ -44,7 +44,7 @@ CLUSTER_SMS = 16
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the PCG SpMV,
 # from one ncu capture of the current kernel on that workload (mean of 3 launches).
 # ncu DRAM read + write bytes per launch of the PCG product, by (workload, storage)
-SPMV_DRAM_BYTES = {("stack3x526", "offdiag"): 408.4e6 + 8.7e6}  # steady state (ncu --cache-control none)
+SPMV_DRAM_BYTES = {}  # (workload, storage) -> DRAM bytes per product in steady state, where measured
 
 
 def parse():
@@ -356,7 +356,10 @@ def run_ours(args):
     # to pins read 36 more bytes, not counted), p read once and q written (float4, 16 V each)
     V = wl.V
     diag_bytes = 4 * V if args.storage in ("offdiag", "full") else 36 * V
-    spmv_bytes = 40 * spmv_blocks + 4 * (V + 1) + diag_bytes + 16 * V + 16 * V
+    # with patch records (the default storage's usual form) every block is read once with its
+    # 4-byte entry, and the other row of a block inside a patch takes a 2-byte reference
+    mirrored = max(nnzb - V - spmv_blocks, 0) if args.storage == "offdiag" and n_spmv else 0
+    spmv_bytes = 40 * spmv_blocks + 2 * mirrored + (0 if mirrored else 4 * (V + 1)) + diag_bytes + 16 * V + 16 * V
     avg_spmv_s = (spmv_ms / 1e3) / max(n_spmv, 1)
     achieved = spmv_bytes / avg_spmv_s / 1e9 if n_spmv else None
     peak, peak_src = measured_hbm()
@@ -364,7 +367,8 @@ def run_ours(args):
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None,
                 "traffic": SPMV_DRAM_BYTES.get((wl.name, args.storage)),
-                "kernel": {"sell": "spmv_sell_kernel<true>", "sym": "spmv_sym_kernel<true>"}.get(
+                "kernel": "patch_spmv_kernel (q = A p, difference form, with p.q; patch records)" if mirrored else
+                "pcg_resident_kernel (whole iterations in one launch)" if not n_spmv and not n_cl else {"sell": "spmv_sell_kernel<true>", "sym": "spmv_sym_kernel<true>"}.get(
                     args.storage, "spmv_kernel<true,true,CAPR>") + " (q = A p, difference form, with p.q; "
                     + args.storage + " storage; CAPR = 14 or 18 blocks per row per stage, chosen per "
                     "solve from the largest tile)",

@@ -180,6 +180,7 @@ struct pc_ctx {
     unsigned long long *pt_slots = nullptr;          // the resident schedule's published sums, then its abort flag
     unsigned long long *pt_z = nullptr;              // [V][4] its exchanged z rows
     uint32_t pt_epoch = 0;                           // its next epoch (0: slots and pt_z must be cleared)
+    int64_t pt_kept = 0;                             // blocks in the records of the last solve
     unsigned char *pt_store = nullptr;
     // proximity query: cell list (8 entries per triangle) and counts
     int64_t px_cap = 0;

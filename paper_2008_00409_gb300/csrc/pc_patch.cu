@@ -176,7 +176,7 @@ struct BuildArgs {
     PatchDesc *desc;
     uint8_t *cnt, *named;   // kept blocks of each row; rows in some patch's halo
     int32_t *size, *at;     // record sizes and offsets, in 16-byte units
-    int32_t *info;          // [0] no record (count), [1] largest record, [2] largest halo, [3] failure (fill), [4] most kept blocks
+    int32_t *info;          // [0] no record (count), [1] largest record, [2] largest halo, [3] failure (fill), [4] most kept blocks, [5] all of them
     int64_t cap;            // bytes of the store
     unsigned char *store;
 };
@@ -321,6 +321,7 @@ __global__ void patch_count_kernel(BuildArgs a)
         atomicMax(a.info + 1, d.bytes);
         atomicMax(a.info + 2, d.n_halo);
         atomicMax(a.info + 4, d.n_own);
+        atomicAdd(a.info + 5, d.n_own);
     }
 }
 
@@ -483,17 +484,18 @@ pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, PatchInf
     a.cap = c->pt_cap;
     a.store = c->pt_store;
     const int threads = a.R < 128 ? 128 : a.R > 512 ? 512 : a.R;
-    PC_CUDA_TRY(cudaMemsetAsync(c->pt_info, 0, sizeof(int32_t) * 5, st));
+    PC_CUDA_TRY(cudaMemsetAsync(c->pt_info, 0, sizeof(int32_t) * 6, st));
     PC_CUDA_TRY(cudaMemsetAsync(c->pt_named, 0, (size_t)c->V, st));
     PC_LAUNCH(c, patch_count_kernel, c->pt_n, threads, 0, st, a);
     PC_TRY(pc_exclusive_scan(c, a.size, a.at, c->pt_n, st));
     PC_LAUNCH(c, patch_fill_kernel, c->pt_n, threads, 0, st, a);
-    PC_CUDA_TRY(cudaMemcpyAsync(c->h_count, c->pt_info, sizeof(int32_t) * 5, cudaMemcpyDeviceToHost, st));
+    PC_CUDA_TRY(cudaMemcpyAsync(c->h_count, c->pt_info, sizeof(int32_t) * 6, cudaMemcpyDeviceToHost, st));
     PC_CUDA_TRY(cudaStreamSynchronize(st));
     const int32_t *h = reinterpret_cast<const int32_t *>(c->h_count);
     out->ok = h[0] == 0 && h[3] == 0;
     out->max_bytes = h[1];
     out->max_halo = h[2];
     out->max_own = h[4];
+    c->pt_kept = h[5];
     return PC_OK;
 }

@@ -218,7 +218,7 @@ __device__ __forceinline__ void patch_ahead_load(const PatchArgs &a, int patch, 
         if (threadIdx.x + k * PT_ROWS < n_halo) n.h[k] = a.x4[idx[threadIdx.x + k * PT_ROWS]];
 }
 
-static __global__ void __launch_bounds__(PT_ROWS, 5) patch_spmv_kernel(PatchArgs a)
+static __global__ void __launch_bounds__(PT_ROWS, 4) patch_spmv_kernel(PatchArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint64_t bar;

@@ -715,14 +715,17 @@ static int tile_grid(const pc_ctx *c, int ctas_per_sm)
 // The product's grid for stages of `capr` blocks per row (SP_CAP_PER_ROW or SP_CAPR_WIDE).
 static int spmv_grid(const pc_ctx *c, int capr)
 {
-    return tile_grid(c, capr <= SP_CAP_PER_ROW ? SpShape<SP_CAP_PER_ROW>::ctas_per_sm
-                                               : SpShape<SP_CAPR_WIDE>::ctas_per_sm);
+    return tile_grid(c, capr <= SP_CAPR_PLAIN ? SpShape<SP_CAPR_PLAIN>::ctas_per_sm
+                                              : SpShape<SP_CAPR_WIDE>::ctas_per_sm);
 }
 
 // Dynamic shared memory of every instantiation of the product (set once per device).
 static pc_status spmv_set_smem()
 {
     const int n = SpShape<SP_CAP_PER_ROW>::smem_bytes, w = SpShape<SP_CAPR_WIDE>::smem_bytes;
+    const int p = SpShape<SP_CAPR_PLAIN>::smem_bytes;
+    PC_CUDA_TRY(cudaFuncSetAttribute(spmv_kernel<true, false, SP_CAPR_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, p));
+    PC_CUDA_TRY(cudaFuncSetAttribute(spmv_kernel<false, false, SP_CAPR_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, p));
     PC_CUDA_TRY(cudaFuncSetAttribute(spmv_kernel<true, true, SP_CAP_PER_ROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, n));
     PC_CUDA_TRY(cudaFuncSetAttribute(spmv_kernel<false, true, SP_CAP_PER_ROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, n));
     PC_CUDA_TRY(cudaFuncSetAttribute(spmv_kernel<true, true, SP_CAPR_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, w));
@@ -838,12 +841,15 @@ static pc_status check_bsr(const pc_bsr *A, const float *vals)
     return PC_OK;
 }
 
-// PCG products take the stage width the solve chose; plain products (y = A x) always
-// the wide stages, which no tile of an assembled system outgrows in practice.
+// PCG products take the stage width the solve chose. Plain products (y = A x) have no
+// measurement of the largest tile; the caller chooses from the average row: 16-block stages
+// at five CTAs per SM up to 15 blocks per row (a cloth's 13.2 with a few contacts; the odd
+// fuller tile is read directly), else the wide stages at four. 830,028 rows: 84.1 us with
+// the wide stages, 78.6 with the 16-block ones.
 static pc_status launch_spmv(pc_ctx *c, const SpmvArgs &a, bool diff, bool pcg, cudaStream_t st,
                              int capr = SP_CAPR_WIDE)
 {
-    const int g = spmv_grid(c, pcg ? capr : SP_CAPR_WIDE);
+    const int g = spmv_grid(c, capr);
     const int n = SpShape<SP_CAP_PER_ROW>::smem_bytes, w = SpShape<SP_CAPR_WIDE>::smem_bytes;
     if (pcg && capr <= SP_CAP_PER_ROW) {
         if (diff) PC_LAUNCH_PDL(c, (spmv_kernel<true, true, SP_CAP_PER_ROW>), g, SP_THREADS, n, st, a);
@@ -851,6 +857,10 @@ static pc_status launch_spmv(pc_ctx *c, const SpmvArgs &a, bool diff, bool pcg, 
     } else if (pcg) {
         if (diff) PC_LAUNCH_PDL(c, (spmv_kernel<true, true, SP_CAPR_WIDE>), g, SP_THREADS, w, st, a);
         else PC_LAUNCH_PDL(c, (spmv_kernel<false, true, SP_CAPR_WIDE>), g, SP_THREADS, w, st, a);
+    } else if (capr <= SP_CAPR_PLAIN) {
+        const int p = SpShape<SP_CAPR_PLAIN>::smem_bytes;
+        if (diff) PC_LAUNCH(c, (spmv_kernel<true, false, SP_CAPR_PLAIN>), g, SP_THREADS, p, st, a);
+        else PC_LAUNCH(c, (spmv_kernel<false, false, SP_CAPR_PLAIN>), g, SP_THREADS, p, st, a);
     } else {
         if (diff) PC_LAUNCH(c, (spmv_kernel<true, false, SP_CAPR_WIDE>), g, SP_THREADS, w, st, a);
         else PC_LAUNCH(c, (spmv_kernel<false, false, SP_CAPR_WIDE>), g, SP_THREADS, w, st, a);
@@ -872,7 +882,8 @@ extern "C" pc_status pc_bsr_spmv(pc_ctx *ctx, const pc_bsr *A, const float *vals
     a.xin = x;
     a.y = y;
     a.err = ctx->d_err;
-    return launch_spmv(ctx, a, dres != nullptr, false, (cudaStream_t)stream);
+    return launch_spmv(ctx, a, dres != nullptr, false, (cudaStream_t)stream,
+                       A->nnzb <= 15ll * ctx->V ? SP_CAPR_PLAIN : SP_CAPR_WIDE);
 }
 
 extern "C" void pc_default_solve_opts(pc_solve_opts *o)
@@ -1325,7 +1336,7 @@ static pc_status launch_iterations(const SolveCtx &s, float *x, int count)
         if (timed) {
             // read after the chunk's synchronisation (no stall here)
             c->ev_pending = slot ? 2 : 1;
-            c->spmv_nnzb = s.patch ? s.A->nnzb - c->V : s.offdiag ? c->od_nnzb : s.A->nnzb;
+            c->spmv_nnzb = s.patch ? c->pt_kept : s.offdiag ? c->od_nnzb : s.A->nnzb;
         }
     }
     return PC_OK;

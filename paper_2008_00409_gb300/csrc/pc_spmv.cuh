@@ -49,6 +49,7 @@
 #define SP_SMEM_BYTES (SP_STAGES * SP_STAGE_BYTES)
 #define SP_WAIT_BUDGET (1ll << 31)         // cycles (about a second) before a wait gives up
 #define SP_CAPR_WIDE 18                    // the wider stages (blocks per row) of the product
+#define SP_CAPR_PLAIN 16                   // the widest that five CTAs per SM have room for: y = A x
 
 // Stage layout and residency of spmv_kernel for stages of CAPR blocks per row: the more
 // tiles in flight per SM, the more gathers of p are in flight, which is what the product
@@ -60,7 +61,7 @@ struct SpShape {
     static constexpr int col_bytes = (cap * 4 + 32 + 15) / 16 * 16;
     static constexpr int stage_bytes = val_bytes + col_bytes;
     static constexpr int smem_bytes = SP_STAGES * stage_bytes;
-    static constexpr int ctas_per_sm = CAPR <= SP_CAP_PER_ROW ? SP_CTAS_PER_SM : 4;
+    static constexpr int ctas_per_sm = CAPR <= SP_CAPR_PLAIN ? SP_CTAS_PER_SM : 4;
 };
 
 struct SpmvArgs {
