@@ -10,6 +10,8 @@
 // transpose bit for bit, a row that keeps more than PT_MAX_OWN blocks, a column
 // out of order, or a patch whose halo or store does not fit make the build report failure;
 // the solve then streams the BSR rows.
+#include <algorithm>
+
 #include "pc_patch.cuh"
 
 // ------------------------------------------------------------------------- order
@@ -75,16 +77,17 @@ __device__ __forceinline__ uint64_t spread3(uint32_t x)
     for (int b = 0; b < 16; ++b) r |= (uint64_t)((x >> b) & 1u) << (3 * b);
     return r;
 }
-__global__ void morton_kernel(int V, const float *__restrict__ X, const float *__restrict__ box, uint64_t *keys,
-                              uint32_t *vals)
+__global__ void morton_kernel(int V, const float *__restrict__ X, const float *__restrict__ box, int axis_bits,
+                              uint64_t *keys, uint32_t *vals)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= V) return;
     const float ext = fmaxf(box[3] - box[0], fmaxf(box[4] - box[1], box[5] - box[2]));
-    const float sc = ext > 0.f ? 65535.f / ext : 0.f;
+    const float top = (float)((1 << axis_bits) - 1);
+    const float sc = ext > 0.f ? top / ext : 0.f;
     uint64_t k = 0;
     for (int a = 0; a < 3; ++a) {
-        const float q = fminf(fmaxf((X[3ll * i + a] - box[a]) * sc, 0.f), 65535.f);
+        const float q = fminf(fmaxf((X[3ll * i + a] - box[a]) * sc, 0.f), top);
         k |= spread3((uint32_t)q) << a;
     }
     keys[i] = k;
@@ -95,10 +98,10 @@ __global__ void comp_key_kernel(int V, const int32_t *__restrict__ lab, const ui
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < V) keys[i] = (uint64_t)lab[vals[i]];
 }
-__global__ void patch_key_kernel(int V, int R, const uint32_t *__restrict__ vals, uint64_t *keys)
+__global__ void patch_key_kernel(int V, int R, int bits, const uint32_t *__restrict__ vals, uint64_t *keys)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < V) keys[i] = ((uint64_t)(i / R) << 32) | vals[i];
+    if (i < V) keys[i] = ((uint64_t)(i / R) << bits) | vals[i];
 }
 __global__ void order_kernel(int V, const uint32_t *__restrict__ vals, int32_t *old_of, int32_t *new_of)
 {
@@ -118,51 +121,77 @@ pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
     c->pt_n = (V + c->pt_rows - 1) / c->pt_rows;
     // kept blocks at most all of them; entries 4 bytes each, twice that with the slices' padding
     c->pt_cap = 48 * c->A_cap + (int64_t)c->pt_n * 1024;
-    if (c->sort.cap < V) return PC_OK;  // no order: the solves stream the BSR rows
-    PC_CUDA_TRY(cudaMalloc(&c->pt_old, sizeof(int32_t) * (size_t)V));
-    PC_CUDA_TRY(cudaMalloc(&c->pt_new, sizeof(int32_t) * (size_t)V));
-    PC_CUDA_TRY(cudaMalloc(&c->pt_desc, sizeof(PatchDesc) * (size_t)c->pt_n));
-    PC_CUDA_TRY(cudaMalloc(&c->pt_cnt, (size_t)c->pt_n * c->pt_rows));
-    PC_CUDA_TRY(cudaMalloc(&c->pt_named, (size_t)V));
-    PC_CUDA_TRY(cudaMalloc(&c->pt_size, sizeof(int32_t) * 2 * (c->pt_n + 1ll)));
-    PC_CUDA_TRY(cudaMalloc(&c->pt_info, sizeof(int32_t) * 8));
-    PC_CUDA_TRY(cudaMalloc(&c->pt_store, (size_t)c->pt_cap));
-    if (c->pt_n <= c->num_sms) {
-        PC_CUDA_TRY(cudaMalloc(&c->pt_slots, sizeof(uint64_t) * (12 * (size_t)c->pt_n * c->pt_n + 1)));
-        PC_CUDA_TRY(cudaMalloc(&c->pt_z, 4 * sizeof(uint64_t) * (size_t)V));
+    // the arrays, in one allocation (pc_destroy frees it through pt_old)
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = at;
+        at += (bytes + 255) / 256 * 256;
+        return o;
+    };
+    const bool resident = c->pt_n <= c->num_sms;
+    const size_t o_old = take(sizeof(int32_t) * (size_t)V), o_new = take(sizeof(int32_t) * (size_t)V);
+    const size_t o_desc = take(sizeof(PatchDesc) * (size_t)c->pt_n), o_cnt = take((size_t)c->pt_n * c->pt_rows);
+    const size_t o_named = take((size_t)V), o_size = take(sizeof(int32_t) * 2 * (c->pt_n + 1ll)), o_info = take(32);
+    const size_t o_z = take(resident ? 4 * sizeof(uint64_t) * (size_t)V : 0);
+    const size_t o_slots = take(resident ? sizeof(uint64_t) * (12 * (size_t)c->pt_n * c->pt_n + 1) : 0);
+    const size_t o_store = take((size_t)c->pt_cap);
+    unsigned char *base = nullptr;
+    PC_CUDA_TRY(cudaMalloc(&base, at));
+    c->pt_old = reinterpret_cast<int32_t *>(base + o_old);
+    c->pt_new = reinterpret_cast<int32_t *>(base + o_new);
+    c->pt_desc = base + o_desc;
+    c->pt_cnt = base + o_cnt;
+    c->pt_named = base + o_named;
+    c->pt_size = reinterpret_cast<int32_t *>(base + o_size);
+    c->pt_info = reinterpret_cast<int32_t *>(base + o_info);
+    if (resident) {
+        c->pt_z = reinterpret_cast<unsigned long long *>(base + o_z);
+        c->pt_slots = reinterpret_cast<unsigned long long *>(base + o_slots);
     }
-    uint64_t *keys = nullptr;
-    uint32_t *vals = nullptr;
-    float *box = nullptr;
-    PC_CUDA_TRY(cudaMalloc(&keys, sizeof(uint64_t) * (size_t)V + sizeof(uint32_t) * (size_t)V + 32));
-    vals = reinterpret_cast<uint32_t *>(keys + V);
-    box = reinterpret_cast<float *>(vals + V);
+    // keys and values in the proximity query's lists (8 entries per triangle) where they have room
+    const bool own = c->px_cap < V;
+    uint64_t *keys = c->px_keys;
+    uint32_t *vals = c->px_vals;
+    if (own) {
+        keys = nullptr;
+        PC_CUDA_TRY(cudaMalloc(&keys, (sizeof(uint64_t) + sizeof(uint32_t)) * (size_t)V));
+        vals = reinterpret_cast<uint32_t *>(keys + V);
+    }
+    float *box = reinterpret_cast<float *>(c->pt_info);
     int32_t *lab = c->pt_new, *changed = reinterpret_cast<int32_t *>(c->d_count);
     const unsigned g = pc_blocks(V, 256);
+    // the curve's cells: eight times as fine, along each axis, as V vertices on a square
+    const int axis = std::min(16, pc_bits_for(V) / 2 + 3);
     pc_status s = PC_OK;
     do {
         comp_init_kernel<<<g, 256, 0, st>>>(V, lab);
-        for (int it = 0; it < 64; ++it) {  // the labels halve their number of steps each round; 64 never binds
+        for (int it = 0; it < 32; ++it) {  // each round at least halves the steps that are left; 32 never binds
             cudaMemsetAsync(changed, 0, sizeof(int32_t), st);
-            comp_hook_kernel<<<g, 256, 0, st>>>(V, c->erp, c->ecol, lab, changed);
-            comp_compress_kernel<<<g, 256, 0, st>>>(V, lab);
+            for (int k = 0; k < 3; ++k) {
+                if (k == 2) cudaMemsetAsync(changed, 0, sizeof(int32_t), st);  // the last pass decides
+                comp_hook_kernel<<<g, 256, 0, st>>>(V, c->erp, c->ecol, lab, changed);
+                comp_compress_kernel<<<g, 256, 0, st>>>(V, lab);
+            }
+            c->launches += 6;
             cudaMemcpyAsync(c->h_count, changed, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
             if (cudaStreamSynchronize(st) != cudaSuccess) { s = PC_ERR_CUDA; break; }
             if (*reinterpret_cast<int32_t *>(c->h_count) == 0) break;
         }
         if (s != PC_OK) break;
         bbox_kernel<<<1, 1024, 0, st>>>(V, c->rest, box);
-        morton_kernel<<<g, 256, 0, st>>>(V, c->rest, box, keys, vals);
-        if ((s = pc_radix_sort(c, keys, vals, V, 48, st)) != PC_OK) break;
+        morton_kernel<<<g, 256, 0, st>>>(V, c->rest, box, axis, keys, vals);
+        if ((s = pc_radix_sort(c, keys, vals, V, 3 * axis, st)) != PC_OK) break;
         comp_key_kernel<<<g, 256, 0, st>>>(V, lab, vals, keys);
         if ((s = pc_radix_sort(c, keys, vals, V, pc_bits_for(V), st)) != PC_OK) break;
-        patch_key_kernel<<<g, 256, 0, st>>>(V, c->pt_rows, vals, keys);
-        if ((s = pc_radix_sort(c, keys, vals, V, 32 + pc_bits_for(c->pt_n), st)) != PC_OK) break;
+        // within a patch by original number: the values' low bits first, then the patch
+        patch_key_kernel<<<g, 256, 0, st>>>(V, c->pt_rows, pc_bits_for(V), vals, keys);
+        if ((s = pc_radix_sort(c, keys, vals, V, pc_bits_for(V) + pc_bits_for(c->pt_n), st)) != PC_OK) break;
         order_kernel<<<g, 256, 0, st>>>(V, vals, c->pt_old, c->pt_new);
         c->launches += 6;
         if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) s = PC_ERR_CUDA;
     } while (0);
-    cudaFree(keys);
+    if (own) cudaFree(keys);
+    if (s == PC_OK) c->pt_store = base + o_store;  // (null: no order, the solves stream the BSR rows)
     return s;
 }
 

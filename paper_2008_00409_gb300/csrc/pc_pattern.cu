@@ -3,8 +3,9 @@
 //
 // The paper fills a per-row index table with atomics, then sorts and compacts each row
 // (Sec. 3.2.2 steps 2-3). Here the static mesh pattern is built once by sorting all
-// element keys; each step only the contact keys are sorted, deduplicated and merged into
-// the static pattern by ranking, so row pointers and column indices are bit-exact.
+// element keys; each step only the contacts are placed by row counts, ordered and
+// deduplicated within their rows and merged into the static pattern, so row pointers and
+// column indices are bit-exact.
 #include <stdlib.h>
 #include <string.h>
 
@@ -346,8 +347,7 @@ static void free_ctx(pc_ctx *c)
                     c->sym_uci, c->sym_lcol, c->sym_lsrc, c->sym_uvals, c->sell_perm, c->sell_width,
                     c->sell_base, c->sell_dpos, c->sell_data, c->sell_diag, c->od_rp, c->od_cnt, c->od_dpos,
                     c->od_ci, c->od_vals, c->px_keys, c->px_vals, c->px_cnt, c->px_off, c->px_vcnt, c->px_voff,
-                    c->px_max, c->px_box, c->px_hits, c->px_first, c->dsc, c->fbar, c->pt_old, c->pt_new, c->pt_desc, c->pt_cnt, c->pt_size, c->pt_info,
-                    c->pt_store, c->pt_slots, c->pt_z, c->pt_named};
+                    c->px_max, c->px_box, c->px_hits, c->px_first, c->dsc, c->fbar, c->pt_old /* and the other pt_ arrays */};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (c->sc_host) cudaFreeHost(c->sc_host);
@@ -563,8 +563,8 @@ static pc_status create_impl(pc_ctx *c, const int32_t *tris, const float *rest, 
     PC_CUDA_TRY(cudaMemsetAsync(c->A_dv, 0, sizeof(float) * 3 * (size_t)V, st));
     PC_TRY(pc_solver_alloc(c));
     PC_TRY(pc_batched_alloc(c));
-    PC_TRY(pc_patch_alloc(c, st));
     PC_TRY(pc_proximity_alloc(c));
+    PC_TRY(pc_patch_alloc(c, st));
     PC_CUDA_TRY(cudaStreamSynchronize(st));
     return PC_OK;
 }
