@@ -155,8 +155,11 @@ typedef struct {
  * third more. It takes systems up to about 6,000 rows at cloth density (at most 512 rows
  * per CTA, and every CTA's blocks and copied rows within its shared memory); larger ones
  * return PC_ERR_CAPACITY.
- * PC_SCHED_GRID: kernels over the whole GPU, iterations launched from the host (the
- * storage and fuse options apply).
+ * PC_SCHED_GRID: kernels over the whole GPU (the storage and fuse options apply). Iterations
+ * are launched from the host, except that with the default storage and fuse = 1, in the
+ * difference form, systems of up to 480 rows per SM (72,960 on GB300) whose records fit run
+ * whole stretches of iterations in one cooperative launch, one CTA per SM, out of shared
+ * memory: the same iteration and stop tests, sums in another order.
  * PC_SCHED_AUTO: the cluster schedule when the system fits it, else the grid schedule. */
 #define PC_SCHED_AUTO 0
 #define PC_SCHED_GRID 1
@@ -179,7 +182,11 @@ typedef struct {
 /* PC_STORAGE_OFFDIAG: with the difference-form diagonal given (dres), the products read a
  * copy of the BSR matrix without its diagonal blocks, made at the start of each solve (in
  * the difference form the diagonal block multiplies p_i - p_i = 0, so the copy gives the
- * same product with one block per row fewer to stream). Without dres, or when the copy
+ * same product with one block per row fewer to stream). The copy keeps rows in patches of
+ * neighbouring vertices and stores a block between two rows of a patch once for both, where
+ * the matrix's blocks inside the patches are symmetric bit for bit, as pc_assemble_values
+ * makes them; otherwise, or with rows of more than 64 kept blocks or patches of too many
+ * contacts for shared memory, it is a plain BSR copy. Without dres, or when the copy
  * exceeds the context's capacity, the products read the matrix itself. */
 #define PC_STORAGE_SYM 0
 #define PC_STORAGE_FULL 1
@@ -254,9 +261,9 @@ PC_API pc_status pc_get_rest(const pc_ctx *ctx, int32_t *hinges, float *mass, vo
 
 /* Sec. 3.2.2, dynamic matrix assembly, pattern half: the step's block pattern is the set
  * of (row, col) vertex pairs coupled by any triangle, hinge or contact pair of this step,
- * plus the diagonal, sorted by (row, col) with duplicates removed. The contact keys are
- * sorted with a key sort and merged into the static pattern (no atomics), so row_ptr and
- * col_idx are bit-exact and deterministic.
+ * plus the diagonal, sorted by (row, col) with duplicates removed. The contacts' columns are
+ * put in order row by row (with a key sort when a vertex has more than 64 contacts) and
+ * merged into the static pattern, so row_ptr and col_idx are bit-exact and deterministic.
  * On return A->nnzb holds the block count. If it exceeds A->cap the call returns
  * PC_ERR_CAPACITY with A->nnzb = required size and col_idx untouched beyond cap.
  * Synchronizes `stream`. */

@@ -5,13 +5,14 @@
 // a block (i, j) with both rows in one patch is kept by one of them only and used for both,
 // y_i += B (p_j - p_i) and y_j += B^T (p_i - p_j); a block that leaves its patch is kept by
 // both rows. On a cloth (12 off-diagonal blocks per row) a 128-row patch keeps about 7 blocks
-// per row: about 310 bytes per row in all, instead of the 480 of the BSR rows.
+// per row: about 310 bytes per row in all, instead of the 480 of the BSR rows. At 830,028
+// rows (three 526 x 526 layers) a product takes 53 us, 73 from the BSR rows.
 //
 // The keeping row's thread forms both products from one read of the block and leaves the
 // other row's share in the block's own place; the other row's thread adds it after a
 // barrier. (Reading the kept block a second time, transposed, was built first: twice the
 // shared-memory wavefronts, half of them bank conflicts, and 54 us per product at paper
-// scale.) Each sum has a fixed order.
+// scale.) Each sum has a fixed order, so the product is deterministic.
 //
 // Record of a patch, every part 16-byte aligned (n_own kept blocks; a slice is 32 rows):
 //   first   int32[2][R / 32 + 1]: where each slice's entries and shares begin, in columns of 32
@@ -182,6 +183,12 @@ struct PatchArgs {
 // the p of the halo's first 2 x 128 rows, which wait in registers during the computation. The
 // first record does not depend on the preceding kernel and is requested before the
 // programmatic wait.
+// Bound by shared-memory wavefronts and their latency at 16 warps per SM about as much as by
+// HBM: 52.9 us at 830,028 rows, 275 MB, 5.2 TB/s (the BSR stream: 73 us, 439 MB). Patches of 64
+// and 160 rows take 56.5 and 53.7 us: 128 keeps as many blocks inside as four CTAs of an SM
+// have room for. The slowest SM needs a fifth more cycles than the average; handing out the
+// last patches by ticket evened that out but needs a partial sum per patch to keep the order of
+// p.q, which cost more than it gave (a whole step 629 -> 681 ms).
 #define PT_AHEAD 2  // halo rows per thread fetched a patch ahead
 
 struct PatchAhead {

@@ -2,16 +2,21 @@
 // equations are solved with a preconditioned conjugate gradient solver; Sec. 3.1: the
 // SpMV is the most expensive operator and vector operations are data parallel).
 //
-// Per iteration two kernels run by default:
+// A system whose patch records fit the GPU's shared memory runs whole stretches of iterations
+// in one cooperative launch (pc_resident.cuh; measured against the kernels below there).
+// Otherwise two kernels run per iteration by default:
 //   spmv:           q = A p, partial p.q                             -> alpha = rz / pq
 //   update + dir:   x += alpha p, r -= alpha q, z = D^-1 r, partial r.z, r.r; a grid-wide
 //                   barrier; beta, stop test; p = z + beta p        (pcg_update_dir_kernel)
 // or, when the rows do not fit the fused kernel's registers (or fuse = 0), three:
 //   direction: p = z + beta p; spmv; update (z to memory, the last block forms beta).
-// The SpMV kernel, a bulk-copy pipelined stream over the blocks, is in pc_spmv.cuh; it
-// reads by default a per-solve copy of the matrix without its diagonal blocks, in stages
-// of 14 blocks per row at five CTAs per SM when the matrix's largest 32-row tile fits
-// them, else of 18 at four (measured per solve by tile_max_kernel).
+// The product streams patch records (pc_patch.cuh) where the matrix suits them: the
+// difference form, in-patch blocks symmetric to the bit, records within an SM's shared
+// memory; the vectors are then in the patches' row order. Otherwise it is the bulk-copy
+// pipelined stream over BSR blocks of pc_spmv.cuh, which reads by default a per-solve copy of
+// the matrix without its diagonal blocks, in stages of 14 blocks per row at five CTAs per
+// SM when the matrix's largest 32-row tile fits them, else of 18 at four (measured per solve
+// by tile_max_kernel). Per product at 830,028 rows: 53 us and 73 us.
 // Dot products: FP32 within a thread, FP64 across threads; partials are summed in a fixed
 // order, so every reduction is deterministic. p, q and z are float4 per vertex (each SpMV
 // gather is one 16-byte load); x, r and the scalar Jacobi inverse, only ever streamed,

@@ -119,8 +119,8 @@ __device__ __forceinline__ void strain_from_edges(const dfl *e1, const dfl *e2, 
 // first-order form of h f(x_t + h v_t) (Eq. 2-3); since each Hessian row sums to zero,
 // sum_l H_kl v_l is formed as sum_l H_kl (v_l - v_k).
 // Bound by DRAM (reads 56 B of rest data per triangle, writes 128 B): the records are
-// staged in shared memory so that every store is a full line. 1.65M triangles: 523 us with
-// 256-byte records stored a float at a time.
+// staged in shared memory so that every store is a full line. 1.65M triangles: 64 us (523 with
+// 256-byte records stored a float at a time).
 #define TE_THREADS 128
 
 struct TriFactors {
@@ -339,7 +339,7 @@ __device__ __forceinline__ float hinge_angle_grad(float3 a1, float3 a2, float3 a
 // grad_k too: h f_k = -h (2 kb c_h) (theta - theta_rest) grad_k. Record: four float4 (q_k, w),
 // 64 bytes, instead of 12 contributions and 12 gradients. The gradient sums to zero over
 // the four vertices, so q . v uses velocities relative to edge0. Bound by DRAM (reads 24 B
-// of rest data and writes 64 B per hinge); 2.48M hinges: 247 us with 96-byte records.
+// of rest data and writes 64 B per hinge); 2.48M hinges: 60 us (247 with 96-byte records).
 __global__ void __launch_bounds__(128) hinge_eval_kernel(int H, const int32_t *__restrict__ hinge,
                                                          const float *__restrict__ x, const float *__restrict__ v,
                                                          const float *__restrict__ hcoef,
@@ -552,7 +552,9 @@ __device__ __forceinline__ void row_block(const RowArgs &a, int row, int slot, i
 // Bound by DRAM and L2: 44 B per block written (vals and its column read), about 5
 // contributions of 64..128 B per block read through L1. At 830k rows / 10.9M blocks: before,
 // a warp per row staged every expanded block and each lane compared all of them with
-// its column, 2,825 us.
+// its column, 2,825 us; now 784 us, most of it L1 looking up a line per lane for each
+// 16-byte read of a record (76% of L1's rate; DRAM 20%). Copying a tile's records to shared
+// memory first was slower (1,086 -> 1,525 us for the whole assembly).
 __global__ void __launch_bounds__(RR_THREADS) row_reduce_kernel(RowArgs a)
 {
     __shared__ float s_blk[RR_CAP * 9];
