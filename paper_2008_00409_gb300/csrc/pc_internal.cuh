@@ -130,7 +130,7 @@ struct pc_ctx {
     const int32_t *last_pairs = nullptr;
 
     // element buffers
-    float *tri_buf = nullptr;      // [T][PC_TRI_STRIDE]
+    float4 *tri_buf = nullptr;     // [T / 8, rounded up][PC_TRI_STRIDE / 4][8]: tri_quad (pc_values.cu)
     float *hinge_buf = nullptr;    // [H][PC_HINGE_STRIDE]
     float *cont_buf = nullptr;     // [maxP][PC_CONTACT_STRIDE]
 

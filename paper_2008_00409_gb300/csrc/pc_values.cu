@@ -118,10 +118,17 @@ __device__ __forceinline__ void strain_from_edges(const dfl *e1, const dfl *e2, 
 // c_k = h f_k - sum_l (h^2 H_kl) v_l is the element's share of b = h (f - h K v), the
 // first-order form of h f(x_t + h v_t) (Eq. 2-3); since each Hessian row sums to zero,
 // sum_l H_kl v_l is formed as sum_l H_kl (v_l - v_k).
-// Bound by DRAM (reads 56 B of rest data per triangle, writes 128 B): the records are
-// staged in shared memory so that every store is a full line. 1.65M triangles: 64 us (523 with
-// 256-byte records stored a float at a time).
+// Eight consecutive triangles' records are interleaved, quad by quad (tri_quad): lanes that
+// read the same quad of neighbouring triangles share a line (row reduction at 830k rows: 784
+// us with each record a line of its own, 676 interleaved).
+// Bound by DRAM (reads 56 B of rest data per triangle, writes 128 B): 1.65M triangles: 64 us
+// (523 with 256-byte records stored a float at a time).
 #define TE_THREADS 128
+
+__host__ __device__ __forceinline__ int64_t tri_quad(uint32_t id, int quad)
+{
+    return (int64_t)(PC_TRI_STRIDE / 4) * (id & ~7u) + 8 * quad + (id & 7u);
+}
 
 struct TriFactors {
     float Fg[3][3];  // F g_k
@@ -146,9 +153,8 @@ __global__ void __launch_bounds__(TE_THREADS) tri_eval_kernel(int T, const int32
                                                        const float *__restrict__ dmi_all,
                                                        const float *__restrict__ area, const float *__restrict__ rgram,
                                                        float mu, float lam, float h, float hk,
-                                                       float *__restrict__ out)
+                                                       float4 *__restrict__ out)
 {
-    __shared__ float s_rec[TE_THREADS][PC_TRI_STRIDE + 1];
     const int t = blockIdx.x * TE_THREADS + threadIdx.x;
     if (t < T) {
         int i0 = tri[3 * t], i1 = tri[3 * t + 1], i2 = tri[3 * t + 2];
@@ -242,42 +248,31 @@ __global__ void __launch_bounds__(TE_THREADS) tri_eval_kernel(int T, const int32
                         ck[l][b] = fmaf(e, d[a], ck[l][b]);
                     }
             }
-        float *o = s_rec[threadIdx.x];
         const int m = R.gg[0] >= R.gg[3] && R.gg[0] >= R.gg[5] ? 0 : R.gg[3] >= R.gg[5] ? 1 : 2;
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-#pragma unroll
-            for (int a = 0; a < 3; ++a) o[4 * k + a] = ck[k][a];
-        o[3] = R.cm;
-        o[7] = m == 0 ? R.s[3] : R.s[0];
-        o[11] = m == 0 ? R.s[4] : m == 1 ? R.s[2] : R.s[1];
+        float Fa[3], Fb[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            o[12 + a] = m == 0 ? R.Fg[1][a] : R.Fg[0][a];
-            o[16 + a] = m == 2 ? R.Fg[1][a] : R.Fg[2][a];
-            o[20 + a] = R.M[a];
-            o[24 + a] = R.M[3 + a];
-            o[28 + a] = R.gg[3 + a];
+            Fa[a] = m == 0 ? R.Fg[1][a] : R.Fg[0][a];
+            Fb[a] = m == 2 ? R.Fg[1][a] : R.Fg[2][a];
         }
-        o[15] = m == 2 ? R.s[3] : R.s[5];
-        o[19] = R.gg[0];
-        o[23] = R.gg[1];
-        o[27] = R.gg[2];
-        o[31] = __int_as_float(m);
+        float4 *o = out + tri_quad(t, 0);
+        o[0] = make_float4(ck[0][0], ck[0][1], ck[0][2], R.cm);
+        o[8] = make_float4(ck[1][0], ck[1][1], ck[1][2], m == 0 ? R.s[3] : R.s[0]);
+        o[16] = make_float4(ck[2][0], ck[2][1], ck[2][2], m == 0 ? R.s[4] : m == 1 ? R.s[2] : R.s[1]);
+        o[24] = make_float4(Fa[0], Fa[1], Fa[2], m == 2 ? R.s[3] : R.s[5]);
+        o[32] = make_float4(Fb[0], Fb[1], Fb[2], R.gg[0]);
+        o[40] = make_float4(R.M[0], R.M[1], R.M[2], R.gg[1]);
+        o[48] = make_float4(R.M[3], R.M[4], R.M[5], R.gg[2]);
+        o[56] = make_float4(R.gg[3], R.gg[4], R.gg[5], __int_as_float(m));
     }
-    __syncthreads();
-    const int n = min(TE_THREADS, T - (int)blockIdx.x * TE_THREADS) * PC_TRI_STRIDE;
-    float *o = out + (int64_t)blockIdx.x * TE_THREADS * PC_TRI_STRIDE;
-    for (int i = threadIdx.x; i < n; i += TE_THREADS) o[i] = s_rec[i / PC_TRI_STRIDE][i % PC_TRI_STRIDE];
 }
 
 // The factors of triangle record `id` (cl_cm = lam / mu).
-__device__ __forceinline__ TriFactors tri_load(const float *__restrict__ buf, uint32_t id, float cl_cm)
+__device__ __forceinline__ TriFactors tri_load(const float4 *__restrict__ buf, uint32_t id, float cl_cm)
 {
-    const float4 *r = reinterpret_cast<const float4 *>(buf) + (int64_t)(PC_TRI_STRIDE / 4) * id;
-    const float cm = reinterpret_cast<const float *>(r)[3], saa = reinterpret_cast<const float *>(r)[7],
-                sab = reinterpret_cast<const float *>(r)[11];
-    const float4 fa = r[3], fb = r[4], m0 = r[5], m1 = r[6], q = r[7];
+    const float4 *r = buf + tri_quad(id, 0);
+    const float cm = r[0].w, saa = r[8].w, sab = r[16].w;
+    const float4 fa = r[24], fb = r[32], m0 = r[40], m1 = r[48], q = r[56];
     const int m = __float_as_int(q.w);
     const float Fa[3] = {fa.x, fa.y, fa.z}, Fb[3] = {fb.x, fb.y, fb.z}, sbb = fa.w;
     TriFactors R;
@@ -435,7 +430,7 @@ __global__ void contact_eval_kernel(int P, const int32_t *__restrict__ pairs, co
 // (col, row) has the same elements in the same order and the products commute, so A is
 // bitwise symmetric.
 __device__ __forceinline__ void add_static(const uint32_t *__restrict__ codes, int c0, int c1,
-                                           const float *__restrict__ tri_buf, const float4 *__restrict__ hinge_buf,
+                                           const float4 *__restrict__ tri_buf, const float4 *__restrict__ hinge_buf,
                                            float cl_cm, float acc[9])
 {
     for (int c = c0; c < c1; ++c) {
@@ -514,7 +509,7 @@ struct RowArgs {
     const int32_t *cinc_ptr;
     const uint32_t *cinc;
     const int32_t *pairs;
-    const float *tri_buf;
+    const float4 *tri_buf;
     const float4 *hinge_buf;
     const float *cont_buf;
     const float *mass;
@@ -552,8 +547,8 @@ __device__ __forceinline__ void row_block(const RowArgs &a, int row, int slot, i
 // Bound by DRAM and L2: 44 B per block written (vals and its column read), about 5
 // contributions of 64..128 B per block read through L1. At 830k rows / 10.9M blocks: before,
 // a warp per row staged every expanded block and each lane compared all of them with
-// its column, 2,825 us; now 784 us, most of it L1 looking up a line per lane for each
-// 16-byte read of a record (76% of L1's rate; DRAM 20%). Copying a tile's records to shared
+// its column, 2,825 us; now 676 us, most of it L1 looking up lines for the lanes' 16-byte
+// reads of records (76% of L1's rate before the triangles were interleaved; DRAM 20%). Copying a tile's records to shared
 // memory first was slower (1,086 -> 1,525 us for the whole assembly).
 __global__ void __launch_bounds__(RR_THREADS) row_reduce_kernel(RowArgs a)
 {
@@ -596,7 +591,7 @@ __global__ void __launch_bounds__(RR_THREADS) row_reduce_kernel(RowArgs a)
                 u[4] = __fadd_rn(u[4], __fmul_rn(q.y, q.z));
                 u[5] = __fadd_rn(u[5], __fmul_rn(q.z, q.z));
             } else {
-                const float4 c = reinterpret_cast<const float4 *>(a.tri_buf)[8ll * id + k];
+                const float4 c = a.tri_buf[tri_quad(id, k)];
                 f[0] += c.x;
                 f[1] += c.y;
                 f[2] += c.z;
