@@ -181,6 +181,28 @@ def test_values_at_tile_edges_match_oracle(pc, wl):
     cl.close()
 
 
+# a vertex shared by many separate fans of eight triangles: more blocks in a tile of 32 rows
+# than its staging holds; with contacts between the fans and without
+@pytest.mark.parametrize("fans,contacts", [(59, False), (60, False), (60, True), (140, False), (140, True)])
+def test_values_of_a_vertex_with_many_blocks(pc, fans, contacts):
+    a = 2.0 * np.pi * np.arange(8) / 8
+    ring = np.stack([0.1 * np.cos(a), 0.1 * np.sin(a), 0.0 * a], -1)
+    rest = np.concatenate([[[0.0, 0.0, 0.02]]] + [ring + [0.0, 0.0, 0.002 * k] for k in range(fans)])
+    tris = [[0, 1 + 8 * f + k, 1 + 8 * f + (k + 1) % 8] for f in range(fans) for k in range(8)]
+    wl = _workload(rest, tris, [3])
+    cl, om = pc.Cloth(wl, max_contacts=fans), oracle.Mesh.from_workload(wl)
+    pairs = w = tp = tw = None
+    if contacts:
+        pairs = np.array([[1 + 8 * f, *tris[8 * (f + 1) + 3]] for f in range(fans // 2)], np.int32)
+        w = np.random.default_rng(2).dirichlet([1.0, 1.0, 1.0], len(pairs)).astype(np.float32)
+        tp, tw = torch.from_numpy(pairs).cuda(), torch.from_numpy(w).cuda()
+    s = cl.assemble(tp, tw)
+    rp, ci, vals, b = om.assemble(wl.x0.astype(np.float64), wl.v0.astype(np.float64), pairs, w, wl.h)
+    np.testing.assert_array_equal(_np(s["col_idx"])[: s["nnzb"]], ci)
+    assert H.block_errors(rp, ci, _np(s["vals"])[: 9 * s["nnzb"]], vals).max() <= 0
+    cl.close()
+
+
 @pytest.mark.parametrize("layers,delta", [(3, 5.5e-4), (5, 1.2e-3), (2, 5e-5)])
 def test_proximity_of_many_and_of_far_apart_triangles(pc, layers, delta):
     """More pairs at a vertex than the counting pass remembers (vertices right above each
