@@ -78,6 +78,8 @@ struct BtArgs {
     double tol, refresh;
     int max_iter, refresh_every;
     int spmv_chunked;          // SpMV entry order: 0 strided, 1 contiguous chunks (autotuned)
+    long long l2_room;         // bytes of L2 for the vectors and what it keeps of the matrix (pc_l2_keep)
+    int tile_bytes;            // of the SpMV phase's matrix, on average
     long long bar_wait;        // cycles a grid-barrier wait may take before the launch aborts
 };
 
@@ -453,6 +455,10 @@ __device__ void bt_phase_spmv(const BtArgs &a, const bt_list &L, unsigned char *
             bt_cursor cu;
             bt_cursor_load(a, L, bt_find(L, j0), cu);
             int issued = 0;
+            // this CTA's share of the tiles that L2 keeps from one product to the next (16 garments,
+            // 321,000 rows, one step: 152 -> 141 ms)
+            const long long room = a.l2_room - 90ll * BT_TILE * L.total;
+            const int keep = room > 0 ? (int)min((long long)nent, room / a.tile_bytes * nent / L.total + 1) : 0;
             for (int e = 0; e < nent; ++e) {
                 const int j = j0 + e * G;
                 if (j >= cu.p1) bt_cursor_load(a, L, bt_find(L, j), cu);
@@ -476,8 +482,13 @@ __device__ void bt_phase_spmv(const BtArgs &a, const bt_list &L, unsigned char *
                     stage_info[s][2] = b0 - c0;
                     stage_info[s][3] = 1;
                     mbar_arrive_expect_tx(&full_bar[s], vbytes + cbytes);
-                    bulk_g2s(base, a.svals + al0, vbytes, &full_bar[s]);
-                    bulk_g2s(base + SpShape<CAPR>::val_bytes, a.sci + c0, cbytes, &full_bar[s]);
+                    if (e < keep) {
+                        bulk_g2s_keep(base, a.svals + al0, vbytes, &full_bar[s]);
+                        bulk_g2s_keep(base + SpShape<CAPR>::val_bytes, a.sci + c0, cbytes, &full_bar[s]);
+                    } else {
+                        bulk_g2s(base, a.svals + al0, vbytes, &full_bar[s]);
+                        bulk_g2s(base + SpShape<CAPR>::val_bytes, a.sci + c0, cbytes, &full_bar[s]);
+                    }
                 } else {
                     stage_info[s][0] = b0;
                     stage_info[s][1] = 0;
@@ -1134,6 +1145,10 @@ static pc_status bt_enqueue(pc_ctx *c, pc_batched_state *B, const pc_bsr *A, con
     a.max_iter = o.max_iter;
     a.refresh_every = o.refresh_every;
     a.spmv_chunked = spmv_order;
+    int64_t room = 0;
+    PC_TRY(pc_l2_keep(c, 0, &room));
+    a.l2_room = room;
+    a.tile_bytes = (int)std::max<int64_t>(1, 40ll * BT_TILE * (A->nnzb - (a.dsc ? V : 0)) / V);
     a.bar_wait = c->bar_wait_cycles > 0 ? (long long)c->bar_wait_cycles : SP_WAIT_BUDGET;
     return bt_launch(c, B, a, dres != nullptr, grid, capr, st);
 }

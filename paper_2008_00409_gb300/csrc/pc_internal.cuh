@@ -315,6 +315,21 @@ pc_status pc_warm_guess(pc_ctx *c, const pc_bsr *A, const float *v, float h, int
 void pc_mlp_ctx_free(pc_ctx *c);
 // Patch storage of the system being solved (pc_patch.cu): allocation and row order, and the
 // records of one matrix (ok = false: the matrix does not suit it and nothing is usable).
+// Bytes of a matrix stream that L2 can hold from one product of an iterative solve to the
+// next beside the solve's vectors (about 90 bytes per row): the stream's first `*keep` bytes
+// are copied with the ordinary policy, the rest evict-first. What every SM reads takes room
+// in both halves of the L2, so about 0.55 of it counts. Patch records, us per iteration with
+// 0 / 20 / 40 / 60 / 80 MB kept (L2 135 MB, so the rule keeps 51, 41, 28 and 0 MB):
+//   262,144 rows 27.5 / 25.3 / 24.1 / 23.4 / 24.6    372,100 rows 36.0 / 34.6 / 32.7 / 33.3 / 37.0
+//   518,400 rows 44.0 / 42.6 / 42.0 / 45.6 / 50.7    829,921 rows 63.3 / 64.9 / 68.4 / 71.9 / 73.1
+inline pc_status pc_l2_keep(const pc_ctx *c, int64_t rows, int64_t *keep)
+{
+    int l2 = 0;
+    PC_CUDA_TRY(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device));
+    const int64_t room = (int64_t)(0.55 * l2) - 90 * rows;
+    *keep = room > 0 ? room : 0;
+    return PC_OK;
+}
 struct PatchInfo {
     bool ok;
     int32_t max_bytes, max_halo, max_own;  // largest record, largest halo, most kept blocks

@@ -164,6 +164,7 @@ struct PatchArgs {
     int V, R, n;                // rows, rows per patch, patches
     const PatchDesc *desc;
     const unsigned char *store;
+    int64_t keep;               // records below this offset are copied without the evict-first policy
     int rec_cap, halo_cap;      // largest record (rounded up) and halo: the shared memory's parts
     const float *dsc;           // [V] scalar difference diagonal or -1, new numbers
     const float *dres;          // difference diagonal, original numbers
@@ -195,6 +196,14 @@ struct PatchAhead {
     float4 pi, h[PT_AHEAD];
     float s;
 };
+
+// The record of patch `d` to shared memory (one thread).
+__device__ __forceinline__ void patch_copy(const PatchArgs &a, const PatchDesc &d, unsigned char *s_rec, uint64_t *bar)
+{
+    mbar_arrive_expect_tx(bar, (uint32_t)d.bytes);
+    if (d.offset < a.keep) bulk_g2s_keep(s_rec, a.store + d.offset, (uint32_t)d.bytes, bar);
+    else bulk_g2s(s_rec, a.store + d.offset, (uint32_t)d.bytes, bar);
+}
 
 // The halo's first rows go to `idx` in shared memory without passing through registers
 // (a thread reads back only what it asked for itself).
@@ -242,10 +251,7 @@ static __global__ void __launch_bounds__(PT_ROWS, 4) patch_spmv_kernel(PatchArgs
     __syncthreads();
     int patch = blockIdx.x;  // the grid has at most as many CTAs as there are patches
     PatchDesc d = a.desc[patch], nd = a.desc[min(patch + G, last)];
-    if (t == 0) {
-        mbar_arrive_expect_tx(&bar, (uint32_t)d.bytes);
-        bulk_g2s(s_rec, a.store + d.offset, (uint32_t)d.bytes, &bar);
-    }
+    if (t == 0) patch_copy(a, d, s_rec, &bar);
     patch_ahead_index(a, d, s_idx);
     pdl_wait();
     if (t == 0) s_done = a.sc->done;
@@ -288,10 +294,7 @@ static __global__ void __launch_bounds__(PT_ROWS, 4) patch_spmv_kernel(PatchArgs
         patch_row_shares<1>(s_rec, L, share, PT_ROWS, t >> 5, 0, a0, a1, a2);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the shares precede the next copy
         __syncthreads();  // the record and ps are free
-        if (t == 0 && more) {
-            mbar_arrive_expect_tx(&bar, (uint32_t)nd.bytes);
-            bulk_g2s(s_rec, a.store + nd.offset, (uint32_t)nd.bytes, &bar);
-        }
+        if (t == 0 && more) patch_copy(a, nd, s_rec, &bar);
         // not before the computation: the indices, fetched from the record in DRAM, have
         // arrived by now, and the gathers overlap the record's copy
         if (more) patch_ahead_load(a, patch + G, nd.n_halo, s_idx, cur);

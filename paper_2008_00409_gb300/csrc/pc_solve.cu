@@ -920,6 +920,7 @@ struct SolveCtx {
     int capr = SP_CAPR_WIDE;  // the product's stage width (blocks per row)
     bool patch = false;       // the products read the patch storage, the vectors are in its row order
     int pt_grid = 0, pt_smem = 0, pt_rec = 0, pt_halo = 0;
+    int64_t pt_keep = 0;      // bytes of the records that L2 keeps between products
     bool resident = false;    // the iterations run in pcg_resident_kernel
     int pt_share = 0, pt_split = 0;
     const int32_t *new_of = nullptr;  // the vectors' place of an original row (null: the same)
@@ -1274,6 +1275,7 @@ static pc_status launch_iterations(const SolveCtx &s, float *x, int count)
             y.n = c->pt_n;
             y.desc = static_cast<const PatchDesc *>(c->pt_desc);
             y.store = c->pt_store;
+            y.keep = s.pt_keep;
             y.rec_cap = s.pt_rec;
             y.halo_cap = s.pt_halo;
             y.dsc = c->dsc;
@@ -1493,6 +1495,7 @@ static pc_status try_patch(SolveCtx &s)
         PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, patch_spmv_kernel, PT_ROWS, s.pt_smem));
         if (occ < 3) return PC_OK;
         s.pt_grid = std::min(std::min(c->pt_n, c->num_sms * occ), c->max_red_blocks);
+        PC_TRY(pc_l2_keep(c, c->V, &s.pt_keep));
     }
     s.patch = true;
     s.new_of = c->pt_new;
