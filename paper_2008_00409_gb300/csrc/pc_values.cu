@@ -119,8 +119,8 @@ __device__ __forceinline__ void strain_from_edges(const dfl *e1, const dfl *e2, 
 // first-order form of h f(x_t + h v_t) (Eq. 2-3); since each Hessian row sums to zero,
 // sum_l H_kl v_l is formed as sum_l H_kl (v_l - v_k).
 // Eight consecutive triangles' records are interleaved, quad by quad (tri_quad): lanes that
-// read the same quad of neighbouring triangles share a line (row reduction at 830k rows: 784
-// us with each record a line of its own, 676 interleaved).
+// read the same quad of neighbouring triangles share a line (assembly at 830k rows: 1,095 us
+// with each record a line of its own, 987 interleaved).
 // Bound by DRAM (reads 56 B of rest data per triangle, writes 128 B): 1.65M triangles: 64 us
 // (523 with 256-byte records stored a float at a time).
 #define TE_THREADS 128
@@ -422,7 +422,6 @@ __global__ void contact_eval_kernel(int P, const int32_t *__restrict__ pairs, co
 
 #define RR_ROWS 32                     // rows per CTA
 #define RR_THREADS 128
-#define RR_CAP (RR_ROWS * 18)          // blocks of a tile staged in shared memory
 
 // Contributions to one block (row, col), col != row, from the mesh's elements, in incidence
 // order: the static list of (type, k, l, id) codes that pc_create made for the block
@@ -542,22 +541,23 @@ __device__ __forceinline__ void row_block(const RowArgs &a, int row, int slot, i
 // difference-form diagonals, one thread per row over the row's incident elements; the
 // other blocks go one per thread, over the block's own contribution list, in chunks of 32
 // handed out by a shared counter (warp 0 joins when its rows are done; which warp takes a
-// chunk does not change any sum). Blocks are staged in shared memory and leave as whole
-// lines; a tile with more than RR_CAP blocks writes them directly.
-// Bound by DRAM and L2: 44 B per block written (vals and its column read), about 5
-// contributions of 64..128 B per block read through L1. At 830k rows / 10.9M blocks: before,
-// a warp per row staged every expanded block and each lane compared all of them with
-// its column, 2,825 us; now 676 us, most of it L1 looking up lines for the lanes' 16-byte
-// reads of records (76% of L1's rate before the triangles were interleaved; DRAM 20%). Copying a tile's records to shared
-// memory first was slower (1,086 -> 1,525 us for the whole assembly).
-__global__ void __launch_bounds__(RR_THREADS) row_reduce_kernel(RowArgs a)
+// chunk does not change any sum).
+// Bound by L1 and L2: 44 B per block written (vals and its column read), about 5
+// contributions of 64..128 B per block read through L1, a line looked up for nearly every
+// lane. So L1 gets all of an SM's memory: blocks are written where they belong (a warp's 32
+// blocks are 1,152 consecutive bytes), and 56 registers allow nine CTAs per SM. At 830k rows /
+// 10.9M blocks, the whole assembly: 827 us; 987 with the blocks staged in shared memory for
+// whole-line stores (879 unstaged at 64 registers, 891 at 40). Also slower: records copied to
+// shared memory first, a thread per row that adds each element to its blocks in shared memory,
+// CTAs of 256 threads (921). A warp per row that staged every expanded block, each lane
+// comparing all of them with its column, took 2,825 us for this kernel alone.
+__global__ void __launch_bounds__(RR_THREADS, 9) row_reduce_kernel(RowArgs a)
 {
-    __shared__ float s_blk[RR_CAP * 9];
     __shared__ int s_rp[RR_ROWS + 1], s_sp[RR_ROWS + 1], s_cp[RR_ROWS + 1];
     __shared__ int s_next;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r0 = blockIdx.x * RR_ROWS, nr = min(RR_ROWS, a.V - r0);
-    for (int i = threadIdx.x; i <= nr; i += RR_THREADS) {
+    for (int i = threadIdx.x; i <= nr; i += blockDim.x) {
         s_rp[i] = a.rp[r0 + i];
         s_sp[i] = a.srp[r0 + i];
         s_cp[i] = a.cinc_ptr[r0 + i];
@@ -565,7 +565,6 @@ __global__ void __launch_bounds__(RR_THREADS) row_reduce_kernel(RowArgs a)
     if (threadIdx.x == 0) s_next = 0;
     __syncthreads();
     const int b0 = s_rp[0], nblk = s_rp[nr] - b0;
-    const bool staged = nblk <= RR_CAP;
 
     if (warp == 0 && lane < nr) {
         const int row = r0 + lane;
@@ -682,7 +681,7 @@ __global__ void __launch_bounds__(RR_THREADS) row_reduce_kernel(RowArgs a)
             B[4] += mA;
             B[8] += mA;
         }
-        float *dst = staged ? s_blk + 9 * (ds - b0) : a.vals + 9ll * ds;
+        float *dst = a.vals + 9ll * ds;
 #pragma unroll
         for (int q = 0; q < 9; ++q) dst[q] = B[q];
     }
@@ -709,14 +708,10 @@ __global__ void __launch_bounds__(RR_THREADS) row_reduce_kernel(RowArgs a)
         } else {
             row_block(a, row, slot, col, s_rp[r], s_rp[r + 1], s_sp[r], s_sp[r + 1], s_cp[r], s_cp[r + 1], acc);
         }
-        float *dst = staged ? s_blk + 9 * i : a.vals + 9ll * slot;
+        float *dst = a.vals + 9ll * slot;
 #pragma unroll
         for (int q = 0; q < 9; ++q) dst[q] = acc[q];
     }
-    if (!staged) return;
-    __syncthreads();
-    float *o = a.vals + 9ll * b0;
-    for (int i = threadIdx.x; i < 9 * nblk; i += RR_THREADS) o[i] = s_blk[i];
 }
 
 extern "C" pc_status pc_assemble_values(pc_ctx *ctx, const pc_bsr *A, const float *x, const float *v,
