@@ -159,7 +159,7 @@ def test_pattern_and_values_with_many_contacts_at_a_vertex(pc, nx, ny, star):
 
 
 # the edges of a tile of 32 rows; a vertex with many elements, and an element that meets a
-# vertex twice (a tile with more blocks than its staging holds: the star of 300 above)
+# vertex twice (a row of hundreds of blocks: the star of 300 above)
 @pytest.mark.parametrize("wl", [_grid(5, 3), _grid(16, 1 + 1), _grid(11, 3), _grid(17, 3), _fan(8), _fan(40)],
                          ids=["15", "32", "33", "51", "fan8", "fan40"])
 def test_values_at_tile_edges_match_oracle(pc, wl):
@@ -181,8 +181,8 @@ def test_values_at_tile_edges_match_oracle(pc, wl):
     cl.close()
 
 
-# a vertex shared by many separate fans of eight triangles: more blocks in a tile of 32 rows
-# than its staging holds; with contacts between the fans and without
+# a vertex shared by many separate fans of eight triangles: a row of hundreds of blocks, each
+# with few contributions; with contacts between the fans and without
 @pytest.mark.parametrize("fans,contacts", [(59, False), (60, False), (60, True), (140, False), (140, True)])
 def test_values_of_a_vertex_with_many_blocks(pc, fans, contacts):
     a = 2.0 * np.pi * np.arange(8) / 8
