@@ -41,10 +41,9 @@ FALLBACK_HBM_GBS = 6800.0
 # works out of the shared memory of the 16 SMs of one thread-block cluster
 SMEM_BYTES_PER_CLK = 128
 CLUSTER_SMS = 16
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the PCG SpMV,
-# from one ncu capture of the current kernel on that workload (mean of 3 launches).
-# ncu DRAM read + write bytes per launch of the PCG product, by (workload, storage)
-SPMV_DRAM_BYTES = {}  # (workload, storage) -> DRAM bytes per product in steady state, where measured
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the PCG product in
+# steady state, by (workload, storage), where the current kernel has been profiled
+SPMV_DRAM_BYTES = {}
 
 
 def parse():
