@@ -1025,8 +1025,7 @@ static bool cl_layout(int V, int C, bool diff, bool block, size_t smax, int64_t 
     const int64_t cap = (int64_t)((smax - o) / 48);
     if (cap < 8 || share > cap) return false;
     a->o_blk = (uint32_t)o;
-    *smem = o + 48 * (size_t)cap;
-    if (*smem > smax) return false;
+    *smem = smax;  // not the few bytes less: the kernel's limit is the same for every context of the process
     a->Rc = Rc;
     a->Vw = Vw;
     a->cap = (int)cap;

@@ -740,6 +740,24 @@ static pc_status spmv_set_smem()
     return PC_OK;
 }
 
+// The kernels that read patch records take a solve's own size at the launch, and their limit
+// is always all that a CTA can have: a limit belongs to the kernel in the process, and other
+// contexts' solves, in other threads, may be between their launches.
+static pc_status patch_set_smem(const pc_ctx *c)
+{
+    int most = 0;
+    PC_CUDA_TRY(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+    const void *kernels[] = {(const void *)patch_spmv_kernel,
+                             (const void *)pcg_resident_kernel<2, false>, (const void *)pcg_resident_kernel<2, true>,
+                             (const void *)pcg_resident_kernel<4, false>, (const void *)pcg_resident_kernel<4, true>};
+    for (const void *k : kernels) {
+        cudaFuncAttributes fa;
+        PC_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
+        PC_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes));
+    }
+    return PC_OK;
+}
+
 // The largest tile (blocks in SP_ROWS consecutive rows) of a BSR pattern, into *out
 // (zeroed by the caller) with one atomicMax per warp.
 __global__ void tile_max_kernel(int V, const int32_t *__restrict__ rp, long long *out)
@@ -793,6 +811,7 @@ pc_status pc_solver_alloc(pc_ctx *c)
     PC_CUDA_TRY(cudaMemset(c->sc, 0, sizeof(pc_scalars)));
     PC_CUDA_TRY(cudaMallocHost(&c->sc_host, sizeof(pc_scalars)));
     PC_TRY(spmv_set_smem());
+    PC_TRY(patch_set_smem(c));
     PC_CUDA_TRY(cudaFuncSetAttribute(spmv_sym_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SY_SMEM_BYTES));
     PC_CUDA_TRY(cudaFuncSetAttribute(spmv_sym_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SY_SMEM_BYTES));
     if (c->A_cap > 0) {  // symmetric storage for systems up to the step-system capacity
@@ -1483,14 +1502,12 @@ static pc_status try_patch(SolveCtx &s)
         cudaFuncAttributes fa;
         PC_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
         if (!coop || s.pt_smem + (int)fa.sharedSizeBytes > most) return PC_OK;
-        PC_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, s.pt_smem));
         PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, s.pt_split * c->pt_rows, s.pt_smem));
         if (occ < 1) return PC_OK;
         s.resident = true;
     } else {
         s.pt_smem = s.pt_rec + 12 * (c->pt_rows + pi.max_halo);
         if (s.pt_smem > limit / 3) return PC_OK;
-        PC_CUDA_TRY(cudaFuncSetAttribute(patch_spmv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, s.pt_smem));
         int occ = 0;
         PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, patch_spmv_kernel, PT_ROWS, s.pt_smem));
         if (occ < 3) return PC_OK;
