@@ -240,6 +240,7 @@ struct PxArgs {
     const int32_t *first;  // null: more cells than the table holds
     PxGrid g;
     float inv, delta;
+    float round;           // how far outside its box the triangles' rounding can put a closest point
     const int32_t *erp, *ecol;
     int32_t *cnt;          // [V + 1] pairs of each vertex
     uint32_t *hits;        // [PX_HITS][V] their first triangles
@@ -326,9 +327,10 @@ __global__ void __launch_bounds__(128) px_pairs_kernel(PxArgs a)
         pc_set_err(a.err, PC_DERR_INDEX);
         return;
     }
-    // the box already exceeds delta by a hundredth; this far outside it, no rounding of the
-    // coordinates (16 units in their last place) can bring the computed distance below delta
-    const float slack = 0.05f * a.delta + 1e-6f * (fabsf(xp.x) + fabsf(xp.y) + fabsf(xp.z));
+    // the box already exceeds delta by a hundredth; this far outside it, no rounding can bring
+    // the computed distance below delta: of p's coordinates (16 units in their last place), or of
+    // the closest point a + wb (b - a) + wc (c - a) (6 half units of the mesh's largest one)
+    const float slack = 0.05f * a.delta + 1e-6f * (fabsf(xp.x) + fabsf(xp.y) + fabsf(xp.z)) + a.round;
     int64_t lo, hi;
     px_list(a, px_number(a.g, ix, iy, iz), lo, hi);
     for (int64_t i = lo; i < hi; i += 32) {
@@ -445,6 +447,7 @@ extern "C" pc_status pc_proximity_query(pc_ctx *ctx, const float *x, float delta
     a.g = g;
     a.inv = 1.0f / cs;
     a.delta = delta;
+    for (float v : corner) a.round = fmaxf(a.round, 1e-6f * fabsf(v));
     a.erp = ctx->erp;
     a.ecol = ctx->ecol;
     a.cnt = ctx->px_vcnt;
