@@ -28,6 +28,7 @@
 // triangle, Ericson 2005, Sec. 5.1.5) and the test d^2 < delta^2 are decided in FP32
 // with one rounding per operation in a fixed order (the _rn intrinsics keep the compiler
 // from contracting into fused multiply-adds), so the pairs are reproducible bit for bit.
+#include <algorithm>
 #include <cstring>
 
 #include "pc_internal.cuh"
@@ -39,7 +40,8 @@
 // The numbered cells: first coordinates, extents (nx, ny), and how many there are.
 struct PxGrid {
     int x0, y0, z0;
-    int64_t nx, ny, n;
+    int64_t nx, ny;
+    uint64_t n;  // up to 2^63
 };
 
 __device__ __forceinline__ float3 px_ld(const float *x, int i)
@@ -114,7 +116,7 @@ __device__ __forceinline__ int64_t px_number(const PxGrid &g, int ix, int iy, in
     const int64_t x = (int64_t)ix - g.x0, y = (int64_t)iy - g.y0, z = (int64_t)iz - g.z0;
     if (x < 0 || y < 0 || z < 0 || x >= g.nx || y >= g.ny) return -1;
     const int64_t c = (z * g.ny + y) * g.nx + x;
-    return c < g.n ? c : -1;
+    return (uint64_t)c < g.n ? c : -1;
 }
 
 // A float as an unsigned integer of the same order, and back (host side).
@@ -422,12 +424,12 @@ extern "C" pc_status pc_proximity_query(pc_ctx *ctx, const float *x, float delta
             g.x0 = c[0];
             g.y0 = c[1];
             g.z0 = c[2];
-            g.nx = (int64_t)c[3] - c[0] + 1;  // each extent at most 2^21: 63 bits for their product
+            g.nx = (int64_t)c[3] - c[0] + 1;  // each extent at most 2^21: their product at most 2^63
             g.ny = (int64_t)c[4] - c[1] + 1;
-            g.n = g.nx * g.ny * ((int64_t)c[5] - c[2] + 1);
+            g.n = (uint64_t)(g.nx * g.ny) * (uint64_t)((int64_t)c[5] - c[2] + 1);
             PC_LAUNCH(ctx, px_emit_cells_kernel, pc_blocks(T, 256), 256, 0, st, T, ctx->px_box, inv, g, ctx->px_off,
                       cap_k, ctx->px_keys, ctx->px_vals);
-            PC_TRY(pc_radix_sort(ctx, ctx->px_keys, ctx->px_vals, K, pc_bits_for(g.n), st));
+            PC_TRY(pc_radix_sort(ctx, ctx->px_keys, ctx->px_vals, K, pc_bits_for((int64_t)std::min<uint64_t>(g.n, INT64_MAX)), st));
             break;
         }
         if (attempt >= 4) return PC_ERR_CAPACITY;
@@ -443,7 +445,7 @@ extern "C" pc_status pc_proximity_query(pc_ctx *ctx, const float *x, float delta
     a.K = K;
     // a list of its own for every cell where the table has room (sheets do: a few triangles
     // per cell), else binary searches in the sorted keys
-    a.first = g.n <= ctx->px_first_cap ? ctx->px_first : nullptr;
+    a.first = g.n <= (uint64_t)ctx->px_first_cap ? ctx->px_first : nullptr;
     a.g = g;
     a.inv = 1.0f / cs;
     a.delta = delta;
@@ -457,7 +459,7 @@ extern "C" pc_status pc_proximity_query(pc_ctx *ctx, const float *x, float delta
     a.w = w;
     a.err = ctx->d_err;
     if (a.first)
-        PC_LAUNCH(ctx, px_first_kernel, pc_blocks(K + 1, 256), 256, 0, st, K, ctx->px_keys, g.n, ctx->px_first);
+        PC_LAUNCH(ctx, px_first_kernel, pc_blocks(K + 1, 256), 256, 0, st, K, ctx->px_keys, (int64_t)g.n, ctx->px_first);
     PC_LAUNCH(ctx, px_pairs_kernel<false>, pc_blocks(V + 1ll, 128), 128, 0, st, a);
     PC_TRY(pc_exclusive_scan(ctx, ctx->px_vcnt, ctx->px_voff, V, st));
     PC_CUDA_TRY(cudaMemcpyAsync(ctx->h_count, ctx->px_voff + V, sizeof(int32_t), cudaMemcpyDeviceToHost, st));

@@ -70,3 +70,26 @@ def test_long_triangles_with_a_corner_at_a_vertex_near_the_origin(pc, seed, corn
     got_p, got_w = _query(pc, x, tris, delta)
     np.testing.assert_array_equal(got_p, want_p)
     np.testing.assert_array_equal(got_w.view(np.uint32), want_w.view(np.uint32))
+
+
+def test_triangles_at_both_ends_of_the_cell_range(pc):
+    """Cells are of one box's size and their coordinates reach from -2^20 to 2^20 - 1: triangles in
+    both of these along every axis, and a pair at each end."""
+    delta, e = 0.125, 0.75
+    tri = np.array([[0.0, 0.0, 0.0], [e, 0.0, 0.0], [0.0, e, 0.0]])
+    # at the origin: the largest grown box, whose edge is the cell; there 2 pads are exact
+    cell = np.float32((np.float32(e) + 2 * np.float32(delta * np.float32(1.01))) * np.float32(1.001))
+    end = (np.floor((2.0 ** 20 - 0.5) * cell * 8) / 8)  # whole eighths: units in the last place there
+    x = []
+    for base in (np.zeros(3), [end - 1.0, end - 1.0, end - 0.25], np.full(3, -end + 0.25)):
+        x += [tri + base, tri + base + [0.25, 0.25, 0.0]]
+    x = np.concatenate(x).astype(np.float32)
+    pad = np.float32(np.float32(delta) * np.float32(1.01))
+    lo, hi = np.floor((x.min(0) - pad) / cell), np.floor((x.max(0) + pad) / cell)
+    assert (hi == 2 ** 20 - 1).all() and (lo == -2 ** 20).all()
+    tris = np.arange(len(x)).reshape(-1, 3)
+    want_p, want_w = _brute(x, tris, delta)
+    assert set(want_p[:, 0] // 6) == {0, 1, 2}
+    got_p, got_w = _query(pc, x, tris, delta)
+    np.testing.assert_array_equal(got_p, want_p)
+    np.testing.assert_array_equal(got_w.view(np.uint32), want_w.view(np.uint32))
