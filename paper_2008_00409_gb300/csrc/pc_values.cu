@@ -10,6 +10,8 @@
 // the Gram difference of the current and rest edges evaluated in double-float (pairs of
 // FP32 values, exact TwoSum / fma-based TwoProduct), so the strain keeps FP32 relative
 // accuracy; everything else is plain FP32.
+#include <float.h>
+
 #include "pc_internal.cuh"
 
 // ------------------------------------------------------------------------- double-float
@@ -333,13 +335,14 @@ __device__ __forceinline__ float hinge_angle_grad(float3 a1, float3 a2, float3 a
 // contribution h f_k - q_k (q . v) is q_k times one scalar w, because f_k is parallel to
 // grad_k too: h f_k = -h (2 kb c_h) (theta - theta_rest) grad_k. Record: four float4 (q_k, w),
 // 64 bytes, instead of 12 contributions and 12 gradients. The gradient sums to zero over
-// the four vertices, so q . v uses velocities relative to edge0. Bound by DRAM (reads 24 B
-// of rest data and writes 64 B per hinge); 2.48M hinges: 60 us (247 with 96-byte records).
+// the four vertices, so q . v uses velocities relative to edge0. hb = h + beta, hk = h hb,
+// ih = h / hk. Bound by DRAM (reads 24 B of rest data and writes 64 B per hinge); 2.48M hinges:
+// 60 us (247 with 96-byte records).
 __global__ void __launch_bounds__(128) hinge_eval_kernel(int H, const int32_t *__restrict__ hinge,
                                                          const float *__restrict__ x, const float *__restrict__ v,
                                                          const float *__restrict__ hcoef,
-                                                         const float *__restrict__ hrest, float h, float hk,
-                                                         float *__restrict__ out)
+                                                         const float *__restrict__ hrest, float h, float hb, float hk,
+                                                         float ih, float *__restrict__ out)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= H) return;
@@ -353,13 +356,15 @@ __global__ void __launch_bounds__(128) hinge_eval_kernel(int H, const int32_t *_
     // positions relative to edge0
     float3 a1 = sub(X[0], X[2]), a2 = sub(X[1], X[2]), a4 = sub(X[3], X[2]);
     float th = hinge_angle_grad(a1, a2, a4, grad);
-    float sc = sqrtf(hk * kc);
+    const float hkc = hk * kc;
+    // (the force needs sc where its square, which only the Hessian has, leaves FP32's range)
+    const float sc = hkc > 1e-30f ? sqrtf(hkc) : sqrtf(h * kc) * sqrtf(hb);
     float3 q[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) q[k] = mul(sc, grad[k]);
     float qv = dot(q[0], sub(W[0], W[2])) + dot(q[1], sub(W[1], W[2])) + dot(q[3], sub(W[3], W[2]));
     // h f_k = -h kc (theta - rest) grad_k = -(h / hk) sc (theta - rest) q_k
-    const float w = -(h / hk) * sc * (th - hrest[i]) - qv;
+    const float w = -ih * sc * (th - hrest[i]) - qv;
     float4 *o = reinterpret_cast<float4 *>(out) + (int64_t)(PC_HINGE_STRIDE / 4) * i;
 #pragma unroll
     for (int k = 0; k < 4; ++k) o[k] = make_float4(q[k].x, q[k].y, q[k].z, w);
@@ -727,14 +732,14 @@ extern "C" pc_status pc_assemble_values(pc_ctx *ctx, const pc_bsr *A, const floa
     const int V = ctx->V, T = ctx->T, H = ctx->H;
     // Rayleigh damping: element Hessians enter A as h (h + beta) K, the mass as
     // (1 + h alpha) M (beta = alpha = 0: h^2 K and M)
-    const float hk = h * (h + ctx->mat.damp_stiff);
+    const float hb = h + ctx->mat.damp_stiff, hk = h * hb, ih = hk >= FLT_MIN ? h / hk : fminf(1.0f / hb, FLT_MAX);
     const float md = 1.0f + h * ctx->mat.damp_mass, ha = h * ctx->mat.damp_mass;
     if (T > 0)
         PC_LAUNCH(ctx, tri_eval_kernel, pc_blocks(T, TE_THREADS), TE_THREADS, 0, st, T, ctx->tri, x, v, ctx->tri_dmi, ctx->tri_area,
                   ctx->tri_rgram, ctx->mu, ctx->lam, h, hk, ctx->tri_buf);
     if (H > 0)
-        PC_LAUNCH(ctx, hinge_eval_kernel, pc_blocks(H, 128), 128, 0, st, H, ctx->hinge, x, v, ctx->hcoef, ctx->hrest, h,
-                  hk, ctx->hinge_buf);
+        PC_LAUNCH(ctx, hinge_eval_kernel, pc_blocks(H, 128), 128, 0, st, H, ctx->hinge, x, v, ctx->hcoef, ctx->hrest, h, hb,
+                  hk, ih, ctx->hinge_buf);
     if (P > 0)
         PC_LAUNCH(ctx, contact_eval_kernel, pc_blocks(P, 128), 128, 0, st, P, contacts->pairs, contacts->w, x, v,
                   ctx->mat.k_contact, h, hk, ctx->mat.contact_thickness, ctx->cont_buf);
