@@ -546,7 +546,7 @@ static pc_status create_impl(pc_ctx *c, const int32_t *tris, const float *rest, 
     PC_TRY(dalloc(&c->cinc, 4 * P + 1));
     PC_TRY(dalloc(&c->cinc_ptr, V + 1ll));
     PC_TRY(dalloc(&c->row_cnt, 2ll * V + 2));
-    PC_TRY(dalloc(&c->tri_buf, (int64_t)PC_TRI_STRIDE * ((T + 7) & ~7)));
+    PC_TRY(dalloc(&c->tri_buf, (int64_t)(PC_TRI_STRIDE / 4) * ((T + 7) & ~7)));  // float4
     PC_TRY(dalloc(&c->hinge_buf, (int64_t)PC_HINGE_STRIDE * c->H));
     PC_TRY(dalloc(&c->cont_buf, (int64_t)PC_CONTACT_STRIDE * P));
     PC_TRY(dalloc(&c->h_pairs, 4 * P));
