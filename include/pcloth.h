@@ -28,7 +28,9 @@
  *    synchronize the stream before returning.
  *  - A context (pc_ctx) holds one mesh's rest state and all scratch memory of the
  *    assembly and solve calls, allocated once by pc_create: about 5.2 KB per vertex of a
- *    sheet (13 blocks per row). The calls that allocate
+ *    sheet (13 blocks per row) and 1.4 KB per contact of max_contacts. Of it the patch records
+ *    (PC_STORAGE_OFFDIAG, at most 620 bytes per vertex) are left out when there is no memory
+ *    for them. The calls that allocate
  *    device memory are: pc_create; pc_mlp_create (training state); pc_set_warm_mlp
  *    (the context's feature and guess buffers, on the first attach); pc_step_batched
  *    (the CUDA graph it instantiates on its first call for a system shape). pc_mlp_infer

@@ -313,8 +313,6 @@ pc_status pc_warm_guess(pc_ctx *c, const pc_bsr *A, const float *v, float h, int
                         int32_t *guess, double *guess_res, double *guess_energy, double *guess_coef,
                         double *combo_energy, cudaStream_t st);
 void pc_mlp_ctx_free(pc_ctx *c);
-// Patch storage of the system being solved (pc_patch.cu): allocation and row order, and the
-// records of one matrix (ok = false: the matrix does not suit it and nothing is usable).
 // Bytes of a matrix stream that L2 can hold from one product of an iterative solve to the
 // next beside the solve's vectors (about 90 bytes per row): the stream's first `*keep` bytes
 // are copied with the ordinary policy, the rest evict-first. What every SM reads takes room
@@ -330,11 +328,14 @@ inline pc_status pc_l2_keep(const pc_ctx *c, int64_t rows, int64_t *keep)
     *keep = room > 0 ? room : 0;
     return PC_OK;
 }
+// Patch storage of the system being solved (pc_patch.cu): allocation and row order, and the
+// records of one matrix (ok = false: the matrix does not suit it and nothing is usable).
 struct PatchInfo {
     bool ok;
     int32_t max_bytes, max_halo, max_own;  // largest record, largest halo, most kept blocks
 };
 pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st);
+pc_status pc_patch_limit(const pc_ctx *c, bool resident, int *bytes);
 pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, PatchInfo *out, cudaStream_t st);
 // The whole solve in one thread-block cluster (pc_cluster.cu). Runs when the system fits
 // the cluster's shared memory (*ran = true, returns the solve's status); otherwise

@@ -111,6 +111,16 @@ __global__ void order_kernel(int V, const uint32_t *__restrict__ vals, int32_t *
     new_of[vals[i]] = i;
 }
 
+// The largest record that a solve can use: all the shared memory a CTA can have where the
+// record stays in it, a third of an SM's where it is streamed (three CTAs beside each other).
+pc_status pc_patch_limit(const pc_ctx *c, bool resident, int *bytes)
+{
+    PC_CUDA_TRY(cudaDeviceGetAttribute(bytes, resident ? cudaDevAttrMaxSharedMemoryPerBlockOptin
+                                                       : cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device));
+    if (!resident) *bytes /= 3;
+    return PC_OK;
+}
+
 pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
 {
     const int V = c->V;
@@ -119,8 +129,13 @@ pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
     const int per_sm = ((V + c->num_sms - 1) / c->num_sms + 31) / 32 * 32;
     c->pt_rows = per_sm <= PT_RESIDENT_ROWS ? per_sm : PT_ROWS;
     c->pt_n = (V + c->pt_rows - 1) / c->pt_rows;
-    // kept blocks at most all of them; entries 4 bytes each, twice that with the slices' padding
-    c->pt_cap = 48 * c->A_cap + (int64_t)c->pt_n * 1024;
+    const bool resident = c->pt_n <= c->num_sms;
+    // kept blocks at most all of them, entries 4 bytes each, twice that with the slices' padding;
+    // and never more than records that the solves can use (pc_patch_limit), however many
+    // contacts the context has room for
+    int limit = 0;
+    PC_TRY(pc_patch_limit(c, resident, &limit));
+    c->pt_cap = std::min(48 * c->A_cap + (int64_t)c->pt_n * 1024, (int64_t)c->pt_n * pt_up16(limit));
     // the arrays, in one allocation (pc_destroy frees it through pt_old)
     size_t at = 0;
     auto take = [&](size_t bytes) {
@@ -128,15 +143,19 @@ pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
         at += (bytes + 255) / 256 * 256;
         return o;
     };
-    const bool resident = c->pt_n <= c->num_sms;
     const size_t o_old = take(sizeof(int32_t) * (size_t)V), o_new = take(sizeof(int32_t) * (size_t)V);
     const size_t o_desc = take(sizeof(PatchDesc) * (size_t)c->pt_n), o_cnt = take((size_t)c->pt_n * c->pt_rows);
     const size_t o_named = take((size_t)V), o_size = take(sizeof(int32_t) * 2 * (c->pt_n + 1ll)), o_info = take(32);
     const size_t o_z = take(resident ? 4 * sizeof(uint64_t) * (size_t)V : 0);
     const size_t o_slots = take(resident ? sizeof(uint64_t) * (12 * (size_t)c->pt_n * c->pt_n + 1) : 0);
     const size_t o_store = take((size_t)c->pt_cap);
+    // without room for it the context has no order (pt_store stays null: the solves stream the
+    // BSR rows)
     unsigned char *base = nullptr;
-    PC_CUDA_TRY(cudaMalloc(&base, at));
+    if (cudaMalloc(&base, at) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return PC_OK;
+    }
     c->pt_old = reinterpret_cast<int32_t *>(base + o_old);
     c->pt_new = reinterpret_cast<int32_t *>(base + o_new);
     c->pt_desc = base + o_desc;
@@ -154,7 +173,10 @@ pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
     uint32_t *vals = c->px_vals;
     if (own) {
         keys = nullptr;
-        PC_CUDA_TRY(cudaMalloc(&keys, (sizeof(uint64_t) + sizeof(uint32_t)) * (size_t)V));
+        if (cudaMalloc(&keys, (sizeof(uint64_t) + sizeof(uint32_t)) * (size_t)V) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return PC_OK;
+        }
         vals = reinterpret_cast<uint32_t *>(keys + V);
     }
     float *box = reinterpret_cast<float *>(c->pt_info);
@@ -191,7 +213,7 @@ pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
         if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) s = PC_ERR_CUDA;
     } while (0);
     if (own) cudaFree(keys);
-    if (s == PC_OK) c->pt_store = base + o_store;  // (null: no order, the solves stream the BSR rows)
+    if (s == PC_OK) c->pt_store = base + o_store;
     return s;
 }
 

@@ -1485,29 +1485,28 @@ static pc_status try_patch(SolveCtx &s)
     PC_TRY(pc_patch_build(c, s.A, s.vals, &pi, s.st));
     if (!pi.ok) return PC_OK;
     int limit = 0;
-    PC_CUDA_TRY(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device));
+    PC_TRY(pc_patch_limit(c, c->pt_slots != nullptr, &limit));
     s.pt_halo = pi.max_halo;
     s.pt_rec = (pi.max_bytes + 127) / 128 * 128;
     if (c->pt_slots) {
         // one CTA per patch for the whole solve, if everything fits (the fused update's stop
         // tests and direction step; fuse = 0 keeps the separate kernels)
         if (!s.fuse || c->pt_n > c->num_sms) return PC_OK;
-        int coop = 0, most = 0, occ = 0;
+        int coop = 0, occ = 0;
         PC_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
-        PC_CUDA_TRY(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
         s.pt_split = c->pt_rows <= 256 ? 4 : 2;
         s.pt_share = pi.max_own + 1;
         s.pt_smem = s.pt_rec + 16 * s.pt_share + 12 * (c->pt_rows + pi.max_halo) + 12 * (s.pt_split - 1) * c->pt_rows;
         const void *k = resident_kernel(s);
         cudaFuncAttributes fa;
         PC_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
-        if (!coop || s.pt_smem + (int)fa.sharedSizeBytes > most) return PC_OK;
+        if (!coop || s.pt_smem + (int)fa.sharedSizeBytes > limit) return PC_OK;
         PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, s.pt_split * c->pt_rows, s.pt_smem));
         if (occ < 1) return PC_OK;
         s.resident = true;
     } else {
         s.pt_smem = s.pt_rec + 12 * (c->pt_rows + pi.max_halo);
-        if (s.pt_smem > limit / 3) return PC_OK;
+        if (s.pt_smem > limit) return PC_OK;
         int occ = 0;
         PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, patch_spmv_kernel, PT_ROWS, s.pt_smem));
         if (occ < 3) return PC_OK;
