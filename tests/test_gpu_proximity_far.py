@@ -93,3 +93,23 @@ def test_triangles_at_both_ends_of_the_cell_range(pc):
     got_p, got_w = _query(pc, x, tris, delta)
     np.testing.assert_array_equal(got_p, want_p)
     np.testing.assert_array_equal(got_w.view(np.uint32), want_w.view(np.uint32))
+
+
+def test_time_does_not_hang_on_empty_cells(pc):
+    """Two sheets with hundreds of thousands of empty cells between them (inside the cell table) take
+    no longer than the same sheets half a millimetre apart and half as much again."""
+    took = []
+    for gap in (5e-4, 0.1):
+        wl = wk.stacked_sheets(301, 2, seed=4, gap=gap, contact_frac=0.0)
+        cl = pc.Cloth(wl, max_contacts=4 * wl.V)
+        times = []
+        for _ in range(12):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            cl.proximity(5.5e-4)
+            e[1].record()
+            torch.cuda.synchronize()
+            times.append(e[0].elapsed_time(e[1]))
+        took.append(float(np.median(times[2:])))
+        cl.close()
+    assert took[1] <= 1.5 * took[0], took
