@@ -637,18 +637,20 @@ extern "C" pc_status pc_get_rest(const pc_ctx *ctx, int32_t *hinges, float *mass
 //
 // Contacts by row. Each pair has one entry (local vertex k, pair id) in the rows of its four
 // vertices. Integer counts place the entries into their rows' buckets (the order within a
-// bucket does not matter yet), and one thread per row then sorts its bucket by pair id and
-// lists its new columns in order: everything downstream depends only on the sets, so the
-// pattern stays bit-exact. Bound by launches and L2 latency: 4 x 16 B per pair and a few
-// bytes per row. Two key sorts of 6 and 4 entries per pair (5 + 3 passes of three kernels and
-// two scans) did this before: 0.47 of 0.6 ms at 830k rows / 41k pairs, 145 of 285 us at
-// 4,096 rows / 82 pairs. A row of more than PC_BUCKET contacts (its thread's sort is
-// quadratic) sends the whole step to that path, which remains for it.
-#define PC_BUCKET 64
+// bucket does not matter yet), and each row then sorts its bucket by pair id and lists its new
+// columns in order: everything downstream depends only on the sets, so the pattern stays
+// bit-exact. A row of a few contacts is one thread's (insertion), a fuller one its warp's (a
+// bitonic sort), both in place: shared memory for the warps' sorts took L1 from the threads (2 KB
+// per warp: 830k rows of 16 contacts 989 -> 1,192 us) and gained the warps nothing. Bound by
+// launches and L2 latency: 4 x 16 B per pair and a few bytes per row. Two key sorts of 6 and 4
+// entries per pair (5 + 3 passes of three kernels and two scans) did this before: 0.47 of 0.6 ms
+// at 830k rows / 41k pairs, 145 of 285 us at 4,096 rows / 82 pairs. A row of more than PC_BUCKET
+// contacts, which its warp alone would take long to sort, sends the whole step to that path.
+#define PC_BUCKET 1024
 
 // Validates the pairs, counts the entries of each row and each entry's arrival number.
 __global__ void contact_count_kernel(int P, int V, const int32_t *__restrict__ pairs, int32_t *cnt, int32_t *rank,
-                                     uint32_t *err)
+                                     int32_t *heavy, uint32_t *err)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P) return;
@@ -664,7 +666,11 @@ __global__ void contact_count_kernel(int P, int V, const int32_t *__restrict__ p
     } else if (v[0] == v[1] || v[0] == v[2] || v[0] == v[3] || v[1] == v[2] || v[1] == v[3] || v[2] == v[3]) {
         pc_set_err(err, PC_DERR_PAIR);
     }
-    for (int k = 0; k < 4; ++k) rank[4ll * i + k] = atomicAdd(cnt + v[k], 1);
+    for (int k = 0; k < 4; ++k) {
+        const int at = atomicAdd(cnt + v[k], 1);
+        rank[4ll * i + k] = at;
+        if (at >= PC_BUCKET) *heavy = 1;
+    }
 }
 
 __global__ void contact_place_kernel(int P, int V, const int32_t *__restrict__ pairs, const int32_t *__restrict__ ptr,
@@ -679,62 +685,134 @@ __global__ void contact_place_kernel(int P, int V, const int32_t *__restrict__ p
     cinc[ptr[v] + rank[e]] = pc_ref(PC_REF_CONTACT, k, i);
 }
 
-// One thread per row: its entries in ascending pair order (as placed in incidence order by
-// vertex), and its new columns (partners absent from the static row), ascending and without
-// repeats, at newcol[3 ptr[r] ...] (an entry brings at most three). More than PC_BUCKET
-// entries: *heavy is set.
-__global__ void row_contacts_kernel(int V, const int32_t *__restrict__ ptr, uint32_t *cinc,
-                                    const int32_t *__restrict__ pairs, const int32_t *__restrict__ srp,
-                                    const int32_t *__restrict__ scol, int32_t *newcol, int32_t *nnew, int32_t *heavy)
+// Ascending sort by one warp: a bitonic network whose merges all run upwards, so that the places
+// past n (which count as largest) are never touched.
+template <typename T>
+__device__ void warp_sort(T *a, int n, int lane)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= V) return;
-    const int c0 = ptr[r], n = ptr[r + 1] - c0;
-    int m = 0;
-    if (n > PC_BUCKET) {
-        *heavy = 1;
-    } else if (n > 0) {
-        uint32_t *b = cinc + c0;
-        for (int i = 1; i < n; ++i) {
-            const uint32_t x = b[i];
-            int j = i - 1;
-            for (; j >= 0 && pc_ref_id(b[j]) > pc_ref_id(x); --j) b[j + 1] = b[j];
-            b[j + 1] = x;
-        }
-        int32_t *o = newcol + 3ll * c0;
-        const int s0 = srp[r], s1 = srp[r + 1];
-        for (int i = 0; i < n; ++i) {
-            const uint32_t ref = b[i], k = pc_ref_local(ref);
-            const int32_t *pv = pairs + 4ll * pc_ref_id(ref);
-            const int first = k == 0 ? 1 : 0, last = k == 0 ? 3 : 0;  // p couples with a, b, c; they with p
-            for (int l = first; l <= last; ++l) {
-                const int c = pv[l];
-                int lo = s0, hi = s1;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (scol[mid] < c) lo = mid + 1; else hi = mid;
+    for (int k = 2; k < 2 * n; k <<= 1)
+        for (int s = k >> 1; s > 0; s >>= 1) {
+            for (int t = lane;; t += 32) {
+                const int i = 2 * s * (t / s) + t % s;
+                if (i >= n) break;
+                const int j = s == k >> 1 ? i ^ (k - 1) : i + s;  // the first step of a merge mirrors
+                if (j < n && a[i] > a[j]) {
+                    const T x = a[i];
+                    a[i] = a[j];
+                    a[j] = x;
                 }
-                if (lo < s1 && scol[lo] == c) continue;
-                int j = m - 1;
-                while (j >= 0 && o[j] > c) --j;
-                if (j >= 0 && o[j] == c) continue;
-                for (int q = m - 1; q > j; --q) o[q + 1] = o[q];
-                o[j + 1] = c;
-                ++m;
+            }
+            __syncwarp();
+        }
+}
+
+__device__ __forceinline__ bool static_has(const int32_t *__restrict__ scol, int s0, int s1, int c)
+{
+    int lo = s0, hi = s1;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (scol[mid] < c) lo = mid + 1; else hi = mid;
+    }
+    return lo < s1 && scol[lo] == c;
+}
+
+// Per row: its entries in ascending pair order (as placed in incidence order by vertex), and its
+// new columns (partners absent from the static row), ascending and without repeats, at
+// newcol[3 ptr[r] ...] (an entry brings at most three). `rows` rows per warp, a thread each; the
+// warp takes those of more than `few` contacts together. Nothing is done when *heavy is set.
+#define RC_THREADS 64
+__global__ void __launch_bounds__(RC_THREADS) row_contacts_kernel(int V, int rows, int few, const int32_t *__restrict__ ptr,
+                                    uint32_t *cinc, const int32_t *__restrict__ pairs,
+                                    const int32_t *__restrict__ srp, const int32_t *__restrict__ scol,
+                                    int32_t *newcol, int32_t *nnew, const int32_t *__restrict__ heavy)
+{
+    if (*heavy) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r = (blockIdx.x * (RC_THREADS / 32) + warp) * rows + lane;
+    const bool have = lane < rows && r < V;
+    const int c0 = have ? ptr[r] : 0, n = have ? ptr[r + 1] - c0 : 0;
+    if (n <= few) {
+        int m = 0;
+        if (n > 0) {
+            uint32_t *b = cinc + c0;
+            for (int i = 1; i < n; ++i) {
+                const uint32_t x = b[i];
+                int j = i - 1;
+                for (; j >= 0 && pc_ref_id(b[j]) > pc_ref_id(x); --j) b[j + 1] = b[j];
+                b[j + 1] = x;
+            }
+            int32_t *o = newcol + 3ll * c0;
+            const int s0 = srp[r], s1 = srp[r + 1];
+            for (int i = 0; i < n; ++i) {
+                const uint32_t ref = b[i], k = pc_ref_local(ref);
+                const int32_t *pv = pairs + 4ll * pc_ref_id(ref);
+                const int first = k == 0 ? 1 : 0, last = k == 0 ? 3 : 0;  // p couples with a, b, c; they with p
+                for (int l = first; l <= last; ++l) {
+                    const int c = pv[l];
+                    if (static_has(scol, s0, s1, c)) continue;
+                    int j = m - 1;
+                    while (j >= 0 && o[j] > c) --j;
+                    if (j >= 0 && o[j] == c) continue;
+                    for (int q = m - 1; q > j; --q) o[q + 1] = o[q];
+                    o[j + 1] = c;
+                    ++m;
+                }
             }
         }
+        if (have) nnew[r] = m;
     }
-    nnew[r] = m;
+    __syncwarp();
+    for (unsigned full = __ballot_sync(0xffffffffu, n > few); full; full &= full - 1) {
+        const int from = __ffs(full) - 1;
+        const int row = __shfl_sync(0xffffffffu, r, from), b0 = __shfl_sync(0xffffffffu, c0, from);
+        const int cnt = __shfl_sync(0xffffffffu, n, from);
+        uint32_t *ent = cinc + b0;  // sorted as id << 2 | local vertex
+        int32_t *col = newcol + 3ll * b0;
+        for (int i = lane; i < cnt; i += 32) ent[i] = pc_ref_id(ent[i]) << 2 | pc_ref_local(ent[i]);
+        __syncwarp();
+        warp_sort(ent, cnt, lane);
+        const int s0 = srp[row], s1 = srp[row + 1];
+        int m = 0;
+        for (int i0 = 0; i0 < cnt; i0 += 32) {
+            const bool in = i0 + lane < cnt;
+            const uint32_t e = in ? ent[i0 + lane] : 1u, k = e & 3u;
+            const int32_t *pv = pairs + (e & ~3u);
+            if (in) ent[i0 + lane] = pc_ref(PC_REF_CONTACT, k, e >> 2);
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                const bool take = in && (k == 0 || l == 0);
+                const int32_t c = take ? pv[k == 0 ? 1 + l : 0] : 0;
+                const bool fresh = take && !static_has(scol, s0, s1, c);
+                const unsigned f = __ballot_sync(0xffffffffu, fresh);
+                if (fresh) col[m + __popc(f & ((1u << lane) - 1u))] = c;
+                m += __popc(f);
+            }
+        }
+        __syncwarp();
+        warp_sort(col, m, lane);
+        int u = 0;
+        for (int i0 = 0; i0 < m; i0 += 32) {
+            const int i = i0 + lane;
+            const int32_t c = i < m ? col[i] : 0;
+            const bool keep = i < m && (i == 0 || col[i - 1] != c);
+            const unsigned b = __ballot_sync(0xffffffffu, keep);  // (and every lane has read)
+            if (keep) col[u + __popc(b & ((1u << lane) - 1u))] = c;
+            u += __popc(b);
+            __syncwarp();
+        }
+        if (lane == 0) nnew[row] = u;
+    }
 }
 
 // Row r: static row pointer plus the new columns of the rows before it (at[r]); its static
 // and new columns merged, ascending.
 __global__ void merge_rows_kernel(int V, const int32_t *__restrict__ srp, const int32_t *__restrict__ scol,
                                   const int32_t *__restrict__ ptr, const int32_t *__restrict__ newcol,
-                                  const int32_t *__restrict__ at, int64_t cap, int32_t *rp, int32_t *col, uint32_t *err)
+                                  const int32_t *__restrict__ at, const int32_t *__restrict__ heavy, int64_t cap,
+                                  int32_t *rp, int32_t *col, uint32_t *err)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r > V) return;
+    if (r > V || *heavy) return;
     int o = srp[r] + at[r];
     rp[r] = o;
     if (r == V) return;
@@ -882,18 +960,23 @@ extern "C" pc_status pc_assemble_pattern(pc_ctx *ctx, const pc_contacts *contact
     PC_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (P > 0 ? V + 1ll : 2ll * V + 2), st));
     if (P > 0) {
         PC_LAUNCH(ctx, contact_count_kernel, pc_blocks(P, 128), 128, 0, st, P, V, contacts->pairs, cnt, ctx->dflag,
-                  ctx->d_err);
+                  heavy, ctx->d_err);
         PC_TRY(pc_exclusive_scan(ctx, cnt, ctx->cinc_ptr, V, st));
         PC_LAUNCH(ctx, contact_place_kernel, pc_blocks(4ll * P, 256), 256, 0, st, P, V, contacts->pairs, ctx->cinc_ptr,
                   ctx->dflag, ctx->cinc);
-        PC_LAUNCH(ctx, row_contacts_kernel, pc_blocks(V, 64), 64, 0, st, V, ctx->cinc_ptr, ctx->cinc, contacts->pairs,
-                  ctx->srp, ctx->scol, newcol, cnt, heavy);
+        // where there are too few rows to fill the GPU's warps, fewer rows per warp, and a warp for
+        // a row sooner: 12,288 rows of 48 contacts 190 us (325 with a thread for up to 64 and 8 rows),
+        // 830k rows of 16 contacts 910 (2,313 with a thread for up to 8)
+        const bool small = V < 32 * 16 * ctx->num_sms;
+        const int rows = small ? 4 : 32, few = small ? 24 : 64;
+        PC_LAUNCH(ctx, row_contacts_kernel, pc_blocks(V, RC_THREADS / 32 * rows), RC_THREADS, 0, st, V, rows, few, ctx->cinc_ptr,
+                  ctx->cinc, contacts->pairs, ctx->srp, ctx->scol, newcol, cnt, heavy);
         PC_TRY(pc_exclusive_scan(ctx, cnt, at, V, st));
     } else {
         PC_CUDA_TRY(cudaMemsetAsync(ctx->cinc_ptr, 0, sizeof(int32_t) * (V + 1ll), st));
     }
     PC_LAUNCH(ctx, merge_rows_kernel, pc_blocks(V + 1ll, 128), 128, 0, st, V, ctx->srp, ctx->scol, ctx->cinc_ptr, newcol,
-              at, A->cap, A->row_ptr, A->col_idx, ctx->d_err);
+              at, heavy, A->cap, A->row_ptr, A->col_idx, ctx->d_err);
     PC_CUDA_TRY(cudaMemcpyAsync(ctx->h_count, at + V, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     PC_CUDA_TRY(cudaMemcpyAsync(reinterpret_cast<int32_t *>(ctx->h_count) + 1, heavy, sizeof(int32_t),
                                 cudaMemcpyDeviceToHost, st));
