@@ -189,7 +189,8 @@ typedef struct {
  * neighbouring vertices and stores a block between two rows of a patch once for both, where
  * the matrix's blocks inside the patches are symmetric bit for bit, as pc_assemble_values
  * makes them; otherwise, or with rows of more than 64 kept blocks or patches of too many
- * contacts for shared memory, it is a plain BSR copy. Without dres, or when the copy
+ * contacts for shared memory, it is a plain BSR copy (as for more than 480 rows per SM when
+ * max_iter is below 32: the records cost what about 25 products save). Without dres, or when the copy
  * exceeds the context's capacity, the products read the matrix itself. */
 #define PC_STORAGE_SYM 0
 #define PC_STORAGE_FULL 1

@@ -174,6 +174,7 @@ struct pc_ctx {
     int32_t *pt_old = nullptr, *pt_new = nullptr;    // [V] original number of a new one, and back
     void *pt_desc = nullptr;                         // [pt_n] PatchDesc
     uint8_t *pt_cnt = nullptr;                       // [pt_n pt_rows] kept blocks per row
+    uint16_t *pt_cross = nullptr;                    // [2][pt_n pt_rows] blocks that leave the patch; that others keep
     uint8_t *pt_named = nullptr;                     // [V] rows in some patch's halo
     int32_t *pt_size = nullptr;                      // [2][pt_n + 1] record sizes, offsets
     int32_t *pt_info = nullptr;                      // [8]
@@ -336,7 +337,7 @@ struct PatchInfo {
 };
 pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st);
 pc_status pc_patch_limit(const pc_ctx *c, bool resident, int *bytes);
-pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, PatchInfo *out, cudaStream_t st);
+pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, int limit, PatchInfo *out, cudaStream_t st);
 // The whole solve in one thread-block cluster (pc_cluster.cu). Runs when the system fits
 // the cluster's shared memory (*ran = true, returns the solve's status); otherwise
 // returns PC_OK with *ran = false, or PC_ERR_CAPACITY when `required`. Needs c->dinv

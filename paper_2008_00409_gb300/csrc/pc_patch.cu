@@ -149,6 +149,7 @@ pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
     const size_t o_z = take(resident ? 4 * sizeof(uint64_t) * (size_t)V : 0);
     const size_t o_slots = take(resident ? sizeof(uint64_t) * (12 * (size_t)c->pt_n * c->pt_n + 1) : 0);
     const size_t o_store = take((size_t)c->pt_cap);
+    const size_t o_cross = take(2 * sizeof(uint16_t) * (size_t)c->pt_n * c->pt_rows);
     // without room for it the context has no order (pt_store stays null: the solves stream the
     // BSR rows)
     unsigned char *base = nullptr;
@@ -160,6 +161,7 @@ pc_status pc_patch_alloc(pc_ctx *c, cudaStream_t st)
     c->pt_new = reinterpret_cast<int32_t *>(base + o_new);
     c->pt_desc = base + o_desc;
     c->pt_cnt = base + o_cnt;
+    c->pt_cross = reinterpret_cast<uint16_t *>(base + o_cross);
     c->pt_named = base + o_named;
     c->pt_size = reinterpret_cast<int32_t *>(base + o_size);
     c->pt_info = reinterpret_cast<int32_t *>(base + o_info);
@@ -226,16 +228,36 @@ struct BuildArgs {
     const int32_t *new_of, *old_of;
     PatchDesc *desc;
     uint8_t *cnt, *named;   // kept blocks of each row; rows in some patch's halo
+    uint16_t *cross, *mirs; // blocks of each row that leave the patch; that another row keeps
     int32_t *size, *at;     // record sizes and offsets, in 16-byte units
     int32_t *info;          // [0] no record (count), [1] largest record, [2] largest halo, [3] failure (fill), [4] most kept blocks, [5] all of them
+    int limit;              // bytes of the largest record that a solve can use
     int64_t cap;            // bytes of the store
     unsigned char *store;
 };
+
+// f(k, column, its new number) for the blocks k of row r, four columns in flight.
+template <typename F>
+__device__ __forceinline__ void patch_row(const BuildArgs &a, int r, F f)
+{
+    const int k1 = a.rp[r + 1];
+    for (int k = a.rp[r]; k < k1; k += 4) {
+        int c[4], n[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[u] = a.ci[min(k + u, k1 - 1)];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) n[u] = a.new_of[c[u]];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (k + u < k1) f(k + u, c[u], n[u]);
+    }
+}
 
 // The patch's block columns outside it, sorted and without repeats, in s_list; returns
 // their number (-1: too many). n: entries of s_list, not sorted.
 __device__ int halo_sort(int *s_list, int n)
 {
+    __shared__ int s_cnt[32];
     if (n > PT_HALO_CAP) return -1;
     int m = 32;
     while (m < n) m <<= 1;
@@ -243,49 +265,36 @@ __device__ int halo_sort(int *s_list, int n)
     __syncthreads();
     for (int k = 2; k <= m; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < m; i += blockDim.x) {
-                const int o = i ^ j;
-                if (o > i) {
-                    const int x = s_list[i], y = s_list[o];
-                    if ((x > y) == ((i & k) == 0)) {
-                        s_list[i] = y;
-                        s_list[o] = x;
-                    }
+            for (int t = threadIdx.x; t < m / 2; t += blockDim.x) {
+                const int i = 2 * t - (t & (j - 1)), o = i + j;
+                const int x = s_list[i], y = s_list[o];
+                if ((x > y) == ((i & k) == 0)) {
+                    s_list[i] = y;
+                    s_list[o] = x;
                 }
             }
             __syncthreads();
         }
-    // compact in place: every thread takes a run, counts its firsts, then writes them
-    __shared__ int s_run[1024];
-    const int per = (n + blockDim.x - 1) / blockDim.x, b = min((int)threadIdx.x * per, n), e = min(b + per, n);
-    int c = 0;
-    for (int i = b; i < e; ++i) c += i == 0 || s_list[i] != s_list[i - 1];
-    s_run[threadIdx.x] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int s = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) {
-            const int v = s_run[i];
-            s_run[i] = s;
-            s += v;
+    // compact in place, a chunk of one value per thread at a time
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int kept = 0;
+    for (int i0 = 0; i0 < n; i0 += blockDim.x) {
+        const int i = i0 + threadIdx.x;
+        const int v = i < n ? s_list[i] : 0;
+        const bool first = i < n && (i == 0 || s_list[i - 1] != v);
+        const unsigned b = __ballot_sync(0xffffffffu, first);
+        if (lane == 0) s_cnt[warp] = __popc(b);
+        __syncthreads();  // (and the chunk has been read)
+        int at = kept;
+        for (int w = 0; w < nw; ++w) {
+            const int c = s_cnt[w];
+            if (w < warp) at += c;
+            kept += c;
         }
+        if (first) s_list[at + __popc(b & ((1u << lane) - 1u))] = v;
+        __syncthreads();
     }
-    __syncthreads();
-    const int prev = b > 0 && b < n ? s_list[b - 1] : -1;
-    int keep[PT_HALO_CAP / 128 + 1];  // per <= PT_HALO_CAP / blockDim (>= 128)
-    int o = s_run[threadIdx.x], kk = 0;
-    int last = prev;
-    for (int i = b; i < e; ++i) {
-        const int v = s_list[i];
-        if (i == 0 || v != last) keep[kk++] = v;
-        last = v;
-    }
-    __syncthreads();
-    for (int i = 0; i < kk; ++i) s_list[o + i] = keep[i];
-    __shared__ int s_n;
-    if (threadIdx.x == blockDim.x - 1) s_n = o + kk;
-    __syncthreads();
-    return s_n;
+    return kept;
 }
 
 // Whether, of two rows a and b of one patch (local numbers) that share a block, a keeps it: the
@@ -297,55 +306,45 @@ __device__ __forceinline__ bool patch_keeps(const uint16_t *cross, int a, int b)
     return ((a + b) & 1) ? a > b : a < b;
 }
 
-// cross[t]: blocks of local row t whose column lies outside the patch; their columns go to
-// s_list (*s_n of them, at most PT_HALO_CAP kept).
-__device__ void patch_cross(const BuildArgs &a, int base, uint16_t *cross, int *s_list, int *s_n)
+// Count: per row its kept blocks, per patch its record's size. A patch that no solve can use
+// (dense contacts: more blocks than fit) is found before its halo is sorted.
+__global__ void __launch_bounds__(1024) patch_count_kernel(BuildArgs a)
 {
-    for (int t = threadIdx.x; t < a.R; t += blockDim.x) {
-        int x = 0;
-        if (base + t < a.V) {
-            const int r = a.old_of[base + t];
-            for (int k = a.rp[r]; k < a.rp[r + 1]; ++k) {
-                const int nc = a.new_of[a.ci[k]];
-                if (nc < base || nc >= base + a.R) {
-                    ++x;
-                    const int p = atomicAdd(s_n, 1);
-                    if (p < PT_HALO_CAP) s_list[p] = nc;
-                }
-            }
-        }
-        cross[t] = (uint16_t)min(x, 65535);
-    }
-    __syncthreads();
-}
-
-// Count: per row its kept blocks, per patch its record's size.
-__global__ void patch_count_kernel(BuildArgs a)
-{
+    extern __shared__ uint16_t s_cross[];  // [R]
     __shared__ int s_list[PT_HALO_CAP];
-    __shared__ uint16_t s_cross[PT_MAX_ROWS];
     __shared__ int s_n, s_own, s_ent, s_mir, s_bad;
     const int patch = blockIdx.x, base = patch * a.R;
     if (threadIdx.x == 0) s_n = s_own = s_ent = s_mir = s_bad = 0;
     __syncthreads();
-    patch_cross(a, base, s_cross, s_list, &s_n);
+    for (int t = threadIdx.x; t < a.R; t += blockDim.x) {
+        int x = 0;
+        if (base + t < a.V)
+            patch_row(a, a.old_of[base + t], [&](int, int, int nc) {
+                if (nc >= base && nc < base + a.R) return;
+                ++x;
+                const int p = atomicAdd(&s_n, 1);
+                if (p < PT_HALO_CAP) s_list[p] = nc;
+            });
+        a.cross[base + t] = s_cross[t] = (uint16_t)min(x, 65535);
+    }
+    __syncthreads();
     for (int t = threadIdx.x; t < a.R; t += blockDim.x) {
         int own = s_cross[t], mir = 0;
         if (base + t < a.V) {
             const int r = a.old_of[base + t];
             int prev = -1;
-            for (int k = a.rp[r]; k < a.rp[r + 1]; ++k) {
-                const int c = a.ci[k];
+            patch_row(a, r, [&](int, int c, int nc) {
                 if (c <= prev) s_bad = 1;  // columns ascend (a mirrored block is looked up once)
                 prev = c;
-                const int lc = a.new_of[c] - base;
-                if (c == r || lc < 0 || lc >= a.R) continue;
+                const int lc = nc - base;
+                if (c == r || lc < 0 || lc >= a.R) return;
                 if (patch_keeps(s_cross, t, lc)) ++own;
                 else ++mir;
-            }
+            });
             if (own > PT_MAX_OWN || mir > 65535) s_bad = 1;
         }
         a.cnt[base + t] = (uint8_t)min(own, 255);
+        a.mirs[base + t] = (uint16_t)min(mir, 65535);
         const int n = (int)__reduce_add_sync(0xffffffffu, (unsigned)own);
         const int we = (int)__reduce_max_sync(0xffffffffu, (unsigned)own);
         const int wm = (int)__reduce_max_sync(0xffffffffu, (unsigned)mir);
@@ -356,19 +355,20 @@ __global__ void patch_count_kernel(BuildArgs a)
         }
     }
     __syncthreads();
-    const int nh = halo_sort(s_list, s_n);
+    PatchDesc d{};
+    d.n_own = s_own;
+    d.n_ent = s_ent;
+    d.n_mir = s_mir;
+    bool bad = s_bad || s_own > 65534 || s_mir > 4096 || patch_layout(a.R, d).bytes > a.limit;
+    const int nh = bad ? -1 : halo_sort(s_list, s_n);
     for (int i = threadIdx.x; i < nh; i += blockDim.x) a.named[s_list[i]] = 1;
     if (threadIdx.x == 0) {
-        PatchDesc d{};
-        d.n_own = s_own;
-        d.n_ent = s_ent;
-        d.n_mir = s_mir;
         d.n_halo = max(nh, 0);
-        const bool bad = s_bad || nh < 0 || s_own > 65534 || a.R + d.n_halo > 32767 || s_mir > 4096;
+        bad = bad || nh < 0 || a.R + d.n_halo > 32767;
         d.bytes = bad ? 0 : patch_layout(a.R, d).bytes;
         a.desc[patch] = d;
         a.size[patch] = d.bytes / 16;
-        if (bad) atomicOr(a.info, 1);
+        if (bad || d.bytes > a.limit) atomicOr(a.info, 1);
         atomicMax(a.info + 1, d.bytes);
         atomicMax(a.info + 2, d.n_halo);
         atomicMax(a.info + 4, d.n_own);
@@ -376,16 +376,24 @@ __global__ void patch_count_kernel(BuildArgs a)
     }
 }
 
-__global__ void patch_fill_kernel(BuildArgs a)
+// Fill, in three passes with the CTA's barrier between them: each row numbers its blocks (a kept
+// one leaves its place in the matrix, its entry's place and its column in the slot it gets, a
+// mirrored one the row that keeps it); each slot becomes the block and its entry; each mirrored
+// block finds its slot among the keeping row's entries and is compared with it.
+// Bound by the latency of the columns' and blocks' gathers. 271,803 rows with 5% contacts: 191 us,
+// and 50 for 12,288 rows with dense ones (796 and 377 with a thread per row that copied each block,
+// and looked for each mirrored one along the other row's columns).
+__global__ void __launch_bounds__(1024) patch_fill_kernel(BuildArgs a)
 {
+    extern __shared__ unsigned char s_raw[];
     __shared__ int s_list[PT_HALO_CAP];
-    __shared__ uint16_t s_cross[PT_MAX_ROWS];
-    __shared__ unsigned s_mask[PT_SLICES][PT_MAX_OWN];   // rows of the slice with an e-th kept block
-    __shared__ uint16_t s_at[PT_SLICES][PT_MAX_OWN + 1]; // and the slot of the first of them
-    __shared__ int s_base[3][PT_SLICES + 1];             // first slot, entry column, share column of each slice
+    __shared__ int s_base[3][PT_SLICES + 1];  // first slot, entry column, share column of each slice
     __shared__ int s_n;
     const int patch = blockIdx.x, base = patch * a.R, lane = threadIdx.x & 31;
     const int slices = a.R / 32;
+    unsigned *s_mask = reinterpret_cast<unsigned *>(s_raw);                        // [slice][e]: rows with an e-th kept block
+    uint16_t *s_at = reinterpret_cast<uint16_t *>(s_mask + slices * PT_MAX_OWN);   // and the slot of the first of them
+    uint16_t *s_cross = s_at + slices * PT_MAX_OWN;                                // [R]
     PatchDesc d = a.desc[patch];
     d.offset = 16ll * a.at[patch];
     if (a.info[0] || d.offset + d.bytes > a.cap) {  // info[0] is final: this kernel reports in info[3]
@@ -396,32 +404,22 @@ __global__ void patch_fill_kernel(BuildArgs a)
         a.desc[patch].offset = d.offset;
         s_n = 0;
     }
-    __syncthreads();
     unsigned char *rec = a.store + d.offset;
     const PatchLayout L = patch_layout(a.R, d);
-    patch_cross(a, base, s_cross, s_list, &s_n);
     for (int t = threadIdx.x; t < a.R; t += blockDim.x) {
-        const int nr = base + t, sl = t >> 5;
-        const int co = a.cnt[nr];
+        const int sl = t >> 5, co = a.cnt[base + t];
         const int mo = (int)__reduce_max_sync(0xffffffffu, (unsigned)co);
+        const int wm = (int)__reduce_max_sync(0xffffffffu, (unsigned)a.mirs[base + t]);
+        s_cross[t] = a.cross[base + t];
         int at = 0;
         for (int e = 0; e < mo; ++e) {
             const unsigned m = __ballot_sync(0xffffffffu, e < co);
             if (lane == 0) {
-                s_mask[sl][e] = m;
-                s_at[sl][e] = (uint16_t)at;
+                s_mask[sl * PT_MAX_OWN + e] = m;
+                s_at[sl * PT_MAX_OWN + e] = (uint16_t)at;
             }
             at += __popc(m);
         }
-        int mir = 0;
-        if (nr < a.V) {
-            const int r = a.old_of[nr];
-            for (int k = a.rp[r]; k < a.rp[r + 1]; ++k) {
-                const int c = a.ci[k], lc = a.new_of[c] - base;
-                mir += c != r && lc >= 0 && lc < a.R && !patch_keeps(s_cross, t, lc);
-            }
-        }
-        const int wm = (int)__reduce_max_sync(0xffffffffu, (unsigned)mir);
         if (lane == 0) {
             s_base[0][sl] = at;
             s_base[1][sl] = mo;
@@ -439,8 +437,6 @@ __global__ void patch_fill_kernel(BuildArgs a)
         }
     }
     __syncthreads();
-    const int nh = halo_sort(s_list, s_n);
-    for (int i = threadIdx.x; i < nh; i += blockDim.x) reinterpret_cast<int32_t *>(rec + L.halo)[i] = s_list[i];
     uint32_t *ent = reinterpret_cast<uint32_t *>(rec + L.ent);
     uint16_t *mir = reinterpret_cast<uint16_t *>(rec + L.mir);
     float4 *va = reinterpret_cast<float4 *>(rec + L.va), *vb = reinterpret_cast<float4 *>(rec + L.vb);
@@ -452,69 +448,104 @@ __global__ void patch_fill_kernel(BuildArgs a)
     for (int t = threadIdx.x; t < a.R; t += blockDim.x) {
         const int nr = base + t, sl = t >> 5;
         const unsigned lt = (1u << lane) - 1u;
-        const int r = nr < a.V ? a.old_of[nr] : 0;
-        const int k0 = nr < a.V ? a.rp[r] : 0, k1 = nr < a.V ? a.rp[r + 1] : 0;
-        uint32_t *o = ent + 32 * s_base[1][sl] + lane, *o_end = ent + 32 * s_base[1][sl + 1];
-        uint16_t *m = mir + 32 * s_base[2][sl] + lane, *m_end = mir + 32 * s_base[2][sl + 1];
-        int e = 0;
-        for (int k = k0; k < k1; ++k) {
-            const int c = a.ci[k];
-            if (c == r) continue;
-            const int nc = a.new_of[c];
-            int lc = nc - base;
-            const bool out = lc < 0 || lc >= a.R;
-            const float *B = a.vals + 9ll * k;
-            if (out || patch_keeps(s_cross, t, lc)) {
-                const int s = s_base[0][sl] + s_at[sl][e] + __popc(s_mask[sl][e] & lt);
-                ++e;
-                if (out) {
-                    int lo = 0, hi = nh;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (s_list[mid] < nc) lo = mid + 1; else hi = mid;
+        int o = 32 * s_base[1][sl] + lane, m = 32 * s_base[2][sl] + lane, e = 0;
+        if (nr < a.V) {
+            const int r = a.old_of[nr];
+            patch_row(a, r, [&](int k, int c, int nc) {
+                if (c == r) return;
+                const int lc = nc - base;
+                const bool out = lc < 0 || lc >= a.R;
+                if (out || patch_keeps(s_cross, t, lc)) {
+                    const int s = s_base[0][sl] + s_at[sl * PT_MAX_OWN + e] + __popc(s_mask[sl * PT_MAX_OWN + e] & lt);
+                    ++e;
+                    reinterpret_cast<int4 *>(va)[s] = make_int4(k, o, nc, 0);
+                    o += 32;
+                    if (out) {
+                        const int p = atomicAdd(&s_n, 1);
+                        if (p < PT_HALO_CAP) s_list[p] = nc;
                     }
-                    lc = a.R + lo;
+                } else {
+                    mir[m] = (uint16_t)lc;
+                    m += 32;
                 }
-                va[s] = make_float4(B[0], B[1], B[2], B[3]);
-                vb[s] = make_float4(B[4], B[5], B[6], B[7]);
-                vc[s] = B[8];
-                *o = (out ? PT_NO_SHARE : 0u) | ((uint32_t)lc << 16) | (uint32_t)s;
-                o += 32;
-            } else {  // block (c, r), kept by row c: its place among that row's kept blocks
-                const int ls = lc >> 5;
-                int e2 = 0, q = a.rp[c];
-                const int q1 = a.rp[c + 1];
-                for (; q < q1 && a.ci[q] != r; ++q) {
-                    const int l2 = a.new_of[a.ci[q]] - base;
-                    e2 += l2 != lc && (l2 < 0 || l2 >= a.R || patch_keeps(s_cross, lc, l2));
-                }
-                bool same = q < q1;
-                if (same) {
-                    const float *T = a.vals + 9ll * q;
-                    for (int i = 0; i < 3; ++i)
-                        for (int j = 0; j < 3; ++j)
-                            same = same && __float_as_uint(B[3 * i + j]) == __float_as_uint(T[3 * j + i]);
-                }
-                int s = d.n_own;
-                if (!same) atomicOr(a.info + 3, 1);
-                else s = s_base[0][ls] + s_at[ls][e2] + __popc(s_mask[ls][e2] & ((1u << (lc & 31)) - 1u));
-                *m = (uint16_t)s;
-                m += 32;
-            }
+            });
         }
         // missing entries: own p (zero difference), the block of a lane of the same eight,
         // which one 16-byte shared-memory access serves together
-        for (; o < o_end; o += 32, ++e) {
-            const unsigned m8 = s_mask[sl][e] & (0xffu << (lane & 24)), all = s_mask[sl][e];
+        for (; o < 32 * s_base[1][sl + 1]; o += 32, ++e) {
+            const unsigned all = s_mask[sl * PT_MAX_OWN + e], m8 = all & (0xffu << (lane & 24));
             const int from = __ffs(m8 ? m8 : all) - 1;
-            *o = PT_NO_SHARE | ((uint32_t)t << 16) |
-                 (uint32_t)(s_base[0][sl] + s_at[sl][e] + __popc(all & ((1u << from) - 1u)));
+            ent[o] = PT_NO_SHARE | ((uint32_t)t << 16) |
+                     (uint32_t)(s_base[0][sl] + s_at[sl * PT_MAX_OWN + e] + __popc(all & ((1u << from) - 1u)));
         }
-        for (; m < m_end; m += 32) *m = (uint16_t)d.n_own;
+        for (; m < 32 * s_base[2][sl + 1]; m += 32) mir[m] = (uint16_t)d.n_own;
+    }
+    __syncthreads();
+    const int nh = halo_sort(s_list, s_n);
+    for (int i = threadIdx.x; i < nh; i += blockDim.x) reinterpret_cast<int32_t *>(rec + L.halo)[i] = s_list[i];
+    for (int s = threadIdx.x; s < d.n_own; s += blockDim.x) {
+        const int4 w = reinterpret_cast<const int4 *>(va)[s];
+        const float *B = a.vals + 9ll * w.x;
+        float b[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) b[q] = B[q];
+        int lc = w.z - base;
+        const bool out = lc < 0 || lc >= a.R;
+        if (out) {
+            int lo = 0, hi = nh;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (s_list[mid] < w.z) lo = mid + 1; else hi = mid;
+            }
+            lc = a.R + lo;
+        }
+        va[s] = make_float4(b[0], b[1], b[2], b[3]);
+        vb[s] = make_float4(b[4], b[5], b[6], b[7]);
+        vc[s] = b[8];
+        ent[w.y] = (out ? PT_NO_SHARE : 0u) | ((uint32_t)lc << 16) | (uint32_t)s;
+    }
+    __syncthreads();
+    const int parts = max(1, (int)blockDim.x / a.R);
+    for (int i = threadIdx.x; i < parts * a.R; i += blockDim.x) {
+        const int part = i / a.R, t = i - part * a.R, nr = base + t;
+        if (nr >= a.V) continue;
+        const int r = a.old_of[nr], k0 = a.rp[r], k1 = a.rp[r + 1], n = a.mirs[nr];
+        uint16_t *m = mir + 32 * s_base[2][t >> 5] + lane;
+        for (int j = part; j < n; j += parts) {
+            const int lc = m[32 * j], c = a.old_of[base + lc];
+            int lo = k0, hi = k1;  // the block (r, c)
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (a.ci[mid] < c) lo = mid + 1; else hi = mid;
+            }
+            const float *B = a.vals + 9ll * lo;
+            const uint32_t *o = ent + 32 * s_base[1][lc >> 5] + (lc & 31);
+            uint32_t w = 0;
+            const int ne = a.cnt[base + lc];
+            int e = 0;
+            for (; e < ne; ++e) {
+                w = o[32 * e];
+                if ((w >> 16) == (uint32_t)t) break;  // a shared entry (its top bit clear) of column t
+            }
+            const int s = w & 0xffffu;
+            bool same = e < ne;
+            if (same) {
+                const float4 p = va[s], q = vb[s];
+                const float T[9] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w, vc[s]};
+#pragma unroll
+                for (int x = 0; x < 3; ++x)
+#pragma unroll
+                    for (int y = 0; y < 3; ++y)
+                        same = same && __float_as_uint(B[3 * x + y]) == __float_as_uint(T[3 * y + x]);
+            }
+            if (!same) atomicOr(a.info + 3, 1);
+            m[32 * j] = (uint16_t)(same ? s : d.n_own);
+        }
     }
 }
 
-pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, PatchInfo *out, cudaStream_t st)
+// `limit`: bytes of the largest record that the solve can use.
+pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, int limit, PatchInfo *out, cudaStream_t st)
 {
     out->ok = false;
     if (!c->pt_store || A->nnzb > c->A_cap) return PC_OK;
@@ -528,18 +559,24 @@ pc_status pc_patch_build(pc_ctx *c, const pc_bsr *A, const float *vals, PatchInf
     a.old_of = c->pt_old;
     a.desc = static_cast<PatchDesc *>(c->pt_desc);
     a.cnt = c->pt_cnt;
+    a.cross = c->pt_cross;
+    a.mirs = c->pt_cross + (size_t)c->pt_n * c->pt_rows;
     a.named = c->pt_named;
     a.size = c->pt_size;
     a.at = c->pt_size + c->pt_n + 1;
     a.info = c->pt_info;
+    a.limit = limit;
     a.cap = c->pt_cap;
     a.store = c->pt_store;
-    const int threads = a.R < 128 ? 128 : a.R > 512 ? 512 : a.R;
+    // one CTA per SM and patch: as many threads as the rows can use. Else two per row: the passes
+    // over slots and mirrored blocks share them (830,028 rows: 525 us; 596 with one, 679 with four)
+    const int threads = c->pt_slots ? (a.R <= 256 ? 4 : 2) * a.R : 2 * PT_ROWS;
+    const size_t fill_smem = a.R / 32 * PT_MAX_OWN * (sizeof(unsigned) + sizeof(uint16_t)) + sizeof(uint16_t) * a.R;
     PC_CUDA_TRY(cudaMemsetAsync(c->pt_info, 0, sizeof(int32_t) * 6, st));
     PC_CUDA_TRY(cudaMemsetAsync(c->pt_named, 0, (size_t)c->V, st));
-    PC_LAUNCH(c, patch_count_kernel, c->pt_n, threads, 0, st, a);
+    PC_LAUNCH(c, patch_count_kernel, c->pt_n, threads, sizeof(uint16_t) * a.R, st, a);
     PC_TRY(pc_exclusive_scan(c, a.size, a.at, c->pt_n, st));
-    PC_LAUNCH(c, patch_fill_kernel, c->pt_n, threads, 0, st, a);
+    PC_LAUNCH(c, patch_fill_kernel, c->pt_n, threads, fill_smem, st, a);
     PC_CUDA_TRY(cudaMemcpyAsync(c->h_count, c->pt_info, sizeof(int32_t) * 6, cudaMemcpyDeviceToHost, st));
     PC_CUDA_TRY(cudaStreamSynchronize(st));
     const int32_t *h = reinterpret_cast<const int32_t *>(c->h_count);

@@ -1478,29 +1478,40 @@ static pc_status launch_resident(const SolveCtx &s, float *x, const pc_solve_opt
 // Patch storage for the difference-form products where the matrix suits it and at least
 // three CTAs of the product fit an SM beside each other (with fewer, the copies of one no
 // longer hide behind the others): the vectors then take the patches' row order.
-static pc_status try_patch(SolveCtx &s)
+// Streamed records cost as much as about 25 products from them save (830,028 rows: one
+// iteration 1.5 ms without, 1.9 with; 32 iterations 4.0 ms either way; 100 iterations 9.6 and 8.4),
+// so a solve that may not take PT_MIN_ITERS goes without. Resident ones cost no more than the
+// copy that they replace.
+#define PT_MIN_ITERS 32
+static pc_status try_patch(SolveCtx &s, int max_iter)
 {
     pc_ctx *c = s.c;
-    PatchInfo pi{};
-    PC_TRY(pc_patch_build(c, s.A, s.vals, &pi, s.st));
-    if (!pi.ok) return PC_OK;
+    const bool resident = c->pt_slots != nullptr;
     int limit = 0;
-    PC_TRY(pc_patch_limit(c, c->pt_slots != nullptr, &limit));
-    s.pt_halo = pi.max_halo;
-    s.pt_rec = (pi.max_bytes + 127) / 128 * 128;
-    if (c->pt_slots) {
+    PC_TRY(pc_patch_limit(c, resident, &limit));
+    if (resident) {
         // one CTA per patch for the whole solve, if everything fits (the fused update's stop
         // tests and direction step; fuse = 0 keeps the separate kernels)
-        if (!s.fuse || c->pt_n > c->num_sms) return PC_OK;
-        int coop = 0, occ = 0;
+        int coop = 0;
         PC_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
+        if (!s.fuse || !coop || c->pt_n > c->num_sms) return PC_OK;
+    } else if (max_iter < PT_MIN_ITERS) {
+        return PC_OK;
+    }
+    PatchInfo pi{};
+    PC_TRY(pc_patch_build(c, s.A, s.vals, limit, &pi, s.st));
+    if (!pi.ok) return PC_OK;
+    s.pt_halo = pi.max_halo;
+    s.pt_rec = (pi.max_bytes + 127) / 128 * 128;
+    if (resident) {
+        int occ = 0;
         s.pt_split = c->pt_rows <= 256 ? 4 : 2;
         s.pt_share = pi.max_own + 1;
         s.pt_smem = s.pt_rec + 16 * s.pt_share + 12 * (c->pt_rows + pi.max_halo) + 12 * (s.pt_split - 1) * c->pt_rows;
         const void *k = resident_kernel(s);
         cudaFuncAttributes fa;
         PC_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
-        if (!coop || s.pt_smem + (int)fa.sharedSizeBytes > limit) return PC_OK;
+        if (s.pt_smem + (int)fa.sharedSizeBytes > limit) return PC_OK;
         PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, s.pt_split * c->pt_rows, s.pt_smem));
         if (occ < 1) return PC_OK;
         s.resident = true;
@@ -1557,7 +1568,7 @@ static pc_status pcg_solve_impl(pc_ctx *ctx, const pc_bsr *A, const float *vals,
     if (o.storage == PC_STORAGE_SELL) PC_TRY(build_sell(ctx, A, vals, &s.sell, st));
     // the diagonal blocks multiply p_i - p_i = 0 in the difference form only
     if (o.storage == PC_STORAGE_OFFDIAG && s.diff) {
-        if (ctx->dsc && ctx->pt_store) PC_TRY(try_patch(s));
+        if (ctx->dsc && ctx->pt_store) PC_TRY(try_patch(s, o.max_iter));
         if (!s.patch) PC_TRY(build_offdiag(ctx, A, vals, &s.offdiag, st));
     }
     if (s.diff && ctx->dsc) PC_LAUNCH(ctx, dsc_kernel, pc_blocks(V, 256), 256, 0, st, V, dres, ctx->dsc,
