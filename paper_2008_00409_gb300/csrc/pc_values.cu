@@ -374,13 +374,14 @@ __global__ void __launch_bounds__(128) hinge_eval_kernel(int H, const int32_t *_
 
 // One thread per pair (p; a, b, c). Record: right-hand-side contributions (12), unit
 // normal n of (a, b, c) at x (3), weights (3), h^2 kc (1) (h (h + beta) kc with Rayleigh
-// damping; 0 for an inactive thickness contact). With s = (1, -w_a, -w_b, -w_c) the
+// damping; 0 for an inactive thickness contact), 1 when one of the four vertices is pinned. With s = (1, -w_a, -w_b, -w_c) the
 // Hessian block (k, l) is h^2 kc s_k s_l n n^T. The hold penalty is zero at x_t (d = d0)
 // and linear in x, so its contribution h (f - h K v) is -h^2 kc (n . sum_l s_l v_l) s_k n;
 // the thickness penalty adds its force at x_t, h kc (delta - d) s_k n.
 __global__ void contact_eval_kernel(int P, const int32_t *__restrict__ pairs, const float *__restrict__ wts,
                                     const float *__restrict__ x, const float *__restrict__ v, float kc, float h,
-                                    float hk, float thick, float *__restrict__ out)
+                                    float hk, float thick, const uint8_t *__restrict__ pinned,
+                                    float *__restrict__ out)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P) return;
@@ -420,13 +421,15 @@ __global__ void contact_eval_kernel(int P, const int32_t *__restrict__ pairs, co
     o[12] = n.x; o[13] = n.y; o[14] = n.z;
     o[15] = w[0]; o[16] = w[1]; o[17] = w[2];
     o[18] = hk * kc_eff;
-    o[19] = 0.0f;
+    o[19] = pinned[vid[0]] || pinned[vid[1]] || pinned[vid[2]] || pinned[vid[3]] ? 1.0f : 0.0f;
 }
 
 // ------------------------------------------------------------------------- row reduction
 
 #define RR_ROWS 32                     // rows per CTA
+#define RR_FEW_ROWS 8                  // where there are too few rows to fill the GPU with such CTAs
 #define RR_THREADS 128
+#define RR_CTAS_PER_SM 9
 
 // Contributions to one block (row, col), col != row, from the mesh's elements, in incidence
 // order: the static list of (type, k, l, id) codes that pc_create made for the block
@@ -481,24 +484,38 @@ __device__ __forceinline__ void add_static(const uint32_t *__restrict__ codes, i
     }
 }
 
-// Contributions of the row's contacts to block (row, col), in contact order.
+// Contributions of the row's contacts to block (row, col), in contact order. Every block of the row
+// looks at all of them, so four are in flight (12,288 rows of 48 contacts and 28 blocks: the values
+// 260 -> 218 us, 830k rows of 16 contacts 2,566 -> 2,354).
 __device__ __forceinline__ void add_contacts(const uint32_t *__restrict__ cinc, int c0, int c1,
                                              const int32_t *__restrict__ pairs, const float *__restrict__ cont_buf,
                                              int col, float acc[9])
 {
-    for (int i = c0; i < c1; ++i) {
-        const uint32_t ref = cinc[i], k = pc_ref_local(ref), id = pc_ref_id(ref);
-        const int32_t *pv = pairs + 4ll * id;
-        const int l = pv[0] == col ? 0 : pv[1] == col ? 1 : pv[2] == col ? 2 : pv[3] == col ? 3 : -1;
-        if (l < 0) continue;
-        const float *o = cont_buf + (int64_t)PC_CONTACT_STRIDE * id;
-        const float sk = k == 0 ? 1.0f : -o[14 + k], sl = l == 0 ? 1.0f : -o[14 + l];
-        const float cs = o[18] * (sk * sl);
-        const float n[3] = {o[12], o[13], o[14]};
+    for (int i = c0; i < c1; i += 4) {
+        uint32_t ref[4];
+        int l[4];
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
+        for (int u = 0; u < 4; ++u) ref[u] = cinc[min(i + u, c1 - 1)];
 #pragma unroll
-            for (int b = 0; b < 3; ++b) acc[3 * a + b] = __fadd_rn(acc[3 * a + b], __fmul_rn(cs, __fmul_rn(n[a], n[b])));
+        for (int u = 0; u < 4; ++u) {
+            const int32_t *pv = pairs + 4ll * pc_ref_id(ref[u]);
+            const int v0 = pv[0], v1 = pv[1], v2 = pv[2], v3 = pv[3];
+            l[u] = i + u >= c1 ? -1 : v0 == col ? 0 : v1 == col ? 1 : v2 == col ? 2 : v3 == col ? 3 : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (l[u] < 0) continue;
+            const int k = (int)pc_ref_local(ref[u]);
+            const float *o = cont_buf + (int64_t)PC_CONTACT_STRIDE * pc_ref_id(ref[u]);
+            const float sk = k == 0 ? 1.0f : -o[14 + k], sl = l[u] == 0 ? 1.0f : -o[14 + l[u]];
+            const float cs = o[18] * (sk * sl);
+            const float n[3] = {o[12], o[13], o[14]};
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b)
+                    acc[3 * a + b] = __fadd_rn(acc[3 * a + b], __fmul_rn(cs, __fmul_rn(n[a], n[b])));
+        }
     }
 }
 
@@ -542,7 +559,7 @@ __device__ __forceinline__ void row_block(const RowArgs &a, int row, int slot, i
     if (n1 > n0) add_contacts(a.cinc, n0, n1, a.pairs, a.cont_buf, col, acc);
 }
 
-// One CTA per 32 rows. Warp 0 first forms the rows' diagonal blocks, right-hand sides and
+// One CTA per 32 rows (ROWS). Warp 0 first forms the rows' diagonal blocks, right-hand sides and
 // difference-form diagonals, one thread per row over the row's incident elements; the
 // other blocks go one per thread, over the block's own contribution list, in chunks of 32
 // handed out by a shared counter (warp 0 joins when its rows are done; which warp takes a
@@ -556,12 +573,17 @@ __device__ __forceinline__ void row_block(const RowArgs &a, int row, int slot, i
 // shared memory first, a thread per row that adds each element to its blocks in shared memory,
 // CTAs of 256 threads (921). A warp per row that staged every expanded block, each lane
 // comparing all of them with its column, took 2,825 us for this kernel alone.
-__global__ void __launch_bounds__(RR_THREADS, 9) row_reduce_kernel(RowArgs a)
+// Fewer rows than fill the GPU with such CTAs once are latency, and longest where rows have many
+// contacts: CTAs of 8 rows, and registers for four of a row's contacts in flight (12,288 rows of 48
+// contacts 218 -> 167 us, 4,096 rows of 0.08 with the pattern 92.4 -> 87.4; 49,152 rows of 47 495 -> 400,
+// but 271,803 rows of 12 665 -> 764).
+template <int ROWS>
+__global__ void __launch_bounds__(RR_THREADS, ROWS == RR_ROWS ? RR_CTAS_PER_SM : 6) row_reduce_kernel(RowArgs a)
 {
-    __shared__ int s_rp[RR_ROWS + 1], s_sp[RR_ROWS + 1], s_cp[RR_ROWS + 1];
+    __shared__ int s_rp[ROWS + 1], s_sp[ROWS + 1], s_cp[ROWS + 1];
     __shared__ int s_next;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r0 = blockIdx.x * RR_ROWS, nr = min(RR_ROWS, a.V - r0);
+    const int r0 = blockIdx.x * ROWS, nr = min(ROWS, a.V - r0);
     for (int i = threadIdx.x; i <= nr; i += blockDim.x) {
         s_rp[i] = a.rp[r0 + i];
         s_sp[i] = a.srp[r0 + i];
@@ -615,22 +637,41 @@ __global__ void __launch_bounds__(RR_THREADS, 9) row_reduce_kernel(RowArgs a)
             }
         }
         bool adj = a.pin_adj[row] != 0;
-        for (int i = n0; i < n1; ++i) {
-            const uint32_t ref = a.cinc[i], k = pc_ref_local(ref), id = pc_ref_id(ref);
-            const float *o = a.cont_buf + (int64_t)PC_CONTACT_STRIDE * id;
-            f[0] += o[3 * k];
-            f[1] += o[3 * k + 1];
-            f[2] += o[3 * k + 2];
-            const float sk = k == 0 ? 1.0f : -o[14 + k], cs = o[18] * (sk * sk);
-            const float n[3] = {o[12], o[13], o[14]};
-            u[0] = __fadd_rn(u[0], __fmul_rn(cs, __fmul_rn(n[0], n[0])));
-            u[1] = __fadd_rn(u[1], __fmul_rn(cs, __fmul_rn(n[0], n[1])));
-            u[2] = __fadd_rn(u[2], __fmul_rn(cs, __fmul_rn(n[0], n[2])));
-            u[3] = __fadd_rn(u[3], __fmul_rn(cs, __fmul_rn(n[1], n[1])));
-            u[4] = __fadd_rn(u[4], __fmul_rn(cs, __fmul_rn(n[1], n[2])));
-            u[5] = __fadd_rn(u[5], __fmul_rn(cs, __fmul_rn(n[2], n[2])));
-            const int32_t *pv = a.pairs + 4ll * id;
-            adj |= a.pinned[pv[0]] || a.pinned[pv[1]] || a.pinned[pv[2]] || a.pinned[pv[3]];
+        constexpr int W = ROWS == RR_ROWS ? 1 : 4;  // contacts in flight (registers)
+        for (int i = n0; i < n1; i += W) {
+            uint32_t ref[W];
+            float4 p[W], q[W];  // (n, w_a) (w_b, w_c, scale, pinned)
+            float g[W][3], sk[W];
+#pragma unroll
+            for (int w = 0; w < W; ++w) ref[w] = a.cinc[min(i + w, n1 - 1)];
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                const float4 *o = reinterpret_cast<const float4 *>(a.cont_buf + (int64_t)PC_CONTACT_STRIDE * pc_ref_id(ref[w]));
+                const int k = (int)pc_ref_local(ref[w]);
+                p[w] = o[3];
+                q[w] = o[4];
+                const float *c = reinterpret_cast<const float *>(o) + 3 * k;
+                g[w][0] = c[0];
+                g[w][1] = c[1];
+                g[w][2] = c[2];
+                sk[w] = k == 0 ? 1.0f : k == 1 ? -p[w].w : k == 2 ? -q[w].x : -q[w].y;
+            }
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                if (i + w >= n1) break;
+                f[0] += g[w][0];
+                f[1] += g[w][1];
+                f[2] += g[w][2];
+                const float cs = q[w].z * (sk[w] * sk[w]);
+                const float n[3] = {p[w].x, p[w].y, p[w].z};
+                u[0] = __fadd_rn(u[0], __fmul_rn(cs, __fmul_rn(n[0], n[0])));
+                u[1] = __fadd_rn(u[1], __fmul_rn(cs, __fmul_rn(n[0], n[1])));
+                u[2] = __fadd_rn(u[2], __fmul_rn(cs, __fmul_rn(n[0], n[2])));
+                u[3] = __fadd_rn(u[3], __fmul_rn(cs, __fmul_rn(n[1], n[1])));
+                u[4] = __fadd_rn(u[4], __fmul_rn(cs, __fmul_rn(n[1], n[2])));
+                u[5] = __fadd_rn(u[5], __fmul_rn(cs, __fmul_rn(n[2], n[2])));
+                adj |= q[w].w != 0.f;
+            }
         }
         float B[9] = {u[0], u[1], u[2], u[1], u[3], u[4], u[2], u[4], u[5]};
         // the diagonal's slot; its list holds elements that meet the vertex twice (two
@@ -702,7 +743,7 @@ __global__ void __launch_bounds__(RR_THREADS, 9) row_reduce_kernel(RowArgs a)
         const int slot = b0 + i;
         int r = 0;  // the row: last r with s_rp[r] <= slot
 #pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
+        for (int step = ROWS / 2; step > 0; step >>= 1)
             if (r + step < nr && s_rp[r + step] <= slot) r += step;
         const int row = r0 + r, col = a.ci[slot];
         if (col == row) continue;
@@ -742,7 +783,7 @@ extern "C" pc_status pc_assemble_values(pc_ctx *ctx, const pc_bsr *A, const floa
                   hk, ih, ctx->hinge_buf);
     if (P > 0)
         PC_LAUNCH(ctx, contact_eval_kernel, pc_blocks(P, 128), 128, 0, st, P, contacts->pairs, contacts->w, x, v,
-                  ctx->mat.k_contact, h, hk, ctx->mat.contact_thickness, ctx->cont_buf);
+                  ctx->mat.k_contact, h, hk, ctx->mat.contact_thickness, ctx->pinned, ctx->cont_buf);
     RowArgs r{};
     r.V = V;
     r.rp = A->row_ptr;
@@ -773,6 +814,9 @@ extern "C" pc_status pc_assemble_values(pc_ctx *ctx, const pc_bsr *A, const floa
     r.vals = vals;
     r.b = b;
     r.dres = dres;
-    PC_LAUNCH(ctx, row_reduce_kernel, pc_blocks(V, RR_ROWS), RR_THREADS, 0, st, r);
+    if (V < RR_ROWS * RR_CTAS_PER_SM * ctx->num_sms)
+        PC_LAUNCH(ctx, row_reduce_kernel<RR_FEW_ROWS>, pc_blocks(V, RR_FEW_ROWS), RR_THREADS, 0, st, r);
+    else
+        PC_LAUNCH(ctx, row_reduce_kernel<RR_ROWS>, pc_blocks(V, RR_ROWS), RR_THREADS, 0, st, r);
     return PC_OK;
 }

@@ -1,6 +1,8 @@
 """Patterns and values of steps in which vertices have many contacts: rows ordered by a thread, by a
 warp, and the key sort, against the FP64 oracle (pattern exact, values
 within the per-block tolerance of _helpers)."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -64,7 +66,7 @@ def test_one_vertex_with_many_contacts(pc, star):
 
 # every vertex with a few dozen contacts, rows of unequal length side by side; few rows (4 per warp)
 # and many (32, a thread for up to 64)
-@pytest.mark.parametrize("n,per", [(20, 12.0), (64, 12.0), (64, 40.0), (280, 3.0)])
+@pytest.mark.parametrize("n,per", [(20, 12.0), (64, 12.0), (64, 40.0), (281, 3.0)])
 def test_every_vertex_with_many_contacts(pc, n, per):
     wl = wk.square_cloth(n, seed=2, contact_frac=0.0)
     rng = np.random.default_rng(n)
@@ -74,3 +76,33 @@ def test_every_vertex_with_many_contacts(pc, n, per):
     launches, used = _check(pc, wl, pairs, n)
     most = np.bincount(used.reshape(-1), minlength=wl.V).max()
     assert (launches <= 10) == (most <= 1024), (launches, most)
+
+
+# the edges of a tile of eight rows and of two; a tile of 32 (many rows: 281 x 281 above)
+@pytest.mark.parametrize("nx,ny", [(4, 2), (3, 3), (5, 3), (4, 4), (17, 1 + 1)])
+def test_values_at_edges_of_small_tiles(pc, nx, ny):
+    rest, tris, _ = wk.grid_piece(nx, ny, 0.01 * (nx - 1), 0.01 * (ny - 1), jitter=0.2, flip_prob=0.1, seed=nx)
+    wl = wk.Workload("tile", rest, tris, np.array([0], np.int32), rest.copy(), np.zeros_like(rest), 1.0 / 200.0,
+                     wk.Material(), [], 1)
+    p = np.arange(wl.V, dtype=np.int64)[:, None]
+    pairs = np.concatenate([np.repeat(p, wl.T, 0), np.tile(wl.tris, (wl.V, 1))], 1)
+    _check(pc, wl, pairs, nx)
+
+
+def test_values_of_few_rows_with_many_contacts_in_time(pc):
+    """12,288 rows of 48 contacts: the rows' contacts are chains of loads where nothing else hides
+    them. A warp per row that staged them took 192 us, which this call may not exceed."""
+    wl = wk.proximity_stack(64, 3, delta=8e-3, per_vertex=40.0)
+    cl = pc.Cloth(wl)
+    pairs, w = cl.proximity()
+    s = cl.assemble(pairs, w)
+    times = []
+    for _ in range(25):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        pc.pc_assemble_values(cl.ctx, s["row_ptr"], s["col_idx"], s["nnzb"], cl.x, cl.v, pairs, w, cl.h, s["vals"],
+                              s["b"], s["dres"])
+        torch.cuda.synchronize()
+        times.append(time.perf_counter() - t0)
+    assert np.median(times[3:]) <= 192e-6, times
+    cl.close()
