@@ -363,18 +363,26 @@ def run_ours(args):
     achieved = spmv_bytes / avg_spmv_s / 1e9 if n_spmv else None
     peak, peak_src = measured_hbm()
     clocks = clk.summary()
-    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+    resident = bool(n_spmv) and launches < sum(iters)  # the system stays in the SMs' shared memory
+    if resident:
+        mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 2032.0
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        peak = SMEM_BYTES_PER_CLK * sms * mhz * 1e6 / 1e9
+        peak_src = f"derived: {SMEM_BYTES_PER_CLK} B/clk/SM x {sms} SMs x {mhz:.0f} MHz (median SM clock under load)"
+    roofline = {"bound": "smem" if resident else "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None,
                 "traffic": SPMV_DRAM_BYTES.get((wl.name, args.storage)),
-                "kernel": "patch_spmv_kernel (q = A p, difference form, with p.q; patch records)" if mirrored else
-                "pcg_resident_kernel (whole iterations in one launch)" if not n_spmv and not n_cl else {"sell": "spmv_sell_kernel<true>", "sym": "spmv_sym_kernel<true>"}.get(
+                "kernel": "pcg_resident_kernel (q = A p within whole iterations in one launch)" if resident else
+                "patch_spmv_kernel (q = A p, difference form, with p.q; patch records)" if mirrored else
+                {"sell": "spmv_sell_kernel<true>", "sym": "spmv_sym_kernel<true>"}.get(
                     args.storage, "spmv_kernel<true,true,CAPR>") + " (q = A p, difference form, with p.q; "
                     + args.storage + " storage; CAPR = 14 or 18 blocks per row per stage, chosen per "
                     "solve from the largest tile)",
                 "blocks_per_launch": int(spmv_blocks),
                 "bytes_per_launch": spmv_bytes, "peak_source": peak_src,
                 "avg_launch_us": avg_spmv_s * 1e6, "timed_launches": n_spmv,
-                "sampling": "CUDA events around the first and the middle product of each 32-iteration chunk; "
+                "sampling": "CUDA events around the launch, in proportion to its products' cycles" if resident else
+                            "CUDA events around the first and the middle product of each 32-iteration chunk; "
                             "the middle one stands for the chunk's other products"}
     if n_cl and cl_iters:
         # the whole solve ran in one thread-block cluster: its roofline is the shared memory

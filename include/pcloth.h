@@ -604,10 +604,11 @@ PC_API int64_t pc_launch_count(const pc_ctx *ctx);
  * (check_every) with CUDA events on its stream: the chunk's first launch, which follows
  * the host's convergence check, and its middle one, which stands for the chunk's other
  * launches (weighted by the iterations the chunk ran); pc_step brackets its assembly the
- * same way. pc_spmv_stats returns (launches represented, their total ms, the number of
- * blocks that a product of the last matrix reads: with the default storage, where the
- * products run from patch records, each block inside a patch counts once) and resets the
- * counters. Solves whose iterations run inside one launch report no products. */
+ * same way. Where iterations run inside one launch, the launch counts the cycles of its
+ * products and is timed as a whole. pc_spmv_stats returns (products represented, their total ms,
+ * the number of blocks that a product of the last matrix reads: with the default storage, where
+ * the products run from patch records, each block inside a patch counts once) and resets the
+ * counters. */
 PC_API pc_status pc_set_profiling(pc_ctx *ctx, int32_t enable);
 PC_API pc_status pc_spmv_stats(pc_ctx *ctx, int64_t *launches, double *total_ms, int64_t *nnzb);
 /* Likewise for pc_step's assembly (pattern and values, Sec. 3.2.2): (steps timed, total

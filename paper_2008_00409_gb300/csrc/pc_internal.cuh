@@ -69,6 +69,8 @@ struct pc_scalars {
     int32_t status;   // pc_status of the solve
     uint32_t counter; // last-block reduction ticket
     int32_t outer;    // FP64 residual replacements (the cluster solve reports them here)
+    // a profiled resident launch: cycles in its products (the slowest CTA's), and in all of it
+    unsigned long long prod_cycles, all_cycles;
 };
 
 // ------------------------------------------------------------------------- radix sort scratch

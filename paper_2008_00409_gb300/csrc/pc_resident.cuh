@@ -191,13 +191,15 @@ __device__ __forceinline__ void res_precond(const float *D, const float *r, floa
     }
 }
 
-template <int SPLIT, bool BLOCK>
+// PROF: count cycles for pc_spmv_stats (as a flag of the launch it cost 1% of every iteration).
+template <int SPLIT, bool BLOCK, bool PROF>
 __global__ void __launch_bounds__(1024, 1) pcg_resident_kernel(ResArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint64_t bar;
     __shared__ int s_fail, s_stop, s_iter;
     __shared__ float s_rz;
+    __shared__ long long s_cycles[2];  // thread 0's, in products and in the launch
     unsigned char *rec = smem_raw;
     float4 *share = reinterpret_cast<float4 *>(smem_raw + a.rec_cap);
     const PatchP ps{reinterpret_cast<float *>(smem_raw + a.rec_cap + 16 * a.share_cap), a.R + a.halo_cap};
@@ -210,6 +212,10 @@ __global__ void __launch_bounds__(1024, 1) pcg_resident_kernel(ResArgs a)
     const int32_t *halo = reinterpret_cast<const int32_t *>(rec + L.halo);
     if (t == 0) {
         s_fail = 0;
+        if (PROF) {
+            s_cycles[0] = 0;
+            s_cycles[1] = -clock64();
+        }
         mbar_init(&bar, 1);
         mbar_fence_init();
     }
@@ -272,6 +278,7 @@ __global__ void __launch_bounds__(1024, 1) pcg_resident_kernel(ResArgs a)
     bool timeout = false;
     while (!stop) {
         // ---- q = A p
+        if (PROF && t == 0) s_cycles[0] -= clock64();
         float q[3] = {0.f, 0.f, 0.f};
         patch_row_keep<SPLIT, 2>(rec, L, share, ps, slice, pi, part, q[0], q[1], q[2]);
         __syncthreads();
@@ -301,6 +308,7 @@ __global__ void __launch_bounds__(1024, 1) pcg_resident_kernel(ResArgs a)
             }
             hi[0] = fmaf(pi.x, q[0], fmaf(pi.y, q[1], pi.z * q[2]));
         }
+        if (PROF && t == 0) s_cycles[0] += clock64();
         if (!res_sum<1>(a, ++epoch, hi, lo)) {
             timeout = true;
             break;
@@ -404,6 +412,10 @@ __global__ void __launch_bounds__(1024, 1) pcg_resident_kernel(ResArgs a)
         return;
     }
     if (epoch == a.epoch0) return;  // the solve had stopped before this launch
+    if (PROF && t == 0) {
+        atomicMax(&a.sc->prod_cycles, (unsigned long long)s_cycles[0]);
+        if (blockIdx.x == 0) a.sc->all_cycles = (unsigned long long)(s_cycles[1] + clock64());
+    }
     if (mine) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {

@@ -747,9 +747,12 @@ static pc_status patch_set_smem(const pc_ctx *c)
 {
     int most = 0;
     PC_CUDA_TRY(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-    const void *kernels[] = {(const void *)patch_spmv_kernel,
-                             (const void *)pcg_resident_kernel<2, false>, (const void *)pcg_resident_kernel<2, true>,
-                             (const void *)pcg_resident_kernel<4, false>, (const void *)pcg_resident_kernel<4, true>};
+    const void *kernels[] = {
+        (const void *)patch_spmv_kernel,
+        (const void *)pcg_resident_kernel<2, false, false>, (const void *)pcg_resident_kernel<2, false, true>,
+        (const void *)pcg_resident_kernel<2, true, false>, (const void *)pcg_resident_kernel<2, true, true>,
+        (const void *)pcg_resident_kernel<4, false, false>, (const void *)pcg_resident_kernel<4, false, true>,
+        (const void *)pcg_resident_kernel<4, true, false>, (const void *)pcg_resident_kernel<4, true, true>};
     for (const void *k : kernels) {
         cudaFuncAttributes fa;
         PC_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
@@ -1415,11 +1418,17 @@ static pc_status launch_dinv(const SolveCtx &s)
     return PC_OK;
 }
 
+template <int SPLIT, bool BLOCK>
+static const void *resident_kernel(bool profile)
+{
+    return profile ? (const void *)pcg_resident_kernel<SPLIT, BLOCK, true>
+                   : (const void *)pcg_resident_kernel<SPLIT, BLOCK, false>;
+}
 static const void *resident_kernel(const SolveCtx &s)
 {
-    if (s.pt_split == 4)
-        return s.block ? (const void *)pcg_resident_kernel<4, true> : (const void *)pcg_resident_kernel<4, false>;
-    return s.block ? (const void *)pcg_resident_kernel<2, true> : (const void *)pcg_resident_kernel<2, false>;
+    const bool profile = s.c->profiling != 0;
+    if (s.pt_split == 4) return s.block ? resident_kernel<4, true>(profile) : resident_kernel<4, false>(profile);
+    return s.block ? resident_kernel<2, true>(profile) : resident_kernel<2, false>(profile);
 }
 
 // Iterations until the solve stops or needs a residual replacement.
@@ -1465,12 +1474,26 @@ static pc_status launch_resident(const SolveCtx &s, float *x, const pc_solve_opt
     a.sc = c->sc;
     a.err = c->d_err;
     a.budget = c->bar_wait_cycles > 0 ? (long long)c->bar_wait_cycles : PT_WAIT_BUDGET;
+    const bool timed = c->profiling != 0;
+    if (timed) {
+        PC_CUDA_TRY(cudaMemsetAsync(&c->sc->prod_cycles, 0, 2 * sizeof(unsigned long long), s.st));
+        PC_CUDA_TRY(cudaEventRecord(c->ev[4], s.st));
+    }
     void *args[] = {&a};
     PC_CUDA_TRY(cudaLaunchCooperativeKernel(resident_kernel(s), dim3(c->pt_n), dim3(s.pt_split * c->pt_rows), args,
                                             (size_t)s.pt_smem, s.st));
     c->launches++;
+    if (timed) PC_CUDA_TRY(cudaEventRecord(c->ev[5], s.st));
     const int iter0 = c->sc_host->iter;
     PC_TRY(read_scalars(c, s.st));
+    if (timed && c->sc_host->iter > iter0 && c->sc_host->all_cycles > 0) {
+        // the launch's time in the proportion of the cycles
+        float ms = 0.f;
+        PC_CUDA_TRY(cudaEventElapsedTime(&ms, c->ev[4], c->ev[5]));
+        c->spmv_ms += ms * ((double)c->sc_host->prod_cycles / (double)c->sc_host->all_cycles);
+        c->spmv_launches += c->sc_host->iter - iter0;
+        c->spmv_nnzb = c->pt_kept;
+    }
     if (c->sc_host->status != PC_ERR_TIMEOUT) c->pt_epoch = a.epoch0 + 2u * (unsigned)(c->sc_host->iter - iter0) + 1u;
     return PC_OK;
 }
