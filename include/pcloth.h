@@ -189,9 +189,10 @@ typedef struct {
  * neighbouring vertices and stores a block between two rows of a patch once for both, where
  * the matrix's blocks inside the patches are symmetric bit for bit, as pc_assemble_values
  * makes them; otherwise, or with rows of more than 64 kept blocks or patches of too many
- * contacts for shared memory, it is a plain BSR copy (as for more than 480 rows per SM when
- * max_iter is below 32: the records cost what about 25 products save). Without dres, or when the copy
- * exceeds the context's capacity, the products read the matrix itself. */
+ * contacts for shared memory (three sheets: above about 0.5 contacts per vertex; up to 4 where
+ * fewer than 100 rows per SM stay resident), it is a plain BSR copy. So it is above 480 rows per
+ * SM when max_iter is below 32, because the records cost what about 25 products save. Without
+ * dres, or when the copy exceeds the context's capacity, the products read the matrix itself. */
 #define PC_STORAGE_SYM 0
 #define PC_STORAGE_FULL 1
 #define PC_STORAGE_SELL 2
@@ -266,7 +267,7 @@ PC_API pc_status pc_get_rest(const pc_ctx *ctx, int32_t *hinges, float *mass, vo
 /* Sec. 3.2.2, dynamic matrix assembly, pattern half: the step's block pattern is the set
  * of (row, col) vertex pairs coupled by any triangle, hinge or contact pair of this step,
  * plus the diagonal, sorted by (row, col) with duplicates removed. The contacts' columns are
- * put in order row by row (with a key sort when a vertex has more than 64 contacts) and
+ * put in order row by row (with a key sort when a vertex has more than 1,024 contacts) and
  * merged into the static pattern, so row_ptr and col_idx are bit-exact and deterministic.
  * On return A->nnzb holds the block count. If it exceeds A->cap the call returns
  * PC_ERR_CAPACITY with A->nnzb = required size and col_idx untouched beyond cap.
@@ -283,9 +284,9 @@ PC_API pc_status pc_assemble_pattern(pc_ctx *ctx, const pc_contacts *contacts, p
  * dres (optional, float[V][9], may be NULL) receives the "difference-form" diagonal
  * D_i = m_i I - sum over pinned neighbours j of the unzeroed block A_ij, with which
  * (A p)_i = D_i p_i + sum_{j != i} A_ij (p_j - p_i) holds exactly for this model (every
- * element's Hessian rows sum to zero). Element contributions are combined per row by a
- * warp-level reduction in a fixed order (no atomics): results are deterministic and
- * A is bitwise symmetric. x, v: device float[V][3]. Does not synchronize. */
+ * element's Hessian rows sum to zero). Element contributions are added block by block in a
+ * fixed order (no atomics): results are deterministic and A is bitwise symmetric. x, v: device
+ * float[V][3]. Does not synchronize. */
 PC_API pc_status pc_assemble_values(pc_ctx *ctx, const pc_bsr *A, const float *x, const float *v,
                              const pc_contacts *contacts, float h, float *vals, float *b, float *dres,
                              void *stream);

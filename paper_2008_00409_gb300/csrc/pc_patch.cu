@@ -5,11 +5,13 @@
 // patch rows keep the order of their original numbers. The order only decides how much is
 // shared within a patch: any matrix of the context's size is stored correctly with it.
 //
-// Records, once per solve: a counting pass over the patches (one CTA each, one thread per
-// row), a scan of the record sizes, a filling pass. A block whose mirror image is not its
-// transpose bit for bit, a row that keeps more than PT_MAX_OWN blocks, a column
-// out of order, or a patch whose halo or store does not fit make the build report failure;
-// the solve then streams the BSR rows.
+// Records, once per solve: a counting pass over the patches (one CTA each), a scan of the
+// record sizes, a filling pass. A block whose mirror image is not its transpose bit for bit, a
+// row that keeps more than PT_MAX_OWN blocks, a column out of order, or a patch whose halo or
+// record does not fit make the build report failure; the solve then streams the BSR rows.
+// Contacts between sheets join different patches, so both rows keep their blocks: three sheets'
+// records fit with up to 0.5 contacts per vertex where they are streamed (10 kept blocks per row),
+// and with 0.1, 1 and 4 where they stay on SMs of 444, 198 and 81 rows.
 #include <algorithm>
 
 #include "pc_patch.cuh"

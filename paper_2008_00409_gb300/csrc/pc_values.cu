@@ -1,9 +1,9 @@
 // Value assembly (Sec. 3.2.2 "value filling", Eq. 2-3): element kernels evaluate every
 // assembly element once (force and Hessian at x_t) into per-element records, and the
 // right-hand side is Eq. 3's h f(x_t + h v_t) to first order, b = h (f(x_t) - h K v_t);
-// a warp per matrix row then gathers the records of the elements incident to that row
-// and reduces them into the row's blocks in a fixed order. No atomics: the result is
-// deterministic and the matrix is bitwise symmetric.
+// a thread per off-diagonal block then sums the records on the block's own list, and one per row
+// those incident to the row (diagonal and right-hand side), in a fixed order. No atomics: the
+// result is deterministic and the matrix is bitwise symmetric.
 //
 // Precision: the membrane strain G = (F^T F - I)/2 cancels catastrophically in FP32 at
 // cloth strains (1e-5..1e-3). It is formed instead as Dm^-T (Ds^T Ds - Dm^T Dm) Dm^-1 with

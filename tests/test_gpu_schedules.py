@@ -145,3 +145,20 @@ def test_fused_update_barrier_timeout_and_recovery_on_the_matrix(pc):
     again, n, _, _ = _solve(pc, cl, s, storage=pc.PC_STORAGE_FULL)
     assert n == iters and torch.equal(again, ref)
     cl.close()
+
+
+# contacts that join the sheets' patches: records hold a few per vertex where they stay on the SMs,
+# and half a contact per vertex streamed; the proximity query's several per vertex are the copy's
+@pytest.mark.parametrize("n,layers,delta,records", [(64, 3, 5.5e-4, True), (150, 3, 5.5e-4, False),
+                                                    (200, 3, 5.5e-4, False)])
+def test_contacts_too_dense_for_records(pc, n, layers, delta, records):
+    wl = wk.proximity_stack(n, layers, delta=delta)
+    cl = pc.Cloth(wl)
+    pairs, w = cl.proximity()
+    assert pairs.shape[0] > wl.V
+    s = cl.assemble(pairs, w)
+    dv, iters, launches, blocks = _solve(pc, cl, s)
+    assert (launches < iters) == records and (blocks < s["nnzb"] - cl.V) == records
+    general = _solve(pc, cl, s, storage=pc.PC_STORAGE_FULL)
+    assert H.rel_l2(_np(dv), _np(general[0])) <= H.DV_RTOL
+    cl.close()
