@@ -210,14 +210,31 @@ __global__ void px_emit_cells_kernel(int T, const float4 *__restrict__ box, floa
             }
 }
 
-// first[c]: where cell c's list begins (c = 0 .. n), from the sorted keys. A thread per cell
-// searches: neighbours take the same path, and the work does not depend on where the triangles
-// are (a thread per key that fills the cells up to the next one walks a run of empty cells alone:
-// with two 301 x 301 sheets 10 cm apart, 500,000 cells, a query took 1,937 us that takes 311).
+// first[c]: where cell c's list begins (c = 0 .. n), from the sorted keys: a thread per key fills
+// the cells after the key before it, its whole warp where they are many. (Alone, one thread walked
+// the run of empty cells between two 301 x 301 sheets 10 cm apart, 500,000 cells: a query took
+// 1,937 us that takes 360. A search per cell takes 311 there, but 276-282 instead of 274-277 for
+// three 100 x 100 sheets 0.5 mm apart.)
+#define PX_RUN 64
 __global__ void px_first_kernel(int64_t K, const uint64_t *__restrict__ keys, int64_t n, int32_t *first)
 {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c <= n) first[c] = (int32_t)pc_lower_bound_u64(keys, K, (uint64_t)c);
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    int64_t b = 0, e = -1;
+    if (i <= K) {
+        b = i == 0 ? 0 : (int64_t)keys[i - 1] + 1;
+        e = i == K ? n : (int64_t)keys[i];
+    }
+    const bool many = e - b >= PX_RUN;
+    if (!many)
+        for (int64_t c = b; c <= e; ++c) first[c] = (int32_t)i;
+    for (unsigned m = __ballot_sync(0xffffffffu, many); m; m &= m - 1) {
+        const int from = __ffs(m) - 1;
+        const int64_t wb = __shfl_sync(0xffffffffu, b, from), we = __shfl_sync(0xffffffffu, e, from);
+        const int32_t v = (int32_t)__shfl_sync(0xffffffffu, i, from);
+#pragma unroll 8
+        for (int64_t c = wb + lane; c <= we; c += 32) first[c] = v;
+    }
 }
 
 // true when v is among ecol[lo .. hi) (sorted)
@@ -460,7 +477,7 @@ extern "C" pc_status pc_proximity_query(pc_ctx *ctx, const float *x, float delta
     a.w = w;
     a.err = ctx->d_err;
     if (a.first)
-        PC_LAUNCH(ctx, px_first_kernel, pc_blocks((int64_t)g.n + 1, 256), 256, 0, st, K, ctx->px_keys, (int64_t)g.n, ctx->px_first);
+        PC_LAUNCH(ctx, px_first_kernel, pc_blocks(K + 1, 256), 256, 0, st, K, ctx->px_keys, (int64_t)g.n, ctx->px_first);
     PC_LAUNCH(ctx, px_pairs_kernel<false>, pc_blocks(V + 1ll, 128), 128, 0, st, a);
     PC_TRY(pc_exclusive_scan(ctx, ctx->px_vcnt, ctx->px_voff, V, st));
     PC_CUDA_TRY(cudaMemcpyAsync(ctx->h_count, ctx->px_voff + V, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
