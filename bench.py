@@ -42,8 +42,9 @@ FALLBACK_HBM_GBS = 6800.0
 SMEM_BYTES_PER_CLK = 128
 CLUSTER_SMS = 16
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the PCG product in
-# steady state, by (workload, storage), where the current kernel has been profiled
-SPMV_DRAM_BYTES = {}
+# steady state (ncu --cache-control none), by (workload, storage), where the current kernel has
+# been profiled
+SPMV_DRAM_BYTES = {("stack3x526", "offdiag"): 284.2e6 + 6.3e6}
 
 
 def parse():

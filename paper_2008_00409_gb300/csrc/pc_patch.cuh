@@ -185,7 +185,7 @@ struct PatchArgs {
 // first record does not depend on the preceding kernel and is requested before the
 // programmatic wait.
 // Bound by shared-memory wavefronts and their latency at 16 warps per SM about as much as by
-// HBM: 52.9 us at 830,028 rows, 275 MB, 5.2 TB/s (the BSR stream: 73 us, 439 MB). Patches of 64
+// HBM: 52.9 us at 830,028 rows, 290 MB, 5.5 TB/s (the BSR stream: 73 us, 439 MB). Patches of 64
 // and 160 rows take 56.5 and 53.7 us: 128 keeps as many blocks inside as four CTAs of an SM
 // have room for. The slowest SM needs a fifth more cycles than the average; handing out the
 // last patches by ticket evened that out but needs a partial sum per patch to keep the order of
