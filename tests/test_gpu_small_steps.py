@@ -4,7 +4,6 @@ import dataclasses
 
 import numpy as np
 import pytest
-import torch
 
 import oracle
 from paper_2008_00409_gb300 import workloads as wk
