@@ -90,19 +90,23 @@ def test_values_at_edges_of_small_tiles(pc, nx, ny):
 
 
 def test_values_of_few_rows_with_many_contacts_in_time(pc):
-    """12,288 rows of 48 contacts: the rows' contacts are chains of loads where nothing else hides
-    them. A warp per row that staged them took 192 us, which this call may not exceed."""
-    wl = wk.proximity_stack(64, 3, delta=8e-3, per_vertex=40.0)
-    cl = pc.Cloth(wl)
-    pairs, w = cl.proximity()
-    s = cl.assemble(pairs, w)
-    times = []
-    for _ in range(25):
-        torch.cuda.synchronize()
-        t0 = time.perf_counter()
-        pc.pc_assemble_values(cl.ctx, s["row_ptr"], s["col_idx"], s["nnzb"], cl.x, cl.v, pairs, w, cl.h, s["vals"],
-                              s["b"], s["dres"])
-        torch.cuda.synchronize()
-        times.append(time.perf_counter() - t0)
-    assert np.median(times[3:]) <= 192e-6, times
-    cl.close()
+    """12,288 rows of 48 contacts beside four times as many of 47: the few rows' contacts are chains
+    of loads that nothing else hides (32 rows per CTA and one contact at a time: 0.44 of the many
+    rows' time; now 0.34)."""
+    took = []
+    for n, delta in ((64, 8e-3), (128, 3e-3)):
+        wl = wk.proximity_stack(n, 3, delta=delta, per_vertex=40.0)
+        cl = pc.Cloth(wl)
+        pairs, w = cl.proximity()
+        s = cl.assemble(pairs, w)
+        times = []
+        for _ in range(31):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            pc.pc_assemble_values(cl.ctx, s["row_ptr"], s["col_idx"], s["nnzb"], cl.x, cl.v, pairs, w, cl.h, s["vals"],
+                                  s["b"], s["dres"])
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t0)
+        took.append(float(np.median(times[3:])))
+        cl.close()
+    assert took[0] <= 0.4 * took[1], took
